@@ -229,39 +229,47 @@ struct DirParams {
     int *status;
 };
 
-// Cluster-resident plates: one thread-block cluster per plate, the plate's
-// coupling rows held in registers for the whole launch (forward pass).
+// Resident plates (mdx_resident.cu): a plate's coupling tensor held by `sub`
+// CTAs of one thread-block cluster for the whole launch.
 struct ClusterK {
     long long off;     // float offset of the stress mode's class chunk (H)
     int mc, kpos, c;   // chunk size, position in the chunk, class
     int pad;
 };
 
-struct ClusterParams {
-    const InstDesc *inst;
-    const int *plates;            // plate instance indices (one cluster each)
-    const ClusterK *kinfo;        // [total_k]
-    const float *H;
-    const float *kappa;
-    const int *perm;
-    ModeCoef coef;
-    int cs;                       // CTAs per cluster
-    int nkc;                      // stress-mode slots per CTA
-    int wk;                       // warps per slot (rows: class-ordered modes)
-    int steps, n_begin, total_steps;
-    const float *exc;
-    float *audio;
-    float *state_io;              // [4][total_modes]: q_hi, q_lo, v_hi, v_lo
-    long long total_modes;
-    int *status;
+constexpr int kResMaxModes = 256;     // transverse modes of a plate
+constexpr int kResVariants = 7;       // kernel variants, by row length
+
+// Work of one CTA: rank `rank` of the `sub` CTAs that share plate `plate`.
+struct ResCta {
+    int plate;                        // instance, or -1 (empty place of a cluster)
+    int rank, sub;
+    int base;                         // cluster rank of this plate's rank 0
+    int L;                            // padded row length (floats, multiple of 8)
+    int k0, nk;                       // stress modes k0 .. k0 + nk - 1, one per warp
+    int pad;
 };
 
-// Row length (floats) of the register-resident coupling rows: 32 or 64; 0
-// when a plate does not fit.  cluster_plan picks the cluster shape.
-int cluster_row_len(int max_class);
-int cluster_max_threads(int row_len);
-cudaError_t launch_cluster(const ClusterParams &P, int n_plates, int row_len, cudaStream_t s);
-cudaError_t cluster_check(int cs, int threads, int row_len, int *max_clusters);
+struct ResidentParams {
+    PlateParams p;
+    const ResCta *ctas;
+    const ClusterK *kinfo;            // [total_k] (class layout)
+    const int *iperm;                 // inverse class permutation, at each plate's perm_off
+    int variant;                      // kernel variant
+    int warps;                        // warps with a stress mode or a share of the update
+    int L;                            // longest padded row
+    int n_max, no_max;                // most modes of a plate, most modes owned by a CTA
+    int max_sub;
+    int tcols;                        // tensor-memory columns per CTA
+};
+
+int resident_variant(int w, int rows);
+int resident_max_warps(int variant);
+int resident_columns(int variant, int L, int warps);
+size_t resident_smem(int R, const ResidentParams &Q);
+cudaError_t resident_check(int cs, const ResidentParams &Q, size_t smem_optin, int *fit);
+cudaError_t launch_resident(int R, const ResidentParams &Q, int grid, int cs, size_t smem,
+                            cudaStream_t s);
 
 struct TensionParams {
     const InstDesc *inst;

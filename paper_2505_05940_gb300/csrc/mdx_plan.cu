@@ -146,11 +146,12 @@ struct mdx_plan {
     GroupPlan *grp = nullptr;
     std::vector<int> grouped;      // per instance
     bool any_grouped = false;
-    // cluster-resident forward pass (few plates, class layout): one cluster per plate
-    bool cluster_ok = false;
-    int cl_cs = 0, cl_nkc = 0, cl_wk = 0, cl_rl = 0, n_cplates = 0;
-    ClusterK *d_kinfo = nullptr;
-    int *d_cplates = nullptr;
+    // resident plates: the coupling tensors held on the SMs (mdx_resident.cu)
+    bool res_ok = false;
+    int res_cs = 1, res_grid = 0;
+    ResidentParams res{};            // launch shape and tables (p unset)
+    size_t res_smem[4] = {0, 0, 0, 0};   // by right-hand sides
+    bool fused_sweep = false;        // mdx_grad fuses reverse and recompute
 };
 
 namespace {
@@ -249,6 +250,11 @@ struct Piece {
     double cost;
 };
 
+// Chooses how many CTAs share each plate and lays the resident launch out
+// (plan.res_ok stays false when a plate does not fit).
+int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
+                  const std::vector<PlateItem> &items, const std::vector<int> &perm_all,
+                  int smem_optin);
 int configure_tiles(mdx_plan *p, int stage_req, int ring_req);
 void update_l2_keep(mdx_plan *p);
 
@@ -869,58 +875,13 @@ int mdx_plan_create(mdx_plan **out, const mdx_instance *I, int n_inst, const mdx
             if ((rc2 = upload(p, &p->d_perm, perm_all.data(), perm_all.size()))) return bail(rc2);
             if ((rc2 = upload(p, &p->d_kperm, kperm_all.data(), kperm_all.size()))) return bail(rc2);
             if ((rc2 = upload(p, &p->d_chunks, chunks.data(), chunks.size()))) return bail(rc2);
-            // cluster-resident forward pass: every plate's rows in the registers of
-            // one cluster (class layout, class blocks of at most 64 modes, at most
-            // 512 threads a CTA), and all clusters resident at once; not for plans
-            // whose options shape the streaming kernel's work split (tests of it)
-            if (parity && o.force_split <= 0 && o.max_ctas <= 0 && !(p->debug_flags & 1)) {
-                std::vector<int> cplates;
-                int maxN = 0, maxM = 0, maxcls = 0;
-                for (int i = 0; i < n_inst; ++i) {
-                    const InstDesc &d = p->inst[i];
-                    if (d.kind != MDX_KIND_PLATE || d.M == 0 || d.grouped) continue;
-                    cplates.push_back(i);
-                    maxN = std::max(maxN, d.N);
-                    maxM = std::max(maxM, d.M);
-                    for (int a = 0; a < 4; ++a) maxcls = std::max(maxcls, d.ncls[a]);
-                }
-                const int rl = cluster_row_len(maxcls);
-                const int wk = (maxN + 31) / 32;
-                if (!cplates.empty() && rl > 0 && !(p->debug_flags & 16)) {
-                    for (int cs : {std::min(maxM, 8), 16}) {
-                        if (cs > maxM && cs != std::min(maxM, 8)) break;
-                        const int nkc = (maxM + cs - 1) / cs;
-                        const int threads = nkc * wk * 32;
-                        if (threads > cluster_max_threads(rl)) continue;
-                        int fit = 0;
-                        if (cluster_check(cs, threads, rl, &fit) != cudaSuccess) {
-                            cudaGetLastError();
-                            continue;
-                        }
-                        if (fit < (int)cplates.size()) continue;
-                        std::vector<ClusterK> kinfo(std::max<long long>(p->total_k, 1));
-                        for (const auto &it : items)
-                            for (int ci = it.chunk0; ci < it.chunk1; ++ci)
-                                for (int q = 0; q < chunks[ci].mc; ++q) {
-                                    ClusterK &K = kinfo[p->inst[it.inst].k_off + chunks[ci].kl0 + q];
-                                    K.off = chunks[ci].off;
-                                    K.mc = chunks[ci].mc;
-                                    K.kpos = q;
-                                    K.c = chunks[ci].c;
-                                }
-                        if ((rc2 = upload(p, &p->d_kinfo, kinfo.data(), kinfo.size()))) return bail(rc2);
-                        if ((rc2 = upload(p, &p->d_cplates, cplates.data(), cplates.size())))
-                            return bail(rc2);
-                        p->cluster_ok = true;
-                        p->cl_cs = cs;
-                        p->cl_nkc = nkc;
-                        p->cl_wk = wk;
-                        p->cl_rl = rl;
-                        p->n_cplates = (int)cplates.size();
-                        break;
-                    }
-                }
+            // resident plates, not for plans whose options shape the streaming
+            // kernel's work split (tests of it)
+            if (o.force_split <= 0 && o.max_ctas <= 0 && !(p->debug_flags & (1 | 16))) {
+                const int rcr = plan_resident(p, chunks, items, perm_all, smem_optin);
+                if (rcr) return bail(rcr);
             }
+            p->fused_sweep = p->fuse || (p->res_ok && !(p->debug_flags & 2));
             // contraction units: plates with a direction tensor (direction
             // derivative), and every plate (full dL/dH output)
             auto build_units = [&](bool all, std::vector<DirUnit> &units,
@@ -1207,35 +1168,228 @@ TensionParams base_tension(mdx_plan *p, int mode, int steps, int n_begin, int to
     return T;
 }
 
-int run_cluster(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
-    ClusterParams C{};
-    C.inst = p->d_inst;
-    C.plates = p->d_cplates;
-    C.kinfo = p->d_kinfo;
-    C.H = p->d_H;
-    C.kappa = p->d_kappa;
-    C.perm = p->d_perm;
-    C.coef = p->coef;
-    C.cs = p->cl_cs;
-    C.nkc = p->cl_nkc;
-    C.wk = p->cl_wk;
-    C.steps = P.steps;
-    C.n_begin = P.n_begin;
-    C.total_steps = P.total_steps;
-    C.exc = P.exc;
-    C.audio = P.audio;
-    C.state_io = P.state_io;
-    C.total_modes = p->total_modes;
-    C.status = P.status;
+// Step time of one CTA in SM cycles: a fixed chain (barriers, reductions,
+// update; with peers also the two exchanges) and the packed FMAs of one stress
+// mode per warp (L / 8 rows of L columns a lane) over four schedulers.
+double res_step_cycles(int nk, int L, int sub) {
+    return 700.0 + (sub > 1 ? 800.0 + 10.0 * sub : 0.0) + 0.15 * L * L * ((nk + 3) / 4);
+}
+
+int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
+                  const std::vector<PlateItem> &items, const std::vector<int> &perm_all,
+                  int smem_optin) {
+    struct Pl {
+        int inst, N, M, L;
+    };
+    std::vector<Pl> pls;
+    int variant = 0;
+    for (int i = 0; i < p->n_inst; ++i) {
+        const InstDesc &d = p->inst[i];
+        if (d.kind != MDX_KIND_PLATE || d.M == 0 || d.grouped) continue;
+        const int w = d.parity ? *std::max_element(d.ncls, d.ncls + 4) : d.N;
+        const int v = resident_variant(w, d.parity ? (w + 7) / 8 : (d.N + 31) / 32);
+        if (v < 0 || d.N > kResMaxModes) return MDX_OK;
+        variant = std::max(variant, v);
+        pls.push_back({i, d.N, d.M, (w + 7) & ~7});
+    }
+    if (pls.empty()) return MDX_OK;
+    const int wmax = resident_max_warps(variant);
+    auto nk_of = [](const Pl &q, int sub) { return (q.M + sub - 1) / sub; };
+    // warps of a CTA: one per stress mode and, while there is room, others for the
+    // owned modes (32 a warp); enough for two modes of the plate a thread
+    auto warps_of = [&](const Pl &q, int sub) {
+        const int own = ((q.N + sub - 1) / sub + 31) / 32, nk = nk_of(q, sub);
+        return std::max({nk, own, (q.N + 63) / 64, std::min(nk + own, wmax)});
+    };
+    auto ok = [&](const Pl &q, int sub) { return sub <= q.M && warps_of(q, sub) <= wmax; };
+    auto cycles = [&](const Pl &q, int sub) { return res_step_cycles(nk_of(q, sub), q.L, sub); };
+    auto shape = [&](const std::vector<int> &sub) {
+        ResidentParams Q{};
+        Q.variant = variant;
+        for (size_t i = 0; i < pls.size(); ++i) {
+            Q.L = std::max(Q.L, pls[i].L);
+            Q.warps = std::max(Q.warps, warps_of(pls[i], sub[i]));
+            Q.n_max = std::max(Q.n_max, pls[i].N);
+            Q.no_max = std::max(Q.no_max, (pls[i].N + sub[i] - 1) / sub[i]);
+            Q.max_sub = std::max(Q.max_sub, sub[i]);
+        }
+        Q.tcols = resident_columns(variant, Q.L, Q.warps);
+        return Q;
+    };
+    // clusters: plates sorted by (CTAs, time), cs / sub of them per cluster,
+    // longest clusters first (the hardware starts them in order)
+    auto pack = [&](const std::vector<int> &sub, int cs, std::vector<std::vector<int>> &cl,
+                    std::vector<double> &ct) {
+        std::vector<int> ord(pls.size());
+        std::iota(ord.begin(), ord.end(), 0);
+        std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
+            if (sub[a] != sub[b]) return sub[a] > sub[b];
+            return cycles(pls[a], sub[a]) > cycles(pls[b], sub[b]);
+        });
+        std::vector<std::vector<int>> c0;
+        std::vector<double> t0;
+        int room = 0;
+        for (int i : ord) {
+            if (room < sub[i]) {
+                c0.push_back({});
+                t0.push_back(0.0);
+                room = cs;
+            }
+            c0.back().push_back(i);
+            t0.back() = std::max(t0.back(), cycles(pls[i], sub[i]));
+            room -= sub[i];
+        }
+        std::vector<int> co(c0.size());
+        std::iota(co.begin(), co.end(), 0);
+        std::stable_sort(co.begin(), co.end(), [&](int a, int b) { return t0[a] > t0[b]; });
+        cl.clear();
+        ct.clear();
+        for (int c : co) {
+            cl.push_back(c0[c]);
+            ct.push_back(t0[c]);
+        }
+    };
+    // For each bound of the step time every plate takes the fewest CTAs that meet
+    // it; the makespan of the clusters, in launch order, decides between the bounds.
+    double best = 1e300;
+    int best_cs = 0;
+    std::vector<int> best_sub;
+    ResidentParams best_q{};
+    constexpr int kSubs[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16};
+    for (int csmax : {8, 16}) {
+        std::vector<double> taus;
+        bool all = true;
+        for (const Pl &q : pls) {
+            bool any = false;
+            for (int s : kSubs)
+                if (s <= csmax && ok(q, s)) {
+                    any = true;
+                    taus.push_back(cycles(q, s));
+                }
+            all = all && any;
+        }
+        if (!all) continue;
+        std::sort(taus.begin(), taus.end());
+        taus.erase(std::unique(taus.begin(), taus.end()), taus.end());
+        std::vector<int> prev;
+        for (int j = 0; j < 24; ++j) {   // at most 24 bounds, spread over the sorted list
+            const double tau = taus[(taus.size() - 1) * j / 23];
+            std::vector<int> sub(pls.size());
+            int cs = 1;
+            for (size_t i = 0; i < pls.size(); ++i) {
+                int s0 = 0;
+                double t0 = 1e300;
+                for (int s : kSubs) {
+                    if (s > csmax || !ok(pls[i], s)) continue;
+                    const double t = cycles(pls[i], s);
+                    if (t < t0) {
+                        t0 = t;
+                        s0 = s;
+                    }
+                    if (t <= tau) break;
+                }
+                sub[i] = s0;
+                cs = std::max(cs, s0);
+            }
+            if (sub == prev) continue;
+            prev = sub;
+            const ResidentParams Q = shape(sub);
+            int fit = 0;
+            if (resident_check(cs, Q, (size_t)smem_optin, &fit) != cudaSuccess) {
+                cudaGetLastError();
+                continue;
+            }
+            if (fit < 1) continue;
+            std::vector<std::vector<int>> cl;
+            std::vector<double> ct;
+            pack(sub, cs, cl, ct);
+            std::vector<double> m(std::min<size_t>((size_t)fit, cl.size()), 0.0);
+            for (double t : ct) *std::min_element(m.begin(), m.end()) += t;
+            const double span = *std::max_element(m.begin(), m.end());
+            if (span < 0.98 * best) {
+                best = span;
+                best_cs = cs;
+                best_sub = sub;
+                best_q = Q;
+            }
+        }
+    }
+    if (best_cs == 0) return MDX_OK;
+    // ---- tables
+    std::vector<std::vector<int>> cl;
+    std::vector<double> ct;
+    pack(best_sub, best_cs, cl, ct);
+    std::vector<ResCta> ctas;
+    for (const auto &c : cl) {
+        int base = 0;
+        for (int i : c) {
+            const Pl &q = pls[i];
+            const int sub = best_sub[i];
+            for (int r = 0; r < sub; ++r) {
+                ResCta A{};
+                A.plate = q.inst;
+                A.rank = r;
+                A.sub = sub;
+                A.base = base;
+                A.L = q.L;
+                A.k0 = (int)((long long)q.M * r / sub);
+                A.nk = (int)((long long)q.M * (r + 1) / sub) - A.k0;
+                ctas.push_back(A);
+            }
+            base += sub;
+        }
+        for (; base < best_cs; ++base) {
+            ResCta A{};
+            A.plate = -1;
+            ctas.push_back(A);
+        }
+    }
+    std::vector<ClusterK> kinfo(std::max<long long>(p->total_k, 1));
+    for (const auto &it : items)
+        for (int ci = it.chunk0; p->parity && ci < it.chunk1; ++ci)
+            for (int q = 0; q < chunks[ci].mc; ++q) {
+                ClusterK &K = kinfo[p->inst[it.inst].k_off + chunks[ci].kl0 + q];
+                K.off = chunks[ci].off;
+                K.mc = chunks[ci].mc;
+                K.kpos = q;
+                K.c = chunks[ci].c;
+            }
+    std::vector<int> iperm(std::max<size_t>(perm_all.size(), 1), 0);
+    for (const Pl &q : pls) {
+        const InstDesc &d = p->inst[q.inst];
+        for (int c = 0; d.parity && c < d.N; ++c) iperm[d.perm_off + perm_all[d.perm_off + c]] = c;
+    }
+    ResCta *dc = nullptr;
+    ClusterK *dk = nullptr;
+    int *di = nullptr, rc;
+    if ((rc = upload(p, &dc, ctas.data(), ctas.size()))) return rc;
+    if ((rc = upload(p, &dk, kinfo.data(), kinfo.size()))) return rc;
+    if ((rc = upload(p, &di, iperm.data(), iperm.size()))) return rc;
+    p->res = best_q;
+    p->res.ctas = dc;
+    p->res.kinfo = dk;
+    p->res.iperm = di;
+    p->res_cs = best_cs;
+    p->res_grid = (int)ctas.size();
+    for (int r = 1; r <= 3; ++r) p->res_smem[r] = resident_smem(r, best_q);
+    p->res_ok = true;
+    return MDX_OK;
+}
+
+int run_resident(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
+    ResidentParams Q = p->res;
+    Q.p = P;
+    const int R = P.mode == MODE_FUSED ? 3 : (P.mode == MODE_REVERSE ? 2 : 1);
     mdx_plan::Rec rec{};
     if (p->profiling) {
-        rec.which = 6;
+        rec.which = (P.mode == MODE_FORWARD && !P.ckpt) ? 6 : P.mode;
         rec.bytes = (double)P.steps * p->H_bytes_per_step;
         MDX_CUDA(cudaEventCreate(&rec.a), "event");
         MDX_CUDA(cudaEventCreate(&rec.b), "event");
         MDX_CUDA(cudaEventRecord(rec.a, s), "event");
     }
-    MDX_CUDA(launch_cluster(C, p->n_cplates, p->cl_rl, s), "cluster plate kernel");
+    MDX_CUDA(launch_resident(R, Q, p->res_grid, p->res_cs, p->res_smem[R], s),
+             "resident plate kernel");
     if (p->profiling) {
         MDX_CUDA(cudaEventRecord(rec.b, s), "event");
         p->recs.push_back(rec);
@@ -1245,8 +1399,7 @@ int run_cluster(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
 
 int run_plate(mdx_plan *p, PlateParams &P, cudaStream_t s) {
     if (!p->any_plate) return MDX_OK;
-    // a forward pass without checkpoints of a few small plates: cluster-resident
-    if (p->cluster_ok && P.mode == MODE_FORWARD && !P.ckpt) return run_cluster(p, P, s);
+    if (p->res_ok) return run_resident(p, P, s);
     MDX_CUDA(cudaMemsetAsync(p->d_counters, 0, p->n_inst * sizeof(unsigned), s), "memset");
     MDX_CUDA(cudaMemsetAsync(p->d_abort, 0, sizeof(int), s), "memset");
     const size_t smem = (P.mode == MODE_FUSED) ? p->smem_fused
@@ -1350,8 +1503,8 @@ GradWork grad_layout(const mdx_plan *p, int K, void *base) {
     };
     w.seg_q = take((size_t)(K + 1) * TM);
     w.seg_v = take((size_t)(K + 1) * TM);
-    w.seg_q2 = p->fuse ? take((size_t)(K + 1) * TM) : nullptr;
-    w.seg_v2 = p->fuse ? take((size_t)(K + 1) * TM) : nullptr;
+    w.seg_q2 = p->fused_sweep ? take((size_t)(K + 1) * TM) : nullptr;
+    w.seg_v2 = p->fused_sweep ? take((size_t)(K + 1) * TM) : nullptr;
     w.adj = take(AD_N * TM);
     w.gacc = take(2 * GA_N * TM);
     w.kacc = take(2 * TK);
@@ -1497,7 +1650,7 @@ extern "C" int mdx_grad(mdx_plan *p, const float *exc, const double *q0, const d
         return MDX_OK;
     };
     int rc;
-    if (!p->fuse || !p->any_plate) {
+    if (!p->fused_sweep || !p->any_plate) {
         for (int sg = nseg - 1; sg >= 0; --sg) {
             if ((rc = recompute(sg, w.seg_q, w.seg_v, true, true))) return rc;
             PlateParams P;
