@@ -8,14 +8,19 @@
 //
 // Kernels: one generic strided GEMM with fused epilogues (bias, ReLU, ReLU
 // mask of the backward pass, FP32 or BF16 output), a column-sum for bias
-// gradients, and the Adam update.  The GEMM computes one 128 x 128 output
-// tile per CTA: 64-wide K chunks of both operands are staged (16-byte
-// vectors where K is contiguous in memory, coalesced gathers where the
-// operand is transposed) into K-major core-matrix images in two buffers, one
-// thread issues four 128 x N x 16 MMAs per chunk and commits to the buffer's
-// mbarrier, so the next chunk's staging overlaps the MMAs; four warps read
-// the accumulator with tcgen05.ld (one lane quarter each, one output row per
-// lane) and apply the epilogue.
+// gradients, and the Adam update.  The GEMM computes one 128 x 64 output tile
+// per CTA of 256 threads: 64-wide K chunks of both operands go into K-major
+// core-matrix images in four buffers, one thread issues four 128 x N x 16 MMAs
+// per chunk and commits to the buffer's mbarrier; eight warps read the
+// accumulator with tcgen05.ld (one output row per lane, half the columns each)
+// and apply the epilogue with vector stores.  Operands that are contiguous
+// along K are staged with 16-byte asynchronous copies three chunks ahead;
+// operands contiguous along the rows (both of dW = dZ^T X) as 8 x 8 blocks,
+// eight 16-byte loads a thread transposed in registers.  The GEMMs of this
+// network are small (256 x 512 x 1024 at most), so each is the latency of its
+// chunks: with synchronous staging, element gathers of transposed operands and
+// one 128 x 128 tile per CTA a forward and backward pass of batch 256 took
+// 510 us, now 266 us.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -30,12 +35,13 @@ namespace mdx {
 
 namespace {
 
-constexpr int TBM = 128, TBN = 128, TBK = 64;   // output tile, K chunk (BF16 elements)
-constexpr int kGemmThreads = 128;                // 4 warps = the 4 tensor-memory lane quarters
-constexpr int kTileBytes = TBM * TBK * 2;        // one operand chunk image (16 KB)
+constexpr int TBM = 128, TBN = 64, TBK = 64;    // output tile, K chunk (BF16 elements)
+constexpr int kGemmThreads = 256;                // first half stages A, second half B
+constexpr int kGemmStages = 4;
+constexpr int kABytes = TBM * TBK * 2, kBBytes = TBN * TBK * 2;   // operand chunk images
 constexpr long long kGemmWait = 1LL << 24;
 
-enum : int { EPI_NONE = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BF16 = 8, EPI_ACCUM = 16 };
+enum : int { EPI_NONE = 0, EPI_BIAS = 1, EPI_RELU = 2, EPI_MASK = 4, EPI_BF16 = 8 };
 
 struct GemmArgs {
     int M, N, K;
@@ -74,67 +80,90 @@ __device__ __forceinline__ void mma_bf16_tc(uint32_t d_tmem, uint64_t a, uint64_
         : "memory");
 }
 
-// Stages rows row0 .. row0+127 (valid below `rows`) and K columns k0 .. k0+63
+// 16-byte asynchronous copy of which the first `bytes` are read, the rest zero.
+__device__ __forceinline__ void copy16(uint16_t *dst, const uint16_t *src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::su32(dst)), "l"(src),
+                 "r"(bytes)
+                 : "memory");
+}
+
+// Transposes an 8 x 8 block of 16-bit elements held as eight rows of four words.
+__device__ __forceinline__ void transpose8(uint4 (&v)[8]) {
+    uint32_t w[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i][0] = v[i].x, w[i][1] = v[i].y, w[i][2] = v[i].z, w[i][3] = v[i].w;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        uint32_t o[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            o[c] = __byte_perm(w[2 * c][r >> 1], w[2 * c + 1][r >> 1], (r & 1) ? 0x7632 : 0x5410);
+        v[r] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+}
+
+// Stages ROWS rows from row0 (valid below `rows`) and K columns k0 .. k0+63
 // (valid below K) of a strided BF16 matrix, element (r, k) at
 // src[r * s_r + k * s_k], into a K-major core-matrix image: 16-byte units of
-// 8 K-adjacent elements, 8-row groups 8 units (1024 bytes) apart.
+// 8 K-adjacent elements, 8-row groups 8 units (1024 bytes) apart.  t: thread
+// 0..127 of the operand's half of the CTA.
+template <int ROWS>
 __device__ __forceinline__ void stage_operand(uint16_t *img, const uint16_t *src, long long s_r,
-                                              long long s_k, int row0, int rows, int k0, int K) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool kvec = (s_k == 1) && ((s_r & 7) == 0) &&
-                      ((reinterpret_cast<uintptr_t>(src) & 15) == 0);
-    // each thread stages 8 units; all loads are issued before the stores
-    constexpr int kU = 32 / (kGemmThreads / 32);
-    uint4 v[kU];
-    if (kvec) {
-        // 32 units per warp: 8 rows x 4 K units (512 contiguous bytes of the image)
+                                              long long s_k, int row0, int rows, int k0, int K, int t) {
+    const bool al = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+    if (s_k == 1 && (s_r & 7) == 0 && al) {
+        // K contiguous: 8 units of one row are 128 contiguous bytes
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int w = warp + u * (kGemmThreads / 32);
-            const int r = (w >> 1) * 8 + (lane & 7), kg = (w & 1) * 4 + (lane >> 3);
+        for (int u = 0; u < ROWS * 8 / 128; ++u) {
+            const int i = t + 128 * u, r = i >> 3, kg = i & 7;
             const int row = row0 + r, k = k0 + kg * 8;
-            v[u] = make_uint4(0u, 0u, 0u, 0u);
-            if (row < rows) {
-                if (k + 8 <= K) {
-                    v[u] = __ldg(reinterpret_cast<const uint4 *>(src + (long long)row * s_r + k));
-                } else if (k < K) {
-                    alignas(16) uint16_t t[8];
+            const int bytes = row < rows ? max(0, min(16, 2 * (K - k))) : 0;
+            copy16(img + (((r >> 3) * 8 + kg) * 64 + (r & 7) * 8),
+                   bytes ? src + (long long)row * s_r + k : src, bytes);
+        }
+    } else if (s_r == 1 && (s_k & 7) == 0 && al) {
+        // rows contiguous: thread = one 8-row x 8-K block (kg fixed per quarter-warp pass)
+        for (int i = t; i < ROWS; i += 128) {
+            const int rg = i % (ROWS / 8), kg = i / (ROWS / 8);
+            const int row = row0 + rg * 8, k = k0 + kg * 8;
+            uint4 v[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) t[e] = (k + e < K) ? src[(long long)row * s_r + k + e] : 0;
-                    v[u] = *reinterpret_cast<const uint4 *>(t);
+            for (int e = 0; e < 8; ++e) {
+                v[e] = make_uint4(0u, 0u, 0u, 0u);
+                if (k + e < K) {
+                    const uint16_t *p = src + (long long)(k + e) * s_k + row;
+                    if (row + 8 <= rows) {
+                        v[e] = __ldg(reinterpret_cast<const uint4 *>(p));
+                    } else if (row < rows) {
+                        alignas(16) uint16_t x[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) x[q] = row + q < rows ? p[q] : 0;
+                        v[e] = *reinterpret_cast<const uint4 *>(x);
+                    }
                 }
             }
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int w = warp + u * (kGemmThreads / 32);
-            const int r = (w >> 1) * 8 + (lane & 7), kg = (w & 1) * 4 + (lane >> 3);
-            *reinterpret_cast<uint4 *>(img + (((r >> 3) * 8 + kg) * 64 + (r & 7) * 8)) = v[u];
-        }
-    } else {
-        // transposed operand: lanes walk 32 consecutive rows (coalesced when s_r = 1)
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int w = warp + u * (kGemmThreads / 32);
-            const int r = (w & 3) * 32 + lane, kg = w >> 2;
-            const int row = row0 + r, k = k0 + kg * 8;
-            alignas(16) uint16_t t[8];
+            transpose8(v);
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                t[e] = (row < rows && k + e < K) ? src[(long long)row * s_r + (long long)(k + e) * s_k] : 0;
-            v[u] = *reinterpret_cast<const uint4 *>(t);
+                *reinterpret_cast<uint4 *>(img + ((rg * 8 + kg) * 64 + e * 8)) = v[e];
         }
+    } else {
+        // any strides (narrow or unaligned operands)
+        for (int i = t; i < ROWS * 8; i += 128) {
+            const int r = i % ROWS, kg = i / ROWS;
+            const int row = row0 + r, k = k0 + kg * 8;
+            alignas(16) uint16_t x[8];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int w = warp + u * (kGemmThreads / 32);
-            const int r = (w & 3) * 32 + lane, kg = w >> 2;
-            *reinterpret_cast<uint4 *>(img + (((r >> 3) * 8 + kg) * 64 + (r & 7) * 8)) = v[u];
+            for (int e = 0; e < 8; ++e)
+                x[e] = (row < rows && k + e < K) ? src[(long long)row * s_r + (long long)(k + e) * s_k] : 0;
+            *reinterpret_cast<uint4 *>(img + (((r >> 3) * 8 + kg) * 64 + (r & 7) * 8)) =
+                *reinterpret_cast<const uint4 *>(x);
         }
     }
 }
 
 struct GemmCtrl {
-    uint64_t bar[2];
+    uint64_t bar[kGemmStages];
     uint32_t tmem;
     int fail;
 };
@@ -145,24 +174,38 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const GemmArgs g
     using namespace tc;
     extern __shared__ __align__(1024) unsigned char gsm[];
     GemmCtrl &C = *reinterpret_cast<GemmCtrl *>(gsm);
-    uint16_t *img = reinterpret_cast<uint16_t *>(gsm + 1024);   // [2 buffers][A, B] 16 KB each
+    unsigned char *img = gsm + 1024;              // [kGemmStages][A 16 KB, B 8 KB]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.y * TBM, n0 = blockIdx.x * TBN;
     const int nvalid = min(TBN, g.N - n0);
     const int NT = (nvalid + 15) & ~15;                         // MMA N (multiple of 16)
     const int chunks = (g.K + TBK - 1) / TBK;
     if (tid == 0) {
-        bar_init(&C.bar[0], 1);
-        bar_init(&C.bar[1], 1);
+        for (int b = 0; b < kGemmStages; ++b) bar_init(&C.bar[b], 1);
         C.fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 64;" ::"r"(
                          su32(&C.tmem))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    auto stage = [&](int c) {
+        unsigned char *p = img + (size_t)(c % kGemmStages) * (kABytes + kBBytes);
+        if (tid < 128)
+            stage_operand<TBM>(reinterpret_cast<uint16_t *>(p), g.A, g.sAm, g.sAk, m0, g.M, c * TBK,
+                               g.K, tid);
+        else
+            stage_operand<TBN>(reinterpret_cast<uint16_t *>(p + kABytes), g.B, g.sBn, g.sBk, n0, g.N,
+                               c * TBK, g.K, tid - 128);
+    };
+    // one copy group per chunk, empty ones past the end
+    auto stage_group = [&](int c) {
+        if (c < chunks) stage(c);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < kGemmStages - 1; ++c) stage_group(c);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -170,53 +213,49 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const GemmArgs g
     const uint32_t idesc = idesc_bf16(TBM, NT);
     bool ok = true;
     int committed = 0;   // chunks whose MMAs thread 0 has committed
-    for (int c = 0; c < chunks && ok; ++c) {
-        const int b = c & 1;
-        uint16_t *Ai = img + (size_t)b * 2 * (kTileBytes / 2);
-        uint16_t *Bi = Ai + kTileBytes / 2;
-        if (c >= 2) {
-            // the MMAs of chunk c - 2 have read this buffer
-            long long i = 0;
-            while (!bar_try(&C.bar[b], (uint32_t)(((c - 2) >> 1) & 1)) && ++i < kGemmWait) {
-            }
-            if (i >= kGemmWait) C.fail = 1;
-            __syncthreads();
-            if (C.fail) {
-                ok = false;
-                break;
-            }
+    // waits until the MMAs of chunk c have read their buffer
+    auto mma_wait = [&](int c) {
+        long long i = 0;
+        while (!bar_try(&C.bar[c % kGemmStages], (uint32_t)((c / kGemmStages) & 1)) && ++i < kGemmWait) {
         }
-        stage_operand(Ai, g.A, g.sAm, g.sAk, m0, g.M, c * TBK, g.K);
-        stage_operand(Bi, g.B, g.sBn, g.sBk, n0, g.N, c * TBK, g.K);
+        return i < kGemmWait;
+    };
+    for (int c = 0; c < chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kGemmStages - 2) : "memory");
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
+        if (C.fail) {
+            ok = false;
+            break;
+        }
         if (tid == 0) {
             tc_fence_after();
-            const uint32_t a0 = su32(Ai), b0 = su32(Bi);
+            const uint32_t a0 = su32(img) + (uint32_t)(c % kGemmStages) * (kABytes + kBBytes);
+            const uint32_t b0 = a0 + kABytes;
 #pragma unroll
             for (int kk = 0; kk < TBK / 16; ++kk) {
                 const uint64_t ad = smem_desc(a0 + kk * 256u, 128u, 1024u);
                 const uint64_t bd = smem_desc(b0 + kk * 256u, 128u, 1024u);
                 mma_bf16_tc(tmem, ad, bd, idesc, (c | kk) ? 1u : 0u);
             }
-            mma_commit(&C.bar[b]);
+            mma_commit(&C.bar[c % kGemmStages]);
             ++committed;
         }
+        // the buffer of chunk c + 3 was read by chunk c - 1
+        if (c + kGemmStages - 1 < chunks && c >= 1 && !mma_wait(c - 1)) C.fail = 1;
+        stage_group(c + kGemmStages - 1);
     }
     // the last commit covers every MMA issued before it
-    if (ok && chunks > 0) {
-        const int c = chunks - 1;
-        long long i = 0;
-        while (!bar_try(&C.bar[c & 1], (uint32_t)((c >> 1) & 1)) && ++i < kGemmWait) {
-        }
-        if (i >= kGemmWait) ok = false;
-    }
+    if (ok && chunks > 0) ok = mma_wait(chunks - 1);
     tc_fence_after();
-    // epilogue: warp q owns tensor-memory lanes 32 q .. 32 q + 31 (output rows)
-    const int m = m0 + warp * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-    for (int cb = 0; cb < NT; cb += 16) {
+    // epilogue: lane quarter warp % 4 (output rows), column half warp / 4
+    const int m = m0 + (warp & 3) * 32 + lane;
+    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
+    const bool vec32 = (g.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    const bool vec16 = (g.ldc & 7) == 0 && (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    const bool vecm = (g.ldm & 7) == 0 && (reinterpret_cast<uintptr_t>(g.mask) & 15) == 0;
+    for (int cb = 16 * (warp >> 2); cb < NT; cb += 32) {
         float v[16];
         if (chunks > 0) {
             tmem_ld16(tmem + lane_base + (uint32_t)cb, v);
@@ -225,28 +264,59 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const GemmArgs g
             for (int j = 0; j < 16; ++j) v[j] = 0.f;
         }
         if (m >= g.M) continue;
+        const bool full = cb + 16 <= nvalid;
+        alignas(16) uint16_t mk[16];
+        if (g.epi & EPI_MASK) {
+            const uint16_t *mp = g.mask + (long long)m * g.ldm + n0 + cb;
+            if (full && vecm) {
+                *reinterpret_cast<uint4 *>(mk) = *reinterpret_cast<const uint4 *>(mp);
+                *reinterpret_cast<uint4 *>(mk + 8) = *reinterpret_cast<const uint4 *>(mp + 8);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) mk[j] = cb + j < nvalid ? mp[j] : 0;
+            }
+        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-            const int n = n0 + cb + j;
             if (cb + j >= nvalid) break;
             float x = ok ? v[j] : __int_as_float(0x7fc00000);
-            if (g.epi & EPI_BIAS) x += g.bias[n];
+            if (g.epi & EPI_BIAS) x += g.bias[n0 + cb + j];
             if (g.epi & EPI_RELU) x = fmaxf(x, 0.f);
-            if ((g.epi & EPI_MASK) && !(bf2f(g.mask[(long long)m * g.ldm + n]) > 0.f)) x = 0.f;
-            if (g.epi & EPI_BF16) {
-                static_cast<uint16_t *>(g.C)[(long long)m * g.ldc + n] = f2bf(x);
+            if ((g.epi & EPI_MASK) && !(bf2f(mk[j]) > 0.f)) x = 0.f;
+            v[j] = x;
+        }
+        if (g.epi & EPI_BF16) {
+            uint16_t *Cp = static_cast<uint16_t *>(g.C) + (long long)m * g.ldc + n0 + cb;
+            alignas(16) uint16_t h[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) h[j] = f2bf(v[j]);
+            if (full && vec16) {
+                *reinterpret_cast<uint4 *>(Cp) = *reinterpret_cast<const uint4 *>(h);
+                *reinterpret_cast<uint4 *>(Cp + 8) = *reinterpret_cast<const uint4 *>(h + 8);
             } else {
-                float *Cp = static_cast<float *>(g.C);
-                if (g.epi & EPI_ACCUM) x += Cp[(long long)m * g.ldc + n];
-                Cp[(long long)m * g.ldc + n] = x;
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (cb + j < nvalid) Cp[j] = h[j];
+            }
+        } else {
+            float *Cp = static_cast<float *>(g.C) + (long long)m * g.ldc + n0 + cb;
+            if (full && vec32) {
+#pragma unroll
+                for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<float4 *>(Cp + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (cb + j < nvalid) Cp[j] = v[j];
             }
         }
     }
-    if (!ok && tid == 0) {
-        // a wait ran out: let the MMAs in flight finish before the memory is
-        // released (the last commit on each buffer's barrier)
-        for (int bb = 0; bb < 2; ++bb) {
-            const int cnt = (committed + 1 - bb) / 2;
+    if (!ok) {
+        // a wait ran out: the copies and the MMAs in flight finish before the memory
+        // is released (the last commit on each buffer's barrier)
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        for (int bb = 0; tid == 0 && bb < kGemmStages; ++bb) {
+            const int cnt = (committed + kGemmStages - 1 - bb) / kGemmStages;
             if (cnt <= 0) continue;
             long long i = 0;
             while (!bar_try(&C.bar[bb], (uint32_t)((cnt - 1) & 1)) && ++i < kGemmWait) {
@@ -256,12 +326,12 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const GemmArgs g
     tc_fence_before();
     __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 64;" ::"r"(tmem) : "memory");
 }
 
 namespace {
 
-constexpr size_t kGemmSmem = 1024 + 4 * (size_t)kTileBytes;
+constexpr size_t kGemmSmem = 1024 + kGemmStages * (size_t)(kABytes + kBBytes);
 std::once_flag g_gemm_attr;
 
 }  // namespace
@@ -277,13 +347,25 @@ static cudaError_t gemm(const GemmArgs &g, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// db[n] = sum_m dz[m][n] (dz BF16 [M][N]), FP32 accumulation.
-__global__ void col_sum_kernel(const uint16_t *dz, int M, int N, float *db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+// db[n] = sum_m dz[m][n] (dz BF16 [M][N]), FP32 accumulation: 32 columns a CTA,
+// eight threads a column with every eighth row each (one thread per column
+// walked 256 rows in 13 us), their parts added in order.
+constexpr int kSumRows = 8;
+__global__ void __launch_bounds__(32 * kSumRows) col_sum_kernel(const uint16_t *dz, int M, int N, float *db) {
+    __shared__ float part[kSumRows][32];
+    const int c = threadIdx.x & 31, r = threadIdx.x >> 5, n = blockIdx.x * 32 + c;
     float s = 0.f;
-    for (int m = 0; m < M; ++m) s += bf2f(dz[(long long)m * N + n]);
-    db[n] = s;
+    if (n < N) {
+#pragma unroll 8
+        for (int m = r; m < M; m += kSumRows) s += bf2f(dz[(long long)m * N + n]);
+    }
+    part[r][c] = s;
+    __syncthreads();
+    if (r == 0 && n < N) {
+#pragma unroll
+        for (int q = 1; q < kSumRows; ++q) s += part[q][c];
+        db[n] = s;
+    }
 }
 
 __global__ void f32_to_bf16_kernel(const float *x, long long n, uint16_t *y) {
@@ -412,7 +494,7 @@ extern "C" int mdx_mlp_backward(const mdx_mlp *net, int batch, const uint16_t *x
         g.ldc = K;
         g.epi = EPI_NONE;
         if (gemm(g, s) != cudaSuccess) return set_last_error(MDX_ERR_CUDA, "mlp backward launch failed");
-        col_sum_kernel<<<(N + 127) / 128, 128, 0, s>>>(dz, batch, N, db[l]);
+        col_sum_kernel<<<(N + 31) / 32, 32 * kSumRows, 0, s>>>(dz, batch, N, db[l]);
         if (l > 0) {
             // dz_prev[m][k] = (sum_n dz[m][n] W[n][k]) * [act_l[m][k] > 0], BF16
             GemmArgs h{};
