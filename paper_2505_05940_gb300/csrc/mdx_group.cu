@@ -38,10 +38,12 @@
 //   warps 4-7 (epilogue, one tensor-memory lane quarter each): eta from the
 //           accumulators, then f accumulated in a second tensor-memory region;
 //           at the end of the step the partial forces go to global slots.
-// The CTAs of a group then meet at a group barrier (monotonic counter,
-// release / acquire, bounded spin); the owner CTA of each plate sums the
-// partial forces, steps the plate, writes its audio sample and its new q, and
-// the group meets again before the next step's Q images are built.
+// Two monotonic counters per group order the steps (release / acquire, bounded
+// spin): every CTA arrives at the first with its partial forces, on which the
+// owner CTA of each plate waits; it sums the parts, steps the plate, writes
+// its audio sample and its new q, and arrives at the second, on which all wait
+// before they fetch the next step's Q image.  (One counter for both would let
+// CTAs without a plate run ahead into the owners' count.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -354,7 +356,8 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         const unsigned nct = (unsigned)G.n_ctas;
         const int fcol = 2 * nt * Bp;          // first column of the force accumulators
         const int slot_in_group = cta - G.cta0;
-        unsigned *cnt = P.counters + gi;
+        // arrivals of every CTA with its partial forces, and of the owners with new q
+        unsigned *cnt_f = P.counters + 2 * gi, *cnt_q = cnt_f + 1;
         const long long TM = P.total_modes;
         long long ucount = 0;
         bool ok = true;
@@ -370,11 +373,11 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                             P.state_io[d.mode_off + j]);
         }
         epi_bar();
-        if (et == 0) {
+        if (et == 0 && owner) {
             __threadfence();
-            atomicAdd(cnt, 1u);
+            atomicAdd(cnt_q, 1u);
         }
-        auto group_wait = [&](unsigned target) {
+        auto group_wait = [&](unsigned *cnt, unsigned target) {
             if (et == 0) {
                 long long spins = 0;
                 while (ld_acq(cnt) < target) {
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         for (int it = 0; it < steps && ok; ++it) {
             const int n = P.n_begin + it;
             // ---- wait for every owner's q of this step, build the Q images
-            if (!group_wait(nct * (unsigned)(1 + 2 * it))) {
+            if (!group_wait(cnt_q, (unsigned)G.n_owners * (unsigned)(1 + it))) {
                 ok = false;
                 break;
             }
@@ -504,11 +507,11 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
             epi_bar();
             if (et == 0) {
                 __threadfence();
-                atomicAdd(cnt, 1u);
+                atomicAdd(cnt_f, 1u);
             }
             // ---- owners: gather the forces, step the plates, pickup, new q
             if (owner) {
-                if (!group_wait(nct * (unsigned)(2 + 2 * it))) {
+                if (!group_wait(cnt_f, nct * (unsigned)(1 + it))) {
                     ok = false;
                     break;
                 }
@@ -520,10 +523,23 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     float ys = 0.f, ye = 0.f;
                     for (int j = et; j < d.N; j += 128) {
                         const int pos = P.gpos[G.gpos_off + j];
-                        float f = 0.f;
-                        for (int s = 0; s < G.n_ctas; ++s)
-                            f += ldcg(P.part + G.part_off + ((long long)s * Bp + b) * G.Np + pos);
                         const long long m = d.mode_off + j;
+                        // the CTAs' parts in batches, all loads of a batch in flight at
+                        // once (one load per add took 45 us of the step for 38 CTAs and
+                        // plates of 400 modes), added in CTA order
+                        float f = 0.f;
+                        const float *part = P.part + G.part_off + (long long)b * G.Np + pos;
+                        const long long pst = (long long)Bp * G.Np;
+                        constexpr int kPB = 20;
+                        for (int s0 = 0; s0 < G.n_ctas; s0 += kPB) {
+                            float x[kPB];
+#pragma unroll
+                            for (int q = 0; q < kPB; ++q)
+                                x[q] = s0 + q < G.n_ctas ? ldcg(part + (s0 + q) * pst) : 0.f;
+#pragma unroll
+                            for (int q = 0; q < kPB; ++q)
+                                if (s0 + q < G.n_ctas) f += x[q];
+                        }
                         float x0 = P.state_io[m], x1 = P.state_io[TM + m];
                         float x2 = P.state_io[2 * TM + m], x3 = P.state_io[3 * TM + m];
                         sv_step(x0, x1, x2, x3, P.coef.eps[m], P.coef.rw2[m], P.coef.rw2lo[m],
@@ -555,12 +571,12 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     }
                     epi_bar();
                 }
+                if (et == 0) {
+                    __threadfence();
+                    atomicAdd(cnt_q, 1u);
+                }
             }
             epi_bar();
-            if (et == 0) {
-                __threadfence();
-                atomicAdd(cnt, 1u);
-            }
         }
         if (!ok && et == 0) {
             atomicExch((int *)gabort, 1);
@@ -945,6 +961,9 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
             owner_of[b] = d.cta0 + c;
             load[c] += inst[kgs[g].plates[b]].N;
         }
+        std::vector<int> owners(owner_of);
+        std::sort(owners.begin(), owners.end());
+        d.n_owners = (int)(std::unique(owners.begin(), owners.end()) - owners.begin());
         std::vector<int> kc, pi;
         for (int b = 0; b < d.B; ++b) {
             GrpPlate pl{};
@@ -994,7 +1013,7 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
     if (e == cudaSuccess) e = gupload(&gp->d_kap, std::vector<float>(std::max<long long>(kap_off, 1), 0.f));
     if (e == cudaSuccess) e = cudaMalloc(&gp->d_part, std::max<long long>(part_off, 1) * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&gp->d_qbuf, std::max<long long>(qbuf_off, 1) * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&gp->d_counters, std::max(ng, 1) * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc(&gp->d_counters, 2 * std::max(ng, 1) * sizeof(unsigned));
     // every plan sets the same (largest) limit, so plans of different sizes can
     // launch in any order
     if (e == cudaSuccess)
@@ -1034,7 +1053,7 @@ cudaError_t group_plan_launch(GroupPlan *g, const InstDesc *d_inst, const ModeCo
                               float *state_io, long long total_modes, int *status, int *abort_flag,
                               float l2_keep, cudaStream_t s) {
     if (!g || g->n_ctas == 0 || steps <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(g->d_counters, 0, g->groups.size() * sizeof(unsigned), s);
+    cudaError_t e = cudaMemsetAsync(g->d_counters, 0, 2 * g->groups.size() * sizeof(unsigned), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(g->d_qbuf, 0, g->qbuf_floats * sizeof(float), s);
     if (e != cudaSuccess) return e;
     GroupParams P{};

@@ -324,7 +324,7 @@ struct GrpDesc {
     long long qbuf_off;     // the group's Q image in global memory (the layout of the
                             // shared-memory Q region), written by the owners
     int q_floats;           // floats of the Q region (all classes, high and low parts)
-    int pad2;
+    int n_owners;           // CTAs that step at least one plate
 };
 
 // One stress mode of a kernel group (the MMA and epilogue work unit).
