@@ -32,8 +32,6 @@ constexpr int kChunkK = 4;             // stress modes reduced together
 constexpr int kUPartFloats = 1024;     // row groups x N_pad <= 256 threads x 4 columns
 constexpr int kParQmax = 2;            // parity layout: column quads per thread
 constexpr int kParMcMax = 16;          // parity layout: stress modes per chunk
-constexpr int kTensionWarpsPerBlock = 4;
-constexpr int kTensionMaxJ = 32;       // modes per lane (N <= 1024)
 
 enum KernelMode : int {
     MODE_FORWARD = 0,   // simulate: writes audio / checkpoints / final state

@@ -1,39 +1,94 @@
-// Strings (Kirchhoff-Carrier) and membranes (Berger): one warp per instance.
+// Strings (Kirchhoff-Carrier) and membranes (Berger): one warp per instance of up
+// to 128 modes, 2 to 8 warps (128 modes each) above.
 //
 // Per step (Sec. 3.2, Eq. 20 in difference form; Sec. 3.1, Eq. 8):
 //   S       = sum_nu lambda_nu q_nu^2                      (warp reduction)
 //   fnl_mu  = tau' lambda_mu q_mu S
 //   v, q    <- Stormer-Verlet difference-form update
-//   y^n     = sum_mu c_mu q^{n+1}_mu                       (warp reduction)
-// Lane l holds modes l, l+32, ...; the whole time loop runs inside the kernel
-// with the state in registers.  The same kernel re-runs a segment from a
-// checkpoint (storing every state) and sweeps a stored segment backwards
-// (adjoint recursion, J symmetric because fnl = grad V, V = tau'/4 S^2).
+//   y^n     = sum_mu c_mu q^{n+1}_mu
+// Lane l holds modes l, l + G, ... (G lanes; the other lanes repeat them); the
+// whole time loop runs inside the kernel with the state in registers.  The
+// same kernel re-runs a segment from a checkpoint (storing every state) and
+// sweeps a stored segment backwards (adjoint recursion, J symmetric because
+// fnl = grad V, V = tau'/4 S^2).
+//
+// Bound: the dependent chain of a step (update, lambda q^2, the shuffles of S),
+// so everything else is kept off it.  The pickup's terms go to shared memory
+// and are summed once per 32 steps, one step per lane (two interleaved
+// reductions per step took 410 cycles a step for 40 modes, this 330); the
+// reverse sweep's states arrive by asynchronous copies, a block of steps ahead
+// (a fit's step of 48 strings of 40 to 100 modes, forward, recompute and
+// reverse over 4 410 steps, took 5.6 ms with loads inside the step, now 3.5 ms).
+// Fewer lanes than 32 save shuffles where a lane's modes are few (see
+// launch_tension).
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "../../include/mdx.h"
 #include "mdx_common.cuh"
 
 namespace mdx {
 
-template <int J>
-__global__ void __launch_bounds__(32 * kTensionWarpsPerBlock)
-tension_kernel(const TensionParams P) {
-    const int lane = threadIdx.x & 31;
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (w >= P.n_list) return;
-    const int inst = P.list[w];
+namespace {
+
+constexpr int kPickRow = 33;     // pickup row stride (float2): lanes read rows without conflicts
+
+__device__ __forceinline__ void copy4(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Steps per staged block of the reverse sweep: two buffers of (q, v) rows.
+__host__ __device__ constexpr int rev_block(int J) { return J <= 2 ? 16 : 8; }
+
+}  // namespace
+
+// Sums over the instance: the group's lanes, then its warps in order (through
+// shared memory, double-buffered by step: one barrier).
+template <int G, int W, int V>
+__device__ __forceinline__ void instance_sum(float (&v)[V], float (*red)[V][W], int parity, int warp) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int x = 0; x < V; ++x) v[x] += __shfl_xor_sync(0xffffffffu, v[x], o);
+    if constexpr (W > 1) {
+        if ((threadIdx.x & 31) == 0)
+#pragma unroll
+            for (int x = 0; x < V; ++x) red[parity][x][warp] = v[x];
+        __syncthreads();
+#pragma unroll
+        for (int x = 0; x < V; ++x) {
+            v[x] = red[parity][x][0];
+#pragma unroll
+            for (int w = 1; w < W; ++w) v[x] += red[parity][x][w];
+        }
+    }
+}
+
+template <int J, int G, int W, bool REV>
+__global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) {
+    // per warp: forward pickup terms [32][kPickRow] x 2; reverse [2][U][2][32 J]
+    extern __shared__ __align__(16) float tsm_all[];
+    __shared__ float red[2][REV ? 2 : 1][W];
+    __shared__ float2 ypart[W][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *tsm = tsm_all + warp * (REV ? 2 * rev_block(J) * 2 * 32 * J : 2 * 32 * kPickRow);
+    const int inst = P.list[blockIdx.x];
     const InstDesc d = P.inst[inst];
     const int N = d.N;
     const long long mo = d.mode_off;
     const long long TM = P.total_modes;
     const float taup = d.taup;
+    const int l0 = (lane & (G - 1)) + warp * G * J;
+    const bool first = lane < G;        // the other lanes repeat the modes
 
     float eps[J], rw2[J], rw2l[J], r[J], b[J], c[J], clo[J], lam[J];
     float x0[J], x1[J], x2[J], x3[J];   // forward: q_hi, q_lo, v_hi, v_lo ; reverse: a_hi, a_lo, mu
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = lane + 32 * j;
+        const int m = l0 + G * j;
         const bool ok = m < N;
         eps[j] = ok ? P.coef.eps[mo + m] : 0.f;
         rw2[j] = ok ? P.coef.rw2[mo + m] : 0.f;
@@ -46,171 +101,233 @@ tension_kernel(const TensionParams P) {
     }
     const float *exc = P.exc ? P.exc + (long long)inst * P.total_steps : nullptr;
 
-    if (P.mode != MODE_REVERSE) {
+    if constexpr (!REV) {
         // ---------------------------------------------------------- forward / recompute
+        float2 *pk = reinterpret_cast<float2 *>(tsm);
         const float *src = P.state_io;
         if (P.mode == MODE_RECOMPUTE) src = P.ckpt + (long long)(P.n_begin / P.ckpt_K) * kStateArrays * TM;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int m = lane + 32 * j;
+            const int m = l0 + G * j;
             const bool ok = m < N;
             x0[j] = ok ? src[mo + m] : 0.f;
             x1[j] = ok ? src[TM + mo + m] : 0.f;
             x2[j] = ok ? src[2 * TM + mo + m] : 0.f;
             x3[j] = ok ? src[3 * TM + mo + m] : 0.f;
         }
-        float S = 0.f;
+        float S[1] = {0.f};
 #pragma unroll
-        for (int j = 0; j < J; ++j) S = fmaf(lam[j] * x0[j], x0[j], S);
-        S = warp_sum(S);
+        for (int j = 0; j < J; ++j) S[0] = fmaf(lam[j] * x0[j], x0[j], S[0]);
+        instance_sum<G, W, 1>(S, red, 1, warp);
         float *aud = P.audio ? P.audio + (long long)inst * P.total_steps : nullptr;
-        float ybuf = 0.f, ebuf = 0.f;
+        const bool rec = P.mode == MODE_RECOMPUTE;
+        const bool ckpt = P.mode == MODE_FORWARD && P.ckpt;
+        int ck_left = 0;                // steps to the next checkpoint
+        float *ck = ckpt ? P.ckpt + mo : nullptr;
+        float *sq = rec ? P.seg_q + mo : nullptr, *sv = rec ? P.seg_v + mo : nullptr;
         bool bad = false;
-        for (int it = 0; it < P.steps; ++it) {
-            const int n = P.n_begin + it;
-            if ((it & 31) == 0) {
-                const int nn = n + lane;
-                ebuf = (exc && nn < P.total_steps) ? exc[nn] : 0.f;
-            }
-            const float e = __shfl_sync(0xffffffffu, ebuf, it & 31);
-            if (P.mode == MODE_FORWARD && P.ckpt && (n % P.ckpt_K) == 0) {
-                float *ck = P.ckpt + (long long)(n / P.ckpt_K) * kStateArrays * TM;
+        float enext = (exc && P.n_begin + lane < P.total_steps && lane < P.steps) ? exc[P.n_begin + lane] : 0.f;
+        for (int i0 = 0; i0 < P.steps; i0 += 32) {
+            const int cnt = min(32, P.steps - i0);
+            const float ebuf = enext;
+            enext = (exc && i0 + 32 + lane < P.steps) ? exc[P.n_begin + i0 + 32 + lane] : 0.f;
+#pragma unroll 2
+            for (int i = 0; i < cnt; ++i) {
+                const float e = __shfl_sync(0xffffffffu, ebuf, i);
+                if (ckpt) {
+                    if (ck_left == 0) {
+                        ck_left = P.ckpt_K;
+#pragma unroll
+                        for (int j = 0; j < J; ++j) {
+                            const int m = l0 + G * j;
+                            if (first && m < N) {
+                                ck[m] = x0[j];
+                                ck[TM + m] = x1[j];
+                                ck[2 * TM + m] = x2[j];
+                                ck[3 * TM + m] = x3[j];
+                            }
+                        }
+                        ck += (long long)kStateArrays * TM;
+                    }
+                    --ck_left;
+                }
+                if (rec) {
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        const int m = l0 + G * j;
+                        if (first && m < N) {
+                            sq[m] = x0[j];
+                            sv[m] = x2[j];
+                        }
+                    }
+                    sq += TM;
+                    sv += TM;
+                }
+                float ys = 0.f, ye = 0.f, Sp[1] = {0.f};
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
-                    const int m = lane + 32 * j;
-                    if (m < N) {
-                        ck[mo + m] = x0[j];
-                        ck[TM + mo + m] = x1[j];
-                        ck[2 * TM + mo + m] = x2[j];
-                        ck[3 * TM + mo + m] = x3[j];
-                    }
+                    // everything that does not need S first
+                    const float tl = taup * lam[j] * x0[j];
+                    const float rest = fmaf(rw2[j], x0[j], fmaf(rw2l[j], x0[j], rw2[j] * x1[j]));
+                    const float g = fmaf(-eps[j], x2[j], -rest);
+                    const float dv = fmaf(r[j], fmaf(-tl, S[0], b[j] * e), g);
+                    // (v_hi, v_lo) += dv; q += v with v's sum not yet renormalised
+                    const float vs = x2[j] + dv;
+                    const float vb = vs - x2[j];
+                    const float vl = x3[j] + ((x2[j] - (vs - vb)) + (dv - vb));
+                    const float qs = x0[j] + vs;
+                    const float qb = qs - x0[j];
+                    const float ql = x1[j] + ((x0[j] - (qs - qb)) + (vs - qb)) + vl;
+                    x2[j] = vs + vl;
+                    x3[j] = vl - (x2[j] - vs);
+                    x0[j] = qs + ql;
+                    x1[j] = ql - (x0[j] - qs);
+                    Sp[0] = fmaf(lam[j] * x0[j], x0[j], Sp[0]);
                 }
-            }
-            if (P.mode == MODE_RECOMPUTE) {
+                instance_sum<G, W, 1>(Sp, red, i & 1, warp);
+                S[0] = Sp[0];
 #pragma unroll
-                for (int j = 0; j < J; ++j) {
-                    const int m = lane + 32 * j;
-                    if (m < N) {
-                        P.seg_q[(long long)it * TM + mo + m] = x0[j];
-                        P.seg_v[(long long)it * TM + mo + m] = x2[j];
-                    }
-                }
+                for (int j = 0; j < J; ++j) pickup_add(ys, ye, c[j], clo[j], x0[j], x1[j]);
+                pk[i * kPickRow + lane] = make_float2(ys, ye);
             }
-            float ys = 0.f, ye = 0.f, Sp = 0.f;
+            __syncwarp();
+            // lane l sums the terms of step i0 + l
+            float ys = 0.f, ye = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < G; ++k) {
+                const float2 v = pk[lane * kPickRow + k];
+                pickup_merge(ys, ye, v.x, v.y);
+            }
+            if constexpr (W > 1) {
+                ypart[warp][lane] = make_float2(ys, ye);
+                __syncthreads();
 #pragma unroll
-            for (int j = 0; j < J; ++j) {
-                const float f = taup * lam[j] * x0[j] * S;
-                sv_step(x0[j], x1[j], x2[j], x3[j], eps[j], rw2[j], rw2l[j], r[j], fmaf(b[j], e, -f));
-                pickup_add(ys, ye, c[j], clo[j], x0[j], x1[j]);
-                Sp = fmaf(lam[j] * x0[j], x0[j], Sp);
+                for (int w = 1; w < W; ++w)
+                    if (warp == 0) pickup_merge(ys, ye, ypart[w][lane].x, ypart[w][lane].y);
             }
+            if (lane < cnt && warp == 0) {
+                const float y = ys + ye;
+                if (aud) aud[P.n_begin + i0 + lane] = y;
+                if (!isfinite(y)) bad = true;
+            }
+            __syncwarp();
+        }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float s2 = __shfl_xor_sync(0xffffffffu, ys, o);
-                const float e2 = __shfl_xor_sync(0xffffffffu, ye, o);
-                pickup_merge(ys, ye, s2, e2);
-                Sp += __shfl_xor_sync(0xffffffffu, Sp, o);
-            }
-            const float yp = ys + ye;
-            S = Sp;
-            if (lane == (it & 31)) ybuf = yp;
-            if (!isfinite(yp)) bad = true;
-            if (aud && (((it & 31) == 31) || it == P.steps - 1)) {
-                const int base = n - (it & 31);
-                if (lane <= (it & 31)) aud[base + lane] = ybuf;
+        for (int j = 0; j < J; ++j) {
+            const int m = l0 + G * j;
+            if (!first || m >= N) continue;
+            if (rec) {
+                sq[m] = x0[j];
+                sv[m] = x2[j];
+            } else {
+                P.state_io[mo + m] = x0[j];
+                P.state_io[TM + mo + m] = x1[j];
+                P.state_io[2 * TM + mo + m] = x2[j];
+                P.state_io[3 * TM + mo + m] = x3[j];
             }
         }
-        if (P.mode == MODE_RECOMPUTE) {
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
-                const int m = lane + 32 * j;
-                if (m < N) {
-                    P.seg_q[(long long)P.steps * TM + mo + m] = x0[j];
-                    P.seg_v[(long long)P.steps * TM + mo + m] = x2[j];
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = 0; j < J; ++j) {
-                const int m = lane + 32 * j;
-                if (m < N) {
-                    P.state_io[mo + m] = x0[j];
-                    P.state_io[TM + mo + m] = x1[j];
-                    P.state_io[2 * TM + mo + m] = x2[j];
-                    P.state_io[3 * TM + mo + m] = x3[j];
-                }
-            }
-        }
+        bad = __any_sync(0xffffffffu, bad);
         if (bad && lane == 0) set_status(P.status, inst, MDX_ERR_NONFINITE);
-        return;
-    }
-
+    } else {
     // ------------------------------------------------------------------ reverse sweep
     // seg_q[t], seg_v[t] hold q^{n0+t}, v^{n0+t} for t = 0..steps.
+    constexpr int U = rev_block(J);
+    float q1[J];                        // q^{n+1}
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = lane + 32 * j;
+        const int m = l0 + G * j;
         const bool ok = m < N;
         x0[j] = ok ? P.adj[mo + m] : 0.f;
         x1[j] = ok ? P.adj[TM + mo + m] : 0.f;
         x2[j] = ok ? P.adj[2 * TM + mo + m] : 0.f;
+        q1[j] = ok ? P.seg_q[(long long)P.steps * TM + mo + m] : 0.f;
     }
     float gs[GA_N][J], gc[GA_N][J];
 #pragma unroll
     for (int g = 0; g < GA_N; ++g)
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int m = lane + 32 * j;
+            const int m = l0 + G * j;
             const bool ok = m < N;
             gs[g][j] = ok ? P.gacc[(long long)(2 * g) * TM + mo + m] : 0.f;
             gc[g][j] = ok ? P.gacc[(long long)(2 * g + 1) * TM + mo + m] : 0.f;
         }
     float ts = 0.f, tc = 0.f;
-    if (lane == 0) { ts = P.tacc[2 * inst]; tc = P.tacc[2 * inst + 1]; }
+    if (threadIdx.x == 0) { ts = P.tacc[2 * inst]; tc = P.tacc[2 * inst + 1]; }
     const float *yb = P.ybar + (long long)inst * P.total_steps;
     bool bad = false;
-    for (int it = P.steps - 1; it >= 0; --it) {
-        const int n = P.n_begin + it;
-        const float e = exc ? exc[n] : 0.f;
-        const float ybn = yb[n];
-        const float ybm = (n >= 1) ? yb[n - 1] : 0.f;
-        float q[J], v[J], q1[J], wv[J];
-        float S = 0.f, Pq = 0.f;
+    // block k: local steps t = steps - 1 - k U - u, u = 0 .. U - 1
+    auto stage = [&](int k) {
+        float *buf = tsm + (k & 1) * (U * 2 * 32 * J);
+        for (int u = 0; u < U; ++u) {
+            const int t = P.steps - 1 - k * U - u;
+            if (t < 0) break;
+            const float *sq = P.seg_q + (long long)t * TM + mo, *sv = P.seg_v + (long long)t * TM + mo;
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const int m = lane + 32 * j;
-            const bool ok = m < N;
-            q[j] = ok ? P.seg_q[(long long)it * TM + mo + m] : 0.f;
-            v[j] = ok ? P.seg_v[(long long)it * TM + mo + m] : 0.f;
-            q1[j] = ok ? P.seg_q[(long long)(it + 1) * TM + mo + m] : 0.f;
-            wv[j] = r[j] * x0[j];
-            S = fmaf(lam[j] * q[j], q[j], S);
-            Pq = fmaf(lam[j] * q[j], wv[j], Pq);
+            for (int j = 0; j < J; ++j) {
+                const int m = l0 + G * j;
+                float *dst = buf + (u * 2 * J + j) * 32 + lane;
+                if (m < N) {
+                    copy4(dst, sq + m);
+                    copy4(dst + 32 * J, sv + m);
+                }
+            }
         }
+    };
+    for (int e = lane; e < 2 * U * 2 * 32 * J; e += 32) tsm[e] = 0.f;   // lanes beyond N read zeros
+    stage(0);
+    // targets and excitation: a lane holds one of 32 steps
+    float ebuf = 0.f, ybuf = 0.f;
+    float ybn = P.steps > 0 ? yb[P.n_begin + P.steps - 1] : 0.f;
+    for (int k = 0; k * U < P.steps; ++k) {
+        copies_done();                  // each lane reads only what it copied
+        if ((k + 1) * U < P.steps) stage(k + 1);
+        const float *buf = tsm + (k & 1) * (U * 2 * 32 * J);
+#pragma unroll 1
+        for (int u = 0; u < U; ++u) {
+            const int s = k * U + u;
+            if (s >= P.steps) break;
+            if ((s & 31) == 0) {
+                const int tl = P.steps - 1 - s - lane, nl = P.n_begin + tl;
+                ebuf = (exc && tl >= 0) ? exc[nl] : 0.f;
+                ybuf = (tl >= 0 && nl >= 1) ? yb[nl - 1] : 0.f;
+            }
+            const float e = __shfl_sync(0xffffffffu, ebuf, s & 31);
+            const float ybm = __shfl_sync(0xffffffffu, ybuf, s & 31);
+            float q[J], wv[J];
+            float SP[2] = {0.f, 0.f};
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            S += __shfl_xor_sync(0xffffffffu, S, o);
-            Pq += __shfl_xor_sync(0xffffffffu, Pq, o);
-        }
+            for (int j = 0; j < J; ++j) {
+                q[j] = buf[(u * 2 * J + j) * 32 + lane];
+                wv[j] = r[j] * x0[j];
+                SP[0] = fmaf(lam[j] * q[j], q[j], SP[0]);
+                SP[1] = fmaf(lam[j] * q[j], wv[j], SP[1]);
+            }
+            instance_sum<G, W, 2>(SP, red, s & 1, warp);
+            const float S = SP[0], Pq = SP[1];
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const float a = x0[j];
-            const float f = taup * lam[j] * q[j] * S;
-            const float Jw = taup * lam[j] * fmaf(S, wv[j], 2.f * q[j] * Pq);
-            kahan_add(gs[GA_A][j], gc[GA_A][j], a * q[j]);
-            kahan_add(gs[GA_V][j], gc[GA_V][j], a * v[j]);
-            kahan_add(gs[GA_F][j], gc[GA_F][j], a * fmaf(b[j], e, -f));
-            kahan_add(gs[GA_E][j], gc[GA_E][j], a * e);
-            kahan_add(gs[GA_C][j], gc[GA_C][j], ybn * q1[j]);
-            adj_step(x0[j], x1[j], x2[j], eps[j], rw2[j], Jw, c[j] * ybm);
+            for (int j = 0; j < J; ++j) {
+                const float a = x0[j];
+                const float f = taup * lam[j] * q[j] * S;
+                const float Jw = taup * lam[j] * fmaf(S, wv[j], 2.f * q[j] * Pq);
+                adj_step(x0[j], x1[j], x2[j], eps[j], rw2[j], Jw, c[j] * ybm);
+                const float v = buf[(u * 2 * J + J + j) * 32 + lane];
+                kahan_add(gs[GA_A][j], gc[GA_A][j], a * q[j]);
+                kahan_add(gs[GA_V][j], gc[GA_V][j], a * v);
+                kahan_add(gs[GA_F][j], gc[GA_F][j], a * fmaf(b[j], e, -f));
+                kahan_add(gs[GA_E][j], gc[GA_E][j], a * e);
+                kahan_add(gs[GA_C][j], gc[GA_C][j], ybn * q1[j]);
+                q1[j] = q[j];
+            }
+            ybn = ybm;
+            if (threadIdx.x == 0) kahan_add(ts, tc, -S * Pq);
+            if (!isfinite(x0[0])) bad = true;
         }
-        if (lane == 0) kahan_add(ts, tc, -S * Pq);
-        if (!isfinite(x0[0])) bad = true;
     }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = lane + 32 * j;
-        if (m < N) {
+        const int m = l0 + G * j;
+        if (first && m < N) {
             P.adj[mo + m] = x0[j];
             P.adj[TM + mo + m] = x1[j];
             P.adj[2 * TM + mo + m] = x2[j];
@@ -221,36 +338,50 @@ tension_kernel(const TensionParams P) {
             }
         }
     }
-    if (lane == 0) { P.tacc[2 * inst] = ts; P.tacc[2 * inst + 1] = tc; }
+    if (threadIdx.x == 0) { P.tacc[2 * inst] = ts; P.tacc[2 * inst + 1] = tc; }
     if (bad && lane == 0) set_status(P.status, inst, MDX_ERR_NONFINITE);
+    }
 }
 
-// J (modes per lane) buckets: 1, 2, 4, 8, 16, 32.
-static int tension_bucket(int N) {
-    int j = (N + 31) / 32;
-    int b = 1;
-    while (b < j) b <<= 1;
-    return b;
-}
-
-template <int J>
+template <int J, int G, int W>
 static cudaError_t launch_j(const TensionParams &p, cudaStream_t s) {
-    const int threads = 32 * kTensionWarpsPerBlock;
-    const int blocks = (p.n_list + kTensionWarpsPerBlock - 1) / kTensionWarpsPerBlock;
-    if (blocks == 0) return cudaSuccess;
-    tension_kernel<J><<<blocks, threads, 0, s>>>(p);
+    if (p.n_list == 0) return cudaSuccess;
+    if (p.mode == MODE_REVERSE) {
+        const size_t smem = sizeof(float) * W * 2 * rev_block(J) * 2 * 32 * J;
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(
+                tension_kernel<J, G, W, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        tension_kernel<J, G, W, true><<<p.n_list, 32 * W, smem, s>>>(p);
+    } else {
+        const size_t smem = sizeof(float) * W * 2 * 32 * kPickRow;
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(
+                tension_kernel<J, G, W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        tension_kernel<J, G, W, false><<<p.n_list, 32 * W, smem, s>>>(p);
+    }
     return cudaGetLastError();
 }
 
+// Modes per lane, lanes and warps, by the largest instance: a halving of the
+// lanes saves one shuffle (29 cycles of the chain) and doubles a lane's modes
+// (about 35 instructions each, which must still fit the chain's 160 to 250
+// cycles); above 128 modes a further warp costs a barrier and a
+// shared-memory sum (about 90 cycles), four more modes per lane 140.
 cudaError_t launch_tension(const TensionParams &p, int max_n, cudaStream_t s) {
-    switch (tension_bucket(max_n)) {
-        case 1: return launch_j<1>(p, s);
-        case 2: return launch_j<2>(p, s);
-        case 4: return launch_j<4>(p, s);
-        case 8: return launch_j<8>(p, s);
-        case 16: return launch_j<16>(p, s);
-        default: return launch_j<32>(p, s);
-    }
+    if (max_n <= 8) return launch_j<1, 8, 1>(p, s);
+    if (max_n <= 16) return launch_j<1, 16, 1>(p, s);
+    if (max_n <= 32) return launch_j<2, 16, 1>(p, s);
+    if (max_n <= 48) return launch_j<3, 16, 1>(p, s);
+    if (max_n <= 64) return launch_j<2, 32, 1>(p, s);
+    if (max_n <= 96) return launch_j<3, 32, 1>(p, s);
+    if (max_n <= 128) return launch_j<4, 32, 1>(p, s);
+    if (max_n <= 256) return launch_j<4, 32, 2>(p, s);
+    if (max_n <= 512) return launch_j<4, 32, 4>(p, s);
+    return launch_j<4, 32, 8>(p, s);
 }
 
 }  // namespace mdx
