@@ -8,24 +8,23 @@
 // companion matrix A = [[g, p], [1, 0]], whose eigenvalues are the discrete
 // poles of the mode.  The paper evaluates such responses by repeated
 // multiplication with the poles organised as a prefix scan over time; here
-// the scan is blocked in time, in the difference form (q, v = q - q^{n-1}), whose
-// one-step matrix M = [[1 - rho, 1 - eps], [-rho, 1 - eps]] is similar to A:
+// the scan is blocked in time:
 //   1. every chunk of L steps runs its inputs from a zero state (all chunks
 //      and modes in parallel) and keeps only its final state E_j;
 //   2. per mode, the chunk boundary states follow sequentially,
-//      S_j = M^L S_{j-1} + E_j (M^L by repeated squaring, FP64), S_{-1} = X^0;
+//      S_j = A^L S_{j-1} + E_j (A^L by repeated squaring, FP64), S_{-1} = X^0;
 //   3. every chunk reruns from its true incoming state S_{j-1} and writes the
 //      pickup y^n = sum_mu c_mu q_mu^{n+1}.
 //
 // Arithmetic of the passes over the steps: unevaluated FP32 pairs (about 48
-// bits) for state, coefficients and products.  The FP64 units do 2 operations
-// a cycle and SM, the FP32 units 128; a step costs 48 of the latter against 3
-// to 4 of the former, and 64 objects of 20 to 400 modes over 22 050 steps took
-// 5.1 ms in FP64, 0.95 ms so.  The pairs in difference form are no less exact
-// than FP64 in the companion form, whose coefficients g = 2 - eps - rho drop
-// the digits of rho: final states were 4.6e-9 off the difference form in FP64,
-// now 5e-13.  The pickup's terms go through shared memory and each lane sums
-// one step (shuffle sums of every step were the larger half of the time).
+// bits) for state, coefficients and products, in the difference form
+// (q, v = q - q^{n-1}).  The FP64 units do 2 operations a cycle and SM, the FP32
+// units 128; a step costs 48 of the latter against 3 to 4 of the former, and 64
+// objects of 20 to 400 modes over 22 050 steps took 5.1 ms in FP64, 0.86 ms so.
+// The chain over the chunks stays in the FP64 companion form: its rounding sets
+// the digits of the final states beyond the eighth.  The pickup's terms go
+// through shared memory and each lane sums one step (shuffle sums of every step
+// were the larger half of the time).
 #include <cuda_runtime.h>
 
 #include "../../include/mdx.h"
@@ -74,8 +73,15 @@ struct LinCoef {
     Pair neps, nrho, rb;
 };
 
+// eps and rho of the companion form as FP64 holds it: g = 2 - eps - rho and
+// p = eps - 1 are rounded there (rho of a slow mode loses digits against 2), and
+// the difference form of the same recursion keeps those digits, not more.
 __device__ __forceinline__ SchemeCoef scheme_of(const LinearParams &P, long long gm) {
-    return scheme_coef(P.scheme, P.omega2[gm], P.gamma[gm], P.dt[gm]);
+    SchemeCoef k = scheme_coef(P.scheme, P.omega2[gm], P.gamma[gm], P.dt[gm]);
+    const double p = k.eps - 1.0, g = 2.0 - k.eps - k.rho;
+    k.eps = 1.0 + p;
+    k.rho = (1.0 - g) - p;
+    return k;
 }
 
 __device__ __forceinline__ LinCoef lin_coef(const LinearParams &P, long long gm) {
@@ -117,16 +123,16 @@ __global__ void __launch_bounds__(kLinThreads) lin_local_kernel(const LinearPara
         for (int n = 0; n < n1 - n0; ++n) lin_step(k, es[n], q, v);
         double *E = P.E + ((long long)j * P.total_modes + d.mode_off + m) * 2;
         E[0] = value(q);
-        E[1] = value(v);
+        E[1] = value(q) - value(v);
     }
 }
 
 __global__ void lin_carry_kernel(const LinearParams P) {
     const long long gmode = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (gmode >= P.total_modes) return;
-    const SchemeCoef k = scheme_of(P, gmode);
-    // M^L by repeated squaring
-    double a00 = 1.0 - k.rho, a01 = 1.0 - k.eps, a10 = -k.rho, a11 = 1.0 - k.eps;
+    const SchemeCoef k = scheme_coef(P.scheme, P.omega2[gmode], P.gamma[gmode], P.dt[gmode]);
+    // A^L by repeated squaring
+    double a00 = 2.0 - k.eps - k.rho, a01 = k.eps - 1.0, a10 = 1.0, a11 = 0.0;
     double r00 = 1.0, r01 = 0.0, r10 = 0.0, r11 = 1.0;
     for (int L = P.L; L > 0; L >>= 1) {
         if (L & 1) {
@@ -138,12 +144,11 @@ __global__ void lin_carry_kernel(const LinearParams P) {
         const double s10 = a10 * a00 + a11 * a10, s11 = a10 * a01 + a11 * a11;
         a00 = s00, a01 = s01, a10 = s10, a11 = s11;
     }
-    double q = P.q0 ? P.q0[gmode] : 0.0;
-    double v = q - (P.qm1 ? P.qm1[gmode] : 0.0);
+    double s0 = P.q0 ? P.q0[gmode] : 0.0, s1 = P.qm1 ? P.qm1[gmode] : 0.0;
     const long long st = P.total_modes * 2;
     double *S = P.S + gmode * 2;
-    S[0] = q;
-    S[1] = v;
+    S[0] = s0;
+    S[1] = s1;
     // the next chunks' end states are loaded together, ahead of the chain
     constexpr int U = 8;
     for (int j0 = 0; j0 < P.n_chunks - 1; j0 += U) {
@@ -158,12 +163,12 @@ __global__ void lin_carry_kernel(const LinearParams P) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (j0 + u >= P.n_chunks - 1) break;
-            const double t0 = fma(r00, q, fma(r01, v, e0[u]));
-            v = fma(r10, q, fma(r11, v, e1[u]));
-            q = t0;
+            const double t0 = fma(r00, s0, fma(r01, s1, e0[u]));
+            s1 = fma(r10, s0, fma(r11, s1, e1[u]));
+            s0 = t0;
             double *Sj = P.S + (long long)(j0 + u + 1) * st + gmode * 2;
-            Sj[0] = q;
-            Sj[1] = v;
+            Sj[0] = s0;
+            Sj[1] = s1;
         }
     }
 }
@@ -189,7 +194,7 @@ __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams
             k = lin_coef(P, gm);
             const double *S = P.S + ((long long)j * P.total_modes + gm) * 2;
             q = pair_of(S[0]);
-            v = pair_of(S[1]);
+            v = pair_of(S[0] - S[1]);
             c = pair_of(P.c[gm]);
         }
         const int modes = min(32, d.N - m0);
