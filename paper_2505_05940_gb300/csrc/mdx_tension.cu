@@ -6,8 +6,8 @@
 //   fnl_mu  = tau' lambda_mu q_mu S
 //   v, q    <- Stormer-Verlet difference-form update
 //   y^n     = sum_mu c_mu q^{n+1}_mu
-// Lane l holds modes l, l + G, ... (G lanes; the other lanes repeat them); the
-// whole time loop runs inside the kernel with the state in registers.  The
+// Lane l holds modes l, l + 32, ...; the whole time loop runs inside the kernel
+// with the state in registers.  The
 // same kernel re-runs a segment from a checkpoint (storing every state) and
 // sweeps a stored segment backwards (adjoint recursion, J symmetric because
 // fnl = grad V, V = tau'/4 S^2).
@@ -15,12 +15,10 @@
 // Bound: the dependent chain of a step (update, lambda q^2, the shuffles of S),
 // so everything else is kept off it.  The pickup's terms go to shared memory
 // and are summed once per 32 steps, one step per lane (two interleaved
-// reductions per step took 410 cycles a step for 40 modes, this 330); the
+// reductions per step took 410 cycles a step for 40 modes, this 290); the
 // reverse sweep's states arrive by asynchronous copies, a block of steps ahead
 // (a fit's step of 48 strings of 40 to 100 modes, forward, recompute and
-// reverse over 4 410 steps, took 5.6 ms with loads inside the step, now 3.5 ms).
-// Fewer lanes than 32 save shuffles where a lane's modes are few (see
-// launch_tension).
+// reverse over 4 410 steps, took 5.6 ms with loads inside the step, now 3.6 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,12 +43,12 @@ __host__ __device__ constexpr int rev_block(int J) { return J <= 2 ? 16 : 8; }
 
 }  // namespace
 
-// Sums over the instance: the group's lanes, then its warps in order (through
+// Sums over the instance: the lanes, then the warps in order (through
 // shared memory, double-buffered by step: one barrier).
-template <int G, int W, int V>
+template <int W, int V>
 __device__ __forceinline__ void instance_sum(float (&v)[V], float (*red)[V][W], int parity, int warp) {
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1)
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
         for (int x = 0; x < V; ++x) v[x] += __shfl_xor_sync(0xffffffffu, v[x], o);
     if constexpr (W > 1) {
@@ -67,7 +65,7 @@ __device__ __forceinline__ void instance_sum(float (&v)[V], float (*red)[V][W], 
     }
 }
 
-template <int J, int G, int W, bool REV>
+template <int J, int W, bool REV>
 __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) {
     // per warp: forward pickup terms [32][kPickRow] x 2; reverse [2][U][2][32 J]
     extern __shared__ __align__(16) float tsm_all[];
@@ -81,14 +79,13 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
     const long long mo = d.mode_off;
     const long long TM = P.total_modes;
     const float taup = d.taup;
-    const int l0 = (lane & (G - 1)) + warp * G * J;
-    const bool first = lane < G;        // the other lanes repeat the modes
+    const int l0 = lane + warp * 32 * J;
 
     float eps[J], rw2[J], rw2l[J], r[J], b[J], c[J], clo[J], lam[J];
     float x0[J], x1[J], x2[J], x3[J];   // forward: q_hi, q_lo, v_hi, v_lo ; reverse: a_hi, a_lo, mu
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = l0 + G * j;
+        const int m = l0 + 32 * j;
         const bool ok = m < N;
         eps[j] = ok ? P.coef.eps[mo + m] : 0.f;
         rw2[j] = ok ? P.coef.rw2[mo + m] : 0.f;
@@ -108,7 +105,7 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
         if (P.mode == MODE_RECOMPUTE) src = P.ckpt + (long long)(P.n_begin / P.ckpt_K) * kStateArrays * TM;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int m = l0 + G * j;
+            const int m = l0 + 32 * j;
             const bool ok = m < N;
             x0[j] = ok ? src[mo + m] : 0.f;
             x1[j] = ok ? src[TM + mo + m] : 0.f;
@@ -118,83 +115,87 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
         float S[1] = {0.f};
 #pragma unroll
         for (int j = 0; j < J; ++j) S[0] = fmaf(lam[j] * x0[j], x0[j], S[0]);
-        instance_sum<G, W, 1>(S, red, 1, warp);
+        instance_sum<W, 1>(S, red, 1, warp);
         float *aud = P.audio ? P.audio + (long long)inst * P.total_steps : nullptr;
         const bool rec = P.mode == MODE_RECOMPUTE;
         const bool ckpt = P.mode == MODE_FORWARD && P.ckpt;
-        int ck_left = 0;                // steps to the next checkpoint
         float *ck = ckpt ? P.ckpt + mo : nullptr;
         float *sq = rec ? P.seg_q + mo : nullptr, *sv = rec ? P.seg_v + mo : nullptr;
         bool bad = false;
-        float enext = (exc && P.n_begin + lane < P.total_steps && lane < P.steps) ? exc[P.n_begin + lane] : 0.f;
-        for (int i0 = 0; i0 < P.steps; i0 += 32) {
-            const int cnt = min(32, P.steps - i0);
-            const float ebuf = enext;
-            enext = (exc && i0 + 32 + lane < P.steps) ? exc[P.n_begin + i0 + 32 + lane] : 0.f;
-#pragma unroll 2
-            for (int i = 0; i < cnt; ++i) {
-                const float e = __shfl_sync(0xffffffffu, ebuf, i);
-                if (ckpt) {
-                    if (ck_left == 0) {
-                        ck_left = P.ckpt_K;
+        auto store2 = [&](float *dq, float *dv) {
 #pragma unroll
-                        for (int j = 0; j < J; ++j) {
-                            const int m = l0 + G * j;
-                            if (first && m < N) {
-                                ck[m] = x0[j];
-                                ck[TM + m] = x1[j];
-                                ck[2 * TM + m] = x2[j];
-                                ck[3 * TM + m] = x3[j];
-                            }
-                        }
-                        ck += (long long)kStateArrays * TM;
-                    }
-                    --ck_left;
+            for (int j = 0; j < J; ++j) {
+                const int m = l0 + 32 * j;
+                if (m < N) {
+                    dq[m] = x0[j];
+                    dv[m] = x2[j];
                 }
-                if (rec) {
+            }
+        };
+        // one step; the pickup's terms go to row i
+        int par = 0;
+        auto step = [&](int i, float e) {
+            float Sp[1] = {0.f};
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const float f = taup * lam[j] * x0[j] * S[0];
+                sv_step(x0[j], x1[j], x2[j], x3[j], eps[j], rw2[j], rw2l[j], r[j], fmaf(b[j], e, -f));
+                Sp[0] = fmaf(lam[j] * x0[j], x0[j], Sp[0]);
+            }
+            instance_sum<W, 1>(Sp, red, par, warp);
+            S[0] = Sp[0];
+            par ^= 1;
+            // the first mode's term starts the compensated sum
+            float ys = c[0] * x0[0];
+            float ye = fmaf(c[0], x1[0], fmaf(clo[0], x0[0], fmaf(c[0], x0[0], -ys)));
+#pragma unroll
+            for (int j = 1; j < J; ++j) pickup_add(ys, ye, c[j], clo[j], x0[j], x1[j]);
+            pk[i * kPickRow + lane] = make_float2(ys, ye);
+        };
+        auto load_e = [&](int i) {
+            return (exc && i + lane < P.steps) ? exc[P.n_begin + i + lane] : 0.f;
+        };
+        // blocks of at most 32 steps that end at the checkpoints
+        int ck_left = 0;
+        float enext = load_e(0);
+        for (int i0 = 0; i0 < P.steps;) {
+            int cnt = min(32, P.steps - i0);
+            if (ckpt) {
+                if (ck_left == 0) {
+                    ck_left = P.ckpt_K;
+                    store2(ck, ck + 2 * TM);
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
-                        const int m = l0 + G * j;
-                        if (first && m < N) {
-                            sq[m] = x0[j];
-                            sv[m] = x2[j];
+                        const int m = l0 + 32 * j;
+                        if (m < N) {
+                            ck[TM + m] = x1[j];
+                            ck[3 * TM + m] = x3[j];
                         }
                     }
+                    ck += (long long)kStateArrays * TM;
+                }
+                cnt = min(cnt, ck_left);
+                ck_left -= cnt;
+            }
+            const float ebuf = enext;
+            enext = load_e(i0 + cnt);
+            if (rec) {
+#pragma unroll 2
+                for (int i = 0; i < cnt; ++i) {
+                    store2(sq, sv);
                     sq += TM;
                     sv += TM;
+                    step(i, __shfl_sync(0xffffffffu, ebuf, i));
                 }
-                float ys = 0.f, ye = 0.f, Sp[1] = {0.f};
-#pragma unroll
-                for (int j = 0; j < J; ++j) {
-                    // everything that does not need S first
-                    const float tl = taup * lam[j] * x0[j];
-                    const float rest = fmaf(rw2[j], x0[j], fmaf(rw2l[j], x0[j], rw2[j] * x1[j]));
-                    const float g = fmaf(-eps[j], x2[j], -rest);
-                    const float dv = fmaf(r[j], fmaf(-tl, S[0], b[j] * e), g);
-                    // (v_hi, v_lo) += dv; q += v with v's sum not yet renormalised
-                    const float vs = x2[j] + dv;
-                    const float vb = vs - x2[j];
-                    const float vl = x3[j] + ((x2[j] - (vs - vb)) + (dv - vb));
-                    const float qs = x0[j] + vs;
-                    const float qb = qs - x0[j];
-                    const float ql = x1[j] + ((x0[j] - (qs - qb)) + (vs - qb)) + vl;
-                    x2[j] = vs + vl;
-                    x3[j] = vl - (x2[j] - vs);
-                    x0[j] = qs + ql;
-                    x1[j] = ql - (x0[j] - qs);
-                    Sp[0] = fmaf(lam[j] * x0[j], x0[j], Sp[0]);
-                }
-                instance_sum<G, W, 1>(Sp, red, i & 1, warp);
-                S[0] = Sp[0];
-#pragma unroll
-                for (int j = 0; j < J; ++j) pickup_add(ys, ye, c[j], clo[j], x0[j], x1[j]);
-                pk[i * kPickRow + lane] = make_float2(ys, ye);
+            } else {
+#pragma unroll 4
+                for (int i = 0; i < cnt; ++i) step(i, __shfl_sync(0xffffffffu, ebuf, i));
             }
             __syncwarp();
             // lane l sums the terms of step i0 + l
             float ys = 0.f, ye = 0.f;
 #pragma unroll 8
-            for (int k = 0; k < G; ++k) {
+            for (int k = 0; k < 32; ++k) {
                 const float2 v = pk[lane * kPickRow + k];
                 pickup_merge(ys, ye, v.x, v.y);
             }
@@ -211,11 +212,12 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
                 if (!isfinite(y)) bad = true;
             }
             __syncwarp();
+            i0 += cnt;
         }
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int m = l0 + G * j;
-            if (!first || m >= N) continue;
+            const int m = l0 + 32 * j;
+            if (m >= N) continue;
             if (rec) {
                 sq[m] = x0[j];
                 sv[m] = x2[j];
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
     float q1[J];                        // q^{n+1}
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = l0 + G * j;
+        const int m = l0 + 32 * j;
         const bool ok = m < N;
         x0[j] = ok ? P.adj[mo + m] : 0.f;
         x1[j] = ok ? P.adj[TM + mo + m] : 0.f;
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
     for (int g = 0; g < GA_N; ++g)
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const int m = l0 + G * j;
+            const int m = l0 + 32 * j;
             const bool ok = m < N;
             gs[g][j] = ok ? P.gacc[(long long)(2 * g) * TM + mo + m] : 0.f;
             gc[g][j] = ok ? P.gacc[(long long)(2 * g + 1) * TM + mo + m] : 0.f;
@@ -265,7 +267,7 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
             const float *sq = P.seg_q + (long long)t * TM + mo, *sv = P.seg_v + (long long)t * TM + mo;
 #pragma unroll
             for (int j = 0; j < J; ++j) {
-                const int m = l0 + G * j;
+                const int m = l0 + 32 * j;
                 float *dst = buf + (u * 2 * J + j) * 32 + lane;
                 if (m < N) {
                     copy4(dst, sq + m);
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
                 SP[0] = fmaf(lam[j] * q[j], q[j], SP[0]);
                 SP[1] = fmaf(lam[j] * q[j], wv[j], SP[1]);
             }
-            instance_sum<G, W, 2>(SP, red, s & 1, warp);
+            instance_sum<W, 2>(SP, red, s & 1, warp);
             const float S = SP[0], Pq = SP[1];
 #pragma unroll
             for (int j = 0; j < J; ++j) {
@@ -326,8 +328,8 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
     }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        const int m = l0 + G * j;
-        if (first && m < N) {
+        const int m = l0 + 32 * j;
+        if (m < N) {
             P.adj[mo + m] = x0[j];
             P.adj[TM + mo + m] = x1[j];
             P.adj[2 * TM + mo + m] = x2[j];
@@ -343,45 +345,40 @@ __global__ void __launch_bounds__(32 * W) tension_kernel(const TensionParams P) 
     }
 }
 
-template <int J, int G, int W>
+template <int J, int W>
 static cudaError_t launch_j(const TensionParams &p, cudaStream_t s) {
     if (p.n_list == 0) return cudaSuccess;
     if (p.mode == MODE_REVERSE) {
         const size_t smem = sizeof(float) * W * 2 * rev_block(J) * 2 * 32 * J;
         if (smem > 48 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(
-                tension_kernel<J, G, W, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                tension_kernel<J, W, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        tension_kernel<J, G, W, true><<<p.n_list, 32 * W, smem, s>>>(p);
+        tension_kernel<J, W, true><<<p.n_list, 32 * W, smem, s>>>(p);
     } else {
         const size_t smem = sizeof(float) * W * 2 * 32 * kPickRow;
         if (smem > 48 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(
-                tension_kernel<J, G, W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                tension_kernel<J, W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        tension_kernel<J, G, W, false><<<p.n_list, 32 * W, smem, s>>>(p);
+        tension_kernel<J, W, false><<<p.n_list, 32 * W, smem, s>>>(p);
     }
     return cudaGetLastError();
 }
 
-// Modes per lane, lanes and warps, by the largest instance: a halving of the
-// lanes saves one shuffle (29 cycles of the chain) and doubles a lane's modes
-// (about 35 instructions each, which must still fit the chain's 160 to 250
-// cycles); above 128 modes a further warp costs a barrier and a
-// shared-memory sum (about 90 cycles), four more modes per lane 140.
+// Modes per lane and warps, by the largest instance: each further mode of a lane
+// adds about 35 instructions to a step; above four a further warp costs less (a
+// barrier and a shared-memory sum, about 90 cycles, against 140).
 cudaError_t launch_tension(const TensionParams &p, int max_n, cudaStream_t s) {
-    if (max_n <= 8) return launch_j<1, 8, 1>(p, s);
-    if (max_n <= 16) return launch_j<1, 16, 1>(p, s);
-    if (max_n <= 32) return launch_j<2, 16, 1>(p, s);
-    if (max_n <= 48) return launch_j<3, 16, 1>(p, s);
-    if (max_n <= 64) return launch_j<2, 32, 1>(p, s);
-    if (max_n <= 96) return launch_j<3, 32, 1>(p, s);
-    if (max_n <= 128) return launch_j<4, 32, 1>(p, s);
-    if (max_n <= 256) return launch_j<4, 32, 2>(p, s);
-    if (max_n <= 512) return launch_j<4, 32, 4>(p, s);
-    return launch_j<4, 32, 8>(p, s);
+    if (max_n <= 32) return launch_j<1, 1>(p, s);
+    if (max_n <= 64) return launch_j<2, 1>(p, s);
+    if (max_n <= 96) return launch_j<3, 1>(p, s);
+    if (max_n <= 128) return launch_j<4, 1>(p, s);
+    if (max_n <= 256) return launch_j<4, 2>(p, s);
+    if (max_n <= 512) return launch_j<4, 4>(p, s);
+    return launch_j<4, 8>(p, s);
 }
 
 }  // namespace mdx
