@@ -20,7 +20,7 @@
 // network are small (256 x 512 x 1024 at most), so each is the latency of its
 // chunks: with synchronous staging, element gathers of transposed operands and
 // one 128 x 128 tile per CTA a forward and backward pass of batch 256 took
-// 510 us, now 266 us.
+// 519 us, now 144 us.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -162,6 +162,16 @@ __device__ __forceinline__ void stage_operand(uint16_t *img, const uint16_t *src
     }
 }
 
+// One launch: up to two independent GEMMs (of one layer's backward pass) and a
+// column sum, in consecutive block ranges.
+struct LayerArgs {
+    GemmArgs g[2];
+    int nx[2], tiles[2];           // output tiles along N, in all
+    const uint16_t *dz;            // column sum: db[n] = sum_m dz[m][n] (null: none)
+    int M, N;
+    float *db;
+};
+
 struct GemmCtrl {
     uint64_t bar[kGemmStages];
     uint32_t tmem;
@@ -170,13 +180,42 @@ struct GemmCtrl {
 
 }  // namespace
 
-__global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const GemmArgs g) {
+// db[n] = sum_m dz[m][n] (dz BF16 [M][N]), FP32 accumulation: 32 columns a CTA,
+// eight threads a column with every eighth row each (one thread per column
+// walked 256 rows in 13 us), their parts added in order.
+constexpr int kSumRows = kGemmThreads / 32;
+__device__ void col_sum(const uint16_t *dz, int M, int N, float *db, int block) {
+    __shared__ float part[kSumRows][32];
+    const int c = threadIdx.x & 31, r = threadIdx.x >> 5, n = block * 32 + c;
+    float s = 0.f;
+    if (n < N) {
+#pragma unroll 8
+        for (int m = r; m < M; m += kSumRows) s += bf2f(dz[(long long)m * N + n]);
+    }
+    part[r][c] = s;
+    __syncthreads();
+    if (r == 0 && n < N) {
+#pragma unroll
+        for (int q = 1; q < kSumRows; ++q) s += part[q][c];
+        db[n] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const __grid_constant__ LayerArgs A) {
     using namespace tc;
+    int blk = blockIdx.x;
+    if (blk >= A.tiles[0] + A.tiles[1]) {
+        col_sum(A.dz, A.M, A.N, A.db, blk - A.tiles[0] - A.tiles[1]);
+        return;
+    }
+    const int which = blk >= A.tiles[0] ? 1 : 0;
+    const GemmArgs &g = A.g[which];
+    if (which) blk -= A.tiles[0];
     extern __shared__ __align__(1024) unsigned char gsm[];
     GemmCtrl &C = *reinterpret_cast<GemmCtrl *>(gsm);
     unsigned char *img = gsm + 1024;              // [kGemmStages][A 16 KB, B 8 KB]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TBM, n0 = blockIdx.x * TBN;
+    const int m0 = blk / A.nx[which] * TBM, n0 = blk % A.nx[which] * TBN;
     const int nvalid = min(TBN, g.N - n0);
     const int NT = (nvalid + 15) & ~15;                         // MMA N (multiple of 16)
     const int chunks = (g.K + TBK - 1) / TBK;
@@ -336,36 +375,30 @@ std::once_flag g_gemm_attr;
 
 }  // namespace
 
-static cudaError_t gemm(const GemmArgs &g, cudaStream_t s) {
-    if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+// Launches the GEMMs g0 (and g1, may be null) and the column sum of dz into db.
+static cudaError_t layer(const GemmArgs *g0, const GemmArgs *g1, const uint16_t *dz, int M, int N,
+                         float *db, cudaStream_t s) {
     std::call_once(g_gemm_attr, [] {
         cudaFuncSetAttribute(mlp_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kGemmSmem);
     });
-    dim3 grid((g.N + TBN - 1) / TBN, (g.M + TBM - 1) / TBM);
-    mlp_gemm_kernel<<<grid, kGemmThreads, kGemmSmem, s>>>(g);
+    LayerArgs A{};
+    const GemmArgs *gs[2] = {g0, g1};
+    for (int i = 0; i < 2; ++i) {
+        A.nx[i] = 1;
+        if (!gs[i] || gs[i]->M <= 0 || gs[i]->N <= 0) continue;
+        A.g[i] = *gs[i];
+        A.nx[i] = (gs[i]->N + TBN - 1) / TBN;
+        A.tiles[i] = A.nx[i] * ((gs[i]->M + TBM - 1) / TBM);
+    }
+    A.dz = dz;
+    A.M = M;
+    A.N = N;
+    A.db = db;
+    const int blocks = A.tiles[0] + A.tiles[1] + (dz ? (N + 31) / 32 : 0);
+    if (blocks == 0) return cudaSuccess;
+    mlp_gemm_kernel<<<blocks, kGemmThreads, kGemmSmem, s>>>(A);
     return cudaGetLastError();
-}
-
-// db[n] = sum_m dz[m][n] (dz BF16 [M][N]), FP32 accumulation: 32 columns a CTA,
-// eight threads a column with every eighth row each (one thread per column
-// walked 256 rows in 13 us), their parts added in order.
-constexpr int kSumRows = 8;
-__global__ void __launch_bounds__(32 * kSumRows) col_sum_kernel(const uint16_t *dz, int M, int N, float *db) {
-    __shared__ float part[kSumRows][32];
-    const int c = threadIdx.x & 31, r = threadIdx.x >> 5, n = blockIdx.x * 32 + c;
-    float s = 0.f;
-    if (n < N) {
-#pragma unroll 8
-        for (int m = r; m < M; m += kSumRows) s += bf2f(dz[(long long)m * N + n]);
-    }
-    part[r][c] = s;
-    __syncthreads();
-    if (r == 0 && n < N) {
-#pragma unroll
-        for (int q = 1; q < kSumRows; ++q) s += part[q][c];
-        db[n] = s;
-    }
 }
 
 __global__ void f32_to_bf16_kernel(const float *x, long long n, uint16_t *y) {
@@ -448,7 +481,8 @@ extern "C" int mdx_mlp_forward(const mdx_mlp *net, int batch, const uint16_t *x,
             g.epi = EPI_BIAS | EPI_RELU | EPI_BF16;
             in = out;
         }
-        if (gemm(g, s) != cudaSuccess) return set_last_error(MDX_ERR_CUDA, "mlp forward launch failed");
+        if (layer(&g, nullptr, nullptr, 0, 0, nullptr, s) != cudaSuccess)
+            return set_last_error(MDX_ERR_CUDA, "mlp forward launch failed");
     }
     return MDX_OK;
 }
@@ -493,11 +527,9 @@ extern "C" int mdx_mlp_backward(const mdx_mlp *net, int batch, const uint16_t *x
         g.C = dW[l];
         g.ldc = K;
         g.epi = EPI_NONE;
-        if (gemm(g, s) != cudaSuccess) return set_last_error(MDX_ERR_CUDA, "mlp backward launch failed");
-        col_sum_kernel<<<(N + 31) / 32, 32 * kSumRows, 0, s>>>(dz, batch, N, db[l]);
+        // dz_prev[m][k] = (sum_n dz[m][n] W[n][k]) * [act_l[m][k] > 0], BF16
+        GemmArgs h{};
         if (l > 0) {
-            // dz_prev[m][k] = (sum_n dz[m][n] W[n][k]) * [act_l[m][k] > 0], BF16
-            GemmArgs h{};
             h.M = batch;
             h.N = K;
             h.K = N;
@@ -512,11 +544,13 @@ extern "C" int mdx_mlp_backward(const mdx_mlp *net, int batch, const uint16_t *x
             h.mask = in;
             h.ldm = K;
             h.epi = EPI_MASK | EPI_BF16;
-            if (gemm(h, s) != cudaSuccess) return set_last_error(MDX_ERR_CUDA, "mlp backward launch failed");
-            uint16_t *t = dz;
-            dz = dz_next;
-            dz_next = t;
         }
+        // dW, dz_prev and db of a layer need only dz: one launch
+        if (layer(&g, l > 0 ? &h : nullptr, dz, batch, N, db[l], s) != cudaSuccess)
+            return set_last_error(MDX_ERR_CUDA, "mlp backward launch failed");
+        uint16_t *t = dz;
+        dz = dz_next;
+        dz_next = t;
     }
     if (cudaGetLastError() != cudaSuccess) return set_last_error(MDX_ERR_CUDA, "mlp backward launch failed");
     return MDX_OK;
