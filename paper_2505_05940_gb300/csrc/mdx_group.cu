@@ -319,19 +319,28 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                         }
                         float4 *x = reinterpret_cast<float4 *>(ring + (size_t)slot * (kGrpStageBytes / 4));
                         float4 *y = reinterpret_cast<float4 *>(lo + (size_t)slot * (kGrpStageBytes / 4));
-                        for (int i = ct; i < n4; i += 64) {
-                            const float4 v = x[i];
+                        // the thread's share of the stage (eight float4 at most) is
+                        // loaded before the first store: one load, store pair after
+                        // the other made this conversion the pipeline's slowest stage
+                        constexpr int kV = kGrpStageBytes / 16 / 64;
+                        float4 v[kV];
+#pragma unroll
+                        for (int q = 0; q < kV; ++q)
+                            if (ct + 64 * q < n4) v[q] = x[ct + 64 * q];
+#pragma unroll
+                        for (int q = 0; q < kV; ++q) {
+                            if (ct + 64 * q >= n4) continue;
                             float4 h, l;
-                            h.x = tf32_hi(v.x);
-                            h.y = tf32_hi(v.y);
-                            h.z = tf32_hi(v.z);
-                            h.w = tf32_hi(v.w);
-                            l.x = v.x - h.x;
-                            l.y = v.y - h.y;
-                            l.z = v.z - h.z;
-                            l.w = v.w - h.w;
-                            x[i] = h;
-                            y[i] = l;
+                            h.x = tf32_hi(v[q].x);
+                            h.y = tf32_hi(v[q].y);
+                            h.z = tf32_hi(v[q].z);
+                            h.w = tf32_hi(v[q].w);
+                            l.x = v[q].x - h.x;
+                            l.y = v[q].y - h.y;
+                            l.z = v[q].z - h.z;
+                            l.w = v[q].w - h.w;
+                            x[ct + 64 * q] = h;
+                            y[ct + 64 * q] = l;
                         }
                         fence_async_smem();
                         __syncwarp();
