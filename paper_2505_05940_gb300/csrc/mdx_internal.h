@@ -245,7 +245,9 @@ struct ResCta {
     int base;                         // cluster rank of this plate's rank 0
     int L;                            // padded row length (floats, multiple of 8)
     int k0, nk;                       // stress modes k0 .. k0 + nk - 1, one per warp
-    int pad;
+    int seg_last;                     // bit w: warp w's mode ends a part of the force
+    int seg0, segs_all;               // this CTA's first part, parts of the plate
+    unsigned long long new_item;      // bit g: part g starts a new partial sum
 };
 
 struct ResidentParams {
@@ -254,10 +256,11 @@ struct ResidentParams {
     const ClusterK *kinfo;            // [total_k] (class layout)
     const int *iperm;                 // inverse class permutation, at each plate's perm_off
     int variant;                      // kernel variant
+    bool same;                        // the streaming kernel's order of every sum
     int warps;                        // warps with a stress mode or a share of the update
     int L;                            // longest padded row
-    int n_max, no_max;                // most modes of a plate, most modes owned by a CTA
-    int max_sub;
+    int no_max;                       // most modes owned by a CTA
+    int max_sub, segs;                // most CTAs and parts of a plate
     int tcols;                        // tensor-memory columns per CTA
 };
 

@@ -146,11 +146,15 @@ struct mdx_plan {
     GroupPlan *grp = nullptr;
     std::vector<int> grouped;      // per instance
     bool any_grouped = false;
-    // resident plates: the coupling tensors held on the SMs (mdx_resident.cu)
-    bool res_ok = false;
-    int res_cs = 1, res_grid = 0;
-    ResidentParams res{};            // launch shape and tables (p unset)
-    size_t res_smem[4] = {0, 0, 0, 0};   // by right-hand sides
+    // resident plates: the coupling tensors held on the SMs (mdx_resident.cu), with
+    // the streaming kernel's order of every sum (any pass) and with the order
+    // that is fastest (forward passes without checkpoints)
+    struct Resident {
+        bool ok = false;
+        int cs = 1, grid = 0;
+        ResidentParams q{};                  // launch shape and tables (p unset)
+        size_t smem[4] = {0, 0, 0, 0};       // by right-hand sides
+    } res_same, res_fast;
     bool fused_sweep = false;        // mdx_grad fuses reverse and recompute
 };
 
@@ -250,11 +254,10 @@ struct Piece {
     double cost;
 };
 
-// Chooses how many CTAs share each plate and lays the resident launch out
-// (plan.res_ok stays false when a plate does not fit).
+// Chooses how many CTAs share each plate and lays the resident launches out
+// (plan.res_same, plan.res_fast stay unset where a plate does not fit).
 int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
-                  const std::vector<PlateItem> &items, const std::vector<int> &perm_all,
-                  int smem_optin);
+                  const std::vector<PlateItem> &items, int smem_optin);
 int configure_tiles(mdx_plan *p, int stage_req, int ring_req);
 void update_l2_keep(mdx_plan *p);
 
@@ -875,13 +878,6 @@ int mdx_plan_create(mdx_plan **out, const mdx_instance *I, int n_inst, const mdx
             if ((rc2 = upload(p, &p->d_perm, perm_all.data(), perm_all.size()))) return bail(rc2);
             if ((rc2 = upload(p, &p->d_kperm, kperm_all.data(), kperm_all.size()))) return bail(rc2);
             if ((rc2 = upload(p, &p->d_chunks, chunks.data(), chunks.size()))) return bail(rc2);
-            // resident plates, not for plans whose options shape the streaming
-            // kernel's work split (tests of it)
-            if (o.force_split <= 0 && o.max_ctas <= 0 && !(p->debug_flags & (1 | 16))) {
-                const int rcr = plan_resident(p, chunks, items, perm_all, smem_optin);
-                if (rcr) return bail(rcr);
-            }
-            p->fused_sweep = p->fuse || (p->res_ok && !(p->debug_flags & 2));
             // contraction units: plates with a direction tensor (direction
             // derivative), and every plate (full dL/dH output)
             auto build_units = [&](bool all, std::vector<DirUnit> &units,
@@ -1005,6 +1001,13 @@ int mdx_plan_create(mdx_plan **out, const mdx_instance *I, int n_inst, const mdx
             const int rcc = configure_tiles(p, o.stage_bytes, o.ring_stages);
             if (rcc) return bail(rcc);
         }
+        // resident plates, not for plans whose options shape the streaming
+        // kernel's work split (tests of it)
+        if (o.force_split <= 0 && o.max_ctas <= 0 && !(p->debug_flags & (1 | 16))) {
+            const int rcr = plan_resident(p, chunks, items, smem_optin);
+            if (rcr) return bail(rcr);
+        }
+        p->fused_sweep = p->fuse || (p->res_same.ok && !(p->debug_flags & 2));
         update_l2_keep(p);
         int rc;
         if ((rc = upload(p, &p->d_items, items.data(), items.size()))) return bail(rc);
@@ -1168,77 +1171,122 @@ TensionParams base_tension(mdx_plan *p, int mode, int steps, int n_begin, int to
     return T;
 }
 
-// Step time of one CTA in SM cycles: a fixed chain (barriers, reductions,
-// update; with peers also the two exchanges) and the packed FMAs of one stress
-// mode per warp (L / 8 rows of L columns a lane) over four schedulers.
-double res_step_cycles(int nk, int L, int sub) {
-    return 700.0 + (sub > 1 ? 800.0 + 10.0 * sub : 0.0) + 0.15 * L * L * ((nk + 3) / 4);
+// Step time of a CTA with nk stress modes and rows of L columns, in SM cycles:
+// the dependent chain (with peers two exchanges; the products of a warp, one
+// scheduler's warps after each other), and what the CTA takes of its SM's FMA
+// and shared-memory throughput, which counts when CTAs share the SM.
+double res_chain_cycles(int nk, int L, int sub) {
+    return 1100.0 + (sub > 1 ? 1000.0 + 30.0 * sub : 0.0) + 0.3 * L * L * ((nk + 3) / 4);
 }
+double res_load_cycles(int nk, int L) { return 0.1 * L * L * nk; }
 
-int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
-                  const std::vector<PlateItem> &items, const std::vector<int> &perm_all,
-                  int smem_optin) {
-    struct Pl {
-        int inst, N, M, L;
-    };
-    std::vector<Pl> pls;
-    int variant = 0;
-    for (int i = 0; i < p->n_inst; ++i) {
-        const InstDesc &d = p->inst[i];
-        if (d.kind != MDX_KIND_PLATE || d.M == 0 || d.grouped) continue;
-        const int w = d.parity ? *std::max_element(d.ncls, d.ncls + 4) : d.N;
-        const int v = resident_variant(w, d.parity ? (w + 7) / 8 : (d.N + 31) / 32);
-        if (v < 0 || d.N > kResMaxModes) return MDX_OK;
-        variant = std::max(variant, v);
-        pls.push_back({i, d.N, d.M, (w + 7) & ~7});
-    }
-    if (pls.empty()) return MDX_OK;
-    const int wmax = resident_max_warps(variant);
-    auto nk_of = [](const Pl &q, int sub) { return (q.M + sub - 1) / sub; };
+// A plate of the resident launch, and one way to share it: the stress modes of
+// its CTAs are [kb[r], kb[r + 1]).
+struct ResPlate {
+    int inst, N, M, L;
+    std::vector<int> runs;       // lengths of the runs of stress modes summed in one row
+    unsigned long long new_item = 0;
+};
+struct ResShare {
+    int sub, nk, warps;          // CTAs, most stress modes of one, its warps
+    std::vector<int> kb;
+};
+
+// One resident launch: `same` keeps the runs of the streaming kernel's sums.
+int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, bool same,
+                   const ClusterK *kinfo, const int *iperm, int smem_optin, mdx_plan::Resident *out) {
+    int sms = 0;
+    MDX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device), "attr");
     // warps of a CTA: one per stress mode and, while there is room, others for the
     // owned modes (32 a warp); enough for two modes of the plate a thread
-    auto warps_of = [&](const Pl &q, int sub) {
-        const int own = ((q.N + sub - 1) / sub + 31) / 32, nk = nk_of(q, sub);
-        return std::max({nk, own, (q.N + 63) / 64, std::min(nk + own, wmax)});
+    auto warps_of = [&](const ResPlate &q, const ResShare &s, int wmax) {
+        const int own = ((q.N + s.sub - 1) / s.sub + 31) / 32;
+        return std::max({s.nk, own, (q.N + 63) / 64, std::min(s.nk + own, wmax)});
     };
-    auto ok = [&](const Pl &q, int sub) { return sub <= q.M && warps_of(q, sub) <= wmax; };
-    auto cycles = [&](const Pl &q, int sub) { return res_step_cycles(nk_of(q, sub), q.L, sub); };
-    auto shape = [&](const std::vector<int> &sub) {
+    auto shares = [&](const ResPlate &q, int wmax, int csmax) {
+        std::vector<ResShare> v;
+        auto add = [&](ResShare s) {
+            s.nk = 0;
+            for (int r = 0; r < s.sub; ++r) s.nk = std::max(s.nk, s.kb[r + 1] - s.kb[r]);
+            s.warps = warps_of(q, s, wmax);
+            if (s.sub <= csmax && s.warps <= wmax &&
+                (v.empty() || v.back().sub != s.sub))
+                v.push_back(s);
+        };
+        if (same) {
+            // whole runs only, from many CTAs to few, then reversed
+            for (int cap = 1; cap <= wmax; ++cap) {
+                ResShare s{0, 0, 0, {0}};
+                int k = 0, n = 0;
+                bool fits = true;
+                for (int len : q.runs) {
+                    fits = fits && len <= cap;
+                    if (n + len > cap) {
+                        s.kb.push_back(k);
+                        n = 0;
+                    }
+                    n += len;
+                    k += len;
+                }
+                s.kb.push_back(k);
+                s.sub = (int)s.kb.size() - 1;
+                if (fits) add(s);
+            }
+            std::reverse(v.begin(), v.end());
+        } else {
+            for (int sub : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
+                if (sub > q.M) break;
+                ResShare s{sub, 0, 0, {}};
+                for (int r = 0; r <= sub; ++r) s.kb.push_back((int)((long long)q.M * r / sub));
+                add(s);
+            }
+        }
+        return v;
+    };
+    // (150: no warp without a stress mode is left for the pickups)
+    auto cycles = [&](const ResPlate &q, const ResShare &s) {
+        return res_chain_cycles(s.nk, q.L, s.sub) + (s.nk < s.warps ? 0.0 : 150.0);
+    };
+    auto shape = [&](const std::vector<ResShare> &sh) {
         ResidentParams Q{};
         Q.variant = variant;
+        Q.same = same;
         for (size_t i = 0; i < pls.size(); ++i) {
             Q.L = std::max(Q.L, pls[i].L);
-            Q.warps = std::max(Q.warps, warps_of(pls[i], sub[i]));
-            Q.n_max = std::max(Q.n_max, pls[i].N);
-            Q.no_max = std::max(Q.no_max, (pls[i].N + sub[i] - 1) / sub[i]);
-            Q.max_sub = std::max(Q.max_sub, sub[i]);
+            Q.warps = std::max(Q.warps, sh[i].warps);
+            Q.no_max = std::max(Q.no_max, (pls[i].N + sh[i].sub - 1) / sh[i].sub);
+            Q.max_sub = std::max(Q.max_sub, sh[i].sub);
+            Q.segs = std::max(Q.segs, same ? (int)pls[i].runs.size() : sh[i].sub);
         }
         Q.tcols = resident_columns(variant, Q.L, Q.warps);
         return Q;
     };
-    // clusters: plates sorted by (CTAs, time), cs / sub of them per cluster,
-    // longest clusters first (the hardware starts them in order)
-    auto pack = [&](const std::vector<int> &sub, int cs, std::vector<std::vector<int>> &cl,
+    // clusters: plates sorted by (CTAs, time), as many per cluster as fit, longest
+    // clusters first (the hardware starts them in order); ct: their step times
+    // when `share` CTAs use an SM
+    auto pack = [&](const std::vector<ResShare> &sh, int cs, int fit, std::vector<std::vector<int>> &cl,
                     std::vector<double> &ct) {
         std::vector<int> ord(pls.size());
         std::iota(ord.begin(), ord.end(), 0);
         std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) {
-            if (sub[a] != sub[b]) return sub[a] > sub[b];
-            return cycles(pls[a], sub[a]) > cycles(pls[b], sub[b]);
+            if (sh[a].sub != sh[b].sub) return sh[a].sub > sh[b].sub;
+            return cycles(pls[a], sh[a]) > cycles(pls[b], sh[b]);
         });
         std::vector<std::vector<int>> c0;
-        std::vector<double> t0;
         int room = 0;
         for (int i : ord) {
-            if (room < sub[i]) {
+            if (room < sh[i].sub) {
                 c0.push_back({});
-                t0.push_back(0.0);
                 room = cs;
             }
             c0.back().push_back(i);
-            t0.back() = std::max(t0.back(), cycles(pls[i], sub[i]));
-            room -= sub[i];
+            room -= sh[i].sub;
         }
+        const double share = std::max(1.0, (double)std::min<size_t>((size_t)fit, c0.size()) * cs / sms);
+        std::vector<double> t0(c0.size(), 0.0);
+        for (size_t c = 0; c < c0.size(); ++c)
+            for (int i : c0[c])
+                t0[c] = std::max({t0[c], cycles(pls[i], sh[i]), share * res_load_cycles(sh[i].nk, pls[i].L)});
         std::vector<int> co(c0.size());
         std::iota(co.begin(), co.end(), 0);
         std::stable_sort(co.begin(), co.end(), [&](int a, int b) { return t0[a] > t0[b]; });
@@ -1250,93 +1298,103 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
         }
     };
     // For each bound of the step time every plate takes the fewest CTAs that meet
-    // it; the makespan of the clusters, in launch order, decides between the bounds.
+    // it; the makespan of the clusters, in launch order, decides between the
+    // bounds.  CTAs of at most four warps share an SM (their tensor memory is half
+    // of it) and overlap each other's chains; eight warps hold a plate in fewer.
     double best = 1e300;
-    int best_cs = 0;
-    std::vector<int> best_sub;
+    int best_cs = 0, best_fit = 1;
+    std::vector<ResShare> best_sh;
     ResidentParams best_q{};
-    constexpr int kSubs[] = {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16};
-    for (int csmax : {8, 16}) {
-        std::vector<double> taus;
-        bool all = true;
-        for (const Pl &q : pls) {
-            bool any = false;
-            for (int s : kSubs)
-                if (s <= csmax && ok(q, s)) {
-                    any = true;
-                    taus.push_back(cycles(q, s));
-                }
-            all = all && any;
-        }
-        if (!all) continue;
-        std::sort(taus.begin(), taus.end());
-        taus.erase(std::unique(taus.begin(), taus.end()), taus.end());
-        std::vector<int> prev;
-        for (int j = 0; j < 24; ++j) {   // at most 24 bounds, spread over the sorted list
-            const double tau = taus[(taus.size() - 1) * j / 23];
-            std::vector<int> sub(pls.size());
-            int cs = 1;
-            for (size_t i = 0; i < pls.size(); ++i) {
-                int s0 = 0;
-                double t0 = 1e300;
-                for (int s : kSubs) {
-                    if (s > csmax || !ok(pls[i], s)) continue;
-                    const double t = cycles(pls[i], s);
-                    if (t < t0) {
-                        t0 = t;
-                        s0 = s;
+    for (int wmax : {4, resident_max_warps(variant)})
+        for (int csmax : {8, 16}) {
+            std::vector<std::vector<ResShare>> cand;
+            std::vector<double> taus;
+            bool all = true;
+            for (const ResPlate &q : pls) {
+                cand.push_back(shares(q, wmax, csmax));
+                for (const ResShare &s : cand.back()) taus.push_back(cycles(q, s));
+                all = all && !cand.back().empty();
+            }
+            if (!all) continue;
+            std::sort(taus.begin(), taus.end());
+            taus.erase(std::unique(taus.begin(), taus.end()), taus.end());
+            std::vector<int> prev;
+            for (int j = 0; j < 24; ++j) {   // at most 24 bounds, spread over the sorted list
+                const double tau = taus[(taus.size() - 1) * j / 23];
+                std::vector<ResShare> sh;
+                std::vector<int> subs;
+                int cs = 1;
+                for (size_t i = 0; i < pls.size(); ++i) {
+                    const ResShare *pick = nullptr;
+                    for (const ResShare &s : cand[i]) {
+                        if (!pick || cycles(pls[i], s) < cycles(pls[i], *pick)) pick = &s;
+                        if (cycles(pls[i], s) <= tau) break;
                     }
-                    if (t <= tau) break;
+                    sh.push_back(*pick);
+                    subs.push_back(pick->sub);
+                    cs = std::max(cs, pick->sub);
                 }
-                sub[i] = s0;
-                cs = std::max(cs, s0);
-            }
-            if (sub == prev) continue;
-            prev = sub;
-            const ResidentParams Q = shape(sub);
-            int fit = 0;
-            if (resident_check(cs, Q, (size_t)smem_optin, &fit) != cudaSuccess) {
-                cudaGetLastError();
-                continue;
-            }
-            if (fit < 1) continue;
-            std::vector<std::vector<int>> cl;
-            std::vector<double> ct;
-            pack(sub, cs, cl, ct);
-            std::vector<double> m(std::min<size_t>((size_t)fit, cl.size()), 0.0);
-            for (double t : ct) *std::min_element(m.begin(), m.end()) += t;
-            const double span = *std::max_element(m.begin(), m.end());
-            if (span < 0.98 * best) {
-                best = span;
-                best_cs = cs;
-                best_sub = sub;
-                best_q = Q;
+                if (subs == prev) continue;
+                prev = subs;
+                const ResidentParams Q = shape(sh);
+                int fit = 0;
+                if (resident_check(cs, Q, (size_t)smem_optin, &fit) != cudaSuccess) {
+                    cudaGetLastError();
+                    continue;
+                }
+                if (fit < 1) continue;
+                std::vector<std::vector<int>> cl;
+                std::vector<double> ct;
+                pack(sh, cs, fit, cl, ct);
+                std::vector<double> m(std::min<size_t>((size_t)fit, cl.size()), 0.0);
+                for (double t : ct) *std::min_element(m.begin(), m.end()) += t;
+                const double span = *std::max_element(m.begin(), m.end());
+                if (span < 0.98 * best) {
+                    best = span;
+                    best_cs = cs;
+                    best_fit = fit;
+                    best_sh = sh;
+                    best_q = Q;
+                }
             }
         }
-    }
     if (best_cs == 0) return MDX_OK;
     // ---- tables
     std::vector<std::vector<int>> cl;
     std::vector<double> ct;
-    pack(best_sub, best_cs, cl, ct);
+    pack(best_sh, best_cs, best_fit, cl, ct);
     std::vector<ResCta> ctas;
     for (const auto &c : cl) {
         int base = 0;
         for (int i : c) {
-            const Pl &q = pls[i];
-            const int sub = best_sub[i];
-            for (int r = 0; r < sub; ++r) {
+            const ResPlate &q = pls[i];
+            const ResShare &s = best_sh[i];
+            std::vector<char> last(q.M, 0);      // the stress mode ends a run
+            if (same)
+                for (int k = -1, r = 0; r < (int)q.runs.size(); ++r) last[k += q.runs[r]] = 1;
+            else
+                for (int r = 0; r < s.sub; ++r) last[s.kb[r + 1] - 1] = 1;
+            int seg = 0;
+            for (int r = 0; r < s.sub; ++r) {
                 ResCta A{};
                 A.plate = q.inst;
                 A.rank = r;
-                A.sub = sub;
+                A.sub = s.sub;
                 A.base = base;
                 A.L = q.L;
-                A.k0 = (int)((long long)q.M * r / sub);
-                A.nk = (int)((long long)q.M * (r + 1) / sub) - A.k0;
+                A.k0 = s.kb[r];
+                A.nk = s.kb[r + 1] - s.kb[r];
+                A.seg0 = seg;
+                A.new_item = same ? q.new_item : 0ull;
+                A.segs_all = same ? (int)q.runs.size() : s.sub;
+                for (int w = 0; w < A.nk; ++w)
+                    if (last[A.k0 + w]) {
+                        A.seg_last |= 1 << w;
+                        ++seg;
+                    }
                 ctas.push_back(A);
             }
-            base += sub;
+            base += s.sub;
         }
         for (; base < best_cs; ++base) {
             ResCta A{};
@@ -1344,6 +1402,74 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
             ctas.push_back(A);
         }
     }
+    ResCta *dc = nullptr;
+    int rc;
+    if ((rc = upload(p, &dc, ctas.data(), ctas.size()))) return rc;
+    out->q = best_q;
+    out->q.ctas = dc;
+    out->q.kinfo = kinfo;
+    out->q.iperm = iperm;
+    out->cs = best_cs;
+    out->grid = (int)ctas.size();
+    for (int r = 1; r <= (same ? 3 : 1); ++r) out->smem[r] = resident_smem(r, best_q);
+    out->ok = true;
+    return MDX_OK;
+}
+
+int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
+                  const std::vector<PlateItem> &items, int smem_optin) {
+    std::vector<ResPlate> pls;
+    int variant = 0;
+    bool same = true;
+    std::vector<std::vector<const PlateItem *>> its(p->n_inst);
+    for (const auto &it : items) its[it.inst].push_back(&it);
+    for (int i = 0; i < p->n_inst; ++i) {
+        const InstDesc &d = p->inst[i];
+        if (d.kind != MDX_KIND_PLATE || d.M == 0 || d.grouped) continue;
+        const int w = d.parity ? *std::max_element(d.ncls, d.ncls + 4) : d.N;
+        const int v = resident_variant(w, d.parity ? (w + 7) / 8 : (d.N + 31) / 32);
+        if (v < 0 || d.N > kResMaxModes) return MDX_OK;
+        variant = std::max(variant, v);
+        ResPlate q;
+        q.inst = i;
+        q.N = d.N;
+        q.M = d.M;
+        q.L = (w + 7) & ~7;
+        // The streaming kernel's sums of this plate: per item (in contributor order)
+        // a row of FMAs over each class chunk, or over the whole item without
+        // classes.  Gradients depend on them in their last digits, so passes with
+        // checkpoints keep them: the resident kernel takes such a plan when its
+        // runs fit the CTAs and the rows' even / odd chains do not change sides
+        // within a chunk (a stage of an odd number of rows before the last).
+        std::vector<const PlateItem *> &list = its[i];
+        std::sort(list.begin(), list.end(), [](const PlateItem *a, const PlateItem *b) { return a->slot < b->slot; });
+        int k = 0;
+        for (const PlateItem *it : list) {
+            if (it->k0 != k) same = false;       // contributors out of order
+            k = it->k1;
+            if (!q.runs.empty()) {
+                if (q.runs.size() < 64) q.new_item |= 1ull << q.runs.size();
+            }
+            if (!d.parity) {
+                q.runs.push_back(it->k1 - it->k0);
+                same = same && d.N <= 32;
+                continue;
+            }
+            for (int ci = it->chunk0; ci < it->chunk1; ++ci) {
+                const ParityChunk &ch = chunks[ci];
+                q.runs.push_back(ch.mc);
+                for (int a = 0; a < 4; ++a) {
+                    const int na = d.ncls[a], nb = d.ncls[a ^ ch.c];
+                    if (na == 0 || nb == 0) continue;
+                    const int rps = std::max(1, p->stage_bytes / 4 / (ch.mc * ((nb + 3) & ~3)));
+                    if (rps < na && (rps & 1)) same = false;
+                }
+            }
+        }
+        if (k != d.M || q.runs.size() > 64) same = false;
+        pls.push_back(q);
+    }
+    if (pls.empty()) return MDX_OK;
     std::vector<ClusterK> kinfo(std::max<long long>(p->total_k, 1));
     for (const auto &it : items)
         for (int ci = it.chunk0; p->parity && ci < it.chunk1; ++ci)
@@ -1354,30 +1480,24 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
                 K.kpos = q;
                 K.c = chunks[ci].c;
             }
-    std::vector<int> iperm(std::max<size_t>(perm_all.size(), 1), 0);
-    for (const Pl &q : pls) {
-        const InstDesc &d = p->inst[q.inst];
-        for (int c = 0; d.parity && c < d.N; ++c) iperm[d.perm_off + perm_all[d.perm_off + c]] = c;
+    std::vector<int> iperm;
+    for (int i = 0; i < p->n_inst; ++i) {
+        const InstDesc &d = p->inst[i];
+        if (!d.parity) continue;
+        iperm.resize(std::max<size_t>(iperm.size(), (size_t)(d.perm_off + d.N)), 0);
+        for (int c = 0; c < d.N; ++c) iperm[d.perm_off + p->h_perm[i][c]] = c;
     }
-    ResCta *dc = nullptr;
+    iperm.resize(std::max<size_t>(iperm.size(), 1), 0);
     ClusterK *dk = nullptr;
     int *di = nullptr, rc;
-    if ((rc = upload(p, &dc, ctas.data(), ctas.size()))) return rc;
     if ((rc = upload(p, &dk, kinfo.data(), kinfo.size()))) return rc;
     if ((rc = upload(p, &di, iperm.data(), iperm.size()))) return rc;
-    p->res = best_q;
-    p->res.ctas = dc;
-    p->res.kinfo = dk;
-    p->res.iperm = di;
-    p->res_cs = best_cs;
-    p->res_grid = (int)ctas.size();
-    for (int r = 1; r <= 3; ++r) p->res_smem[r] = resident_smem(r, best_q);
-    p->res_ok = true;
-    return MDX_OK;
+    if (same && (rc = build_resident(p, pls, variant, true, dk, di, smem_optin, &p->res_same))) return rc;
+    return build_resident(p, pls, variant, false, dk, di, smem_optin, &p->res_fast);
 }
 
-int run_resident(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
-    ResidentParams Q = p->res;
+int run_resident(mdx_plan *p, const mdx_plan::Resident &res, const PlateParams &P, cudaStream_t s) {
+    ResidentParams Q = res.q;
     Q.p = P;
     const int R = P.mode == MODE_FUSED ? 3 : (P.mode == MODE_REVERSE ? 2 : 1);
     mdx_plan::Rec rec{};
@@ -1388,8 +1508,7 @@ int run_resident(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
         MDX_CUDA(cudaEventCreate(&rec.b), "event");
         MDX_CUDA(cudaEventRecord(rec.a, s), "event");
     }
-    MDX_CUDA(launch_resident(R, Q, p->res_grid, p->res_cs, p->res_smem[R], s),
-             "resident plate kernel");
+    MDX_CUDA(launch_resident(R, Q, res.grid, res.cs, res.smem[R], s), "resident plate kernel");
     if (p->profiling) {
         MDX_CUDA(cudaEventRecord(rec.b, s), "event");
         p->recs.push_back(rec);
@@ -1399,7 +1518,8 @@ int run_resident(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
 
 int run_plate(mdx_plan *p, PlateParams &P, cudaStream_t s) {
     if (!p->any_plate) return MDX_OK;
-    if (p->res_ok) return run_resident(p, P, s);
+    if (P.mode == MODE_FORWARD && !P.ckpt && p->res_fast.ok) return run_resident(p, p->res_fast, P, s);
+    if (p->res_same.ok) return run_resident(p, p->res_same, P, s);
     MDX_CUDA(cudaMemsetAsync(p->d_counters, 0, p->n_inst * sizeof(unsigned), s), "memset");
     MDX_CUDA(cudaMemsetAsync(p->d_abort, 0, sizeof(int), s), "memset");
     const size_t smem = (P.mode == MODE_FUSED) ? p->smem_fused

@@ -38,8 +38,9 @@
 // network takes at 13 cycles per warp store: 730 cycles a step for 8 CTAs of
 // 200 modes (1 525 with three right-hand sides).
 //
-// A spare warp sums the pickups of eight steps at a time (forward and
-// recompute), off the step's chain.
+// Pickups: one warp per chunk of owned modes keeps its terms and sums them every
+// eight steps (with shuffles every step this was 320 cycles of the step's chain);
+// one warp of the last rank adds the chunks' terms.
 //
 // Bound: the packed FMAs (two warps a scheduler) plus the latency of the
 // dependent chain (one barrier, one warp reduction, two exchanges, the update).
@@ -59,8 +60,9 @@ using namespace tc;
 
 typedef unsigned long long u64;
 
-constexpr int kResMaxWarps = 7;              // row warps of a CTA (and the spare warp)
-constexpr int kPickSteps = 8;                // pickups reduced together by the spare warp
+constexpr int kResMaxWarps = 8;              // warps of a CTA
+constexpr int kPickSteps = 8;                // pickups reduced together
+constexpr int kPickPitch = 36;               // terms of a step: 4 lanes x 4 steps on distinct banks
 // Shared memory asked for per tensor-memory column: above 233 472 / 544, the SM's
 // shared memory over one allocation step more than its 512 columns, so any CTAs
 // that fit an SM by shared memory hold at most 512 columns together.
@@ -144,32 +146,37 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
 __host__ __device__ constexpr int rhs_blocks(int R) { return R == 1 ? 1 : R + 1; }
 
 // Shared-memory layout (float offsets from the dynamic base), the same on the
-// host.  W warps, kernel row length LM, N modes at most, NO owned modes at most.
+// host.  W warps, kernel row length LM, NO owned modes and segs parts at most.
 struct ResLayout {
-    int QB, PS;                 // strides: class block, pickup row
-    int rhs, fp, xch, hs, coef, pick, gacc, vst, end;
+    int QB, PS;                 // class block, pickup terms per step
+    int rhs, fp, ke, xch, hs, coef, pick, pst, gacc, vst, end;
 };
 
-__host__ __device__ inline ResLayout res_layout(int R, int W, int LM, int L, int N, int NO, int sub,
+__host__ __device__ inline ResLayout res_layout(int R, int W, int LM, int L, int NO, int sub, int segs,
                                                 int nsm) {
     ResLayout o;
     // class blocks 8 banks apart, so that the four classes' accesses do not collide
     o.QB = ((LM + 31) & ~31) + 8;
-    o.PS = ((2 * N + 31) & ~31) + 8;
+    o.PS = sub * ((NO + 31) / 32);
     int p = 16;                 // mbarriers, tensor-memory base
     o.rhs = p;                  // [blocks][4][QB]
-    p += rhs_blocks(R) * 4 * o.QB;
-    o.fp = p;                   // [W][R][4][QB] forces of each warp
+    p += rhs_blocks(R) * 4 * o.QB + 8;   // (a chunk is read past the last block)
+    o.fp = p;                   // [W][R][4][QB] products of each warp's stress mode
     p += W * R * 4 * o.QB;
-    o.xch = p;                  // [2][sub][NO] x (1, 2 or 4 floats): parts of the owned modes
-    if (sub > 1) p += 2 * sub * NO * (R == 3 ? 4 : R);
+    o.ke = p;                   // [W][8] its factors of the forces
+    p += W * 8;
+    o.xch = p;                  // [2][segs][NO] x (1, 2 or 4 floats): parts of the owned modes
+    if (sub > 1) p += 2 * segs * NO * (R == 3 ? 4 : R);
     p = (p + 3) & ~3;
     o.hs = p;                   // [nsm][L / 4][32 W] x 4: coupling rows (thread-private)
     p += nsm * L * 32 * W;
     o.coef = p;                 // [7][32 W] coefficients of the updated modes
     p += 7 * 32 * W;
-    o.pick = p;                 // [2][kPickSteps][PS] pickup terms
-    if (R == 1) p += 2 * kPickSteps * o.PS;
+    p = (p + 1) & ~1;
+    o.pick = p;                 // [2][kPickSteps][PS] x 2: pickup terms of the owners' chunks
+    if (R == 1) p += 2 * kPickSteps * 2 * o.PS;
+    o.pst = p;                  // [chunks][kPickSteps][kPickPitch] x 2: a chunk's terms of its modes
+    if (R == 1) p += (NO + 31) / 32 * kPickSteps * kPickPitch * 2;
     o.gacc = p;                 // [GA_N][2][32 W] gradient sums
     if (R >= 2) p += GA_N * 2 * 32 * W;
     o.vst = p;                  // [32 W] v^n of the next step
@@ -190,22 +197,23 @@ __device__ __forceinline__ void bar_sync_id(int id, int n) {
     __syncwarp();
     asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
-__device__ __forceinline__ void bar_arrive_id(int id, int n) {
-    __syncwarp();
-    asm volatile("barrier.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
 // One warp's products u[r][x] = sum_j H[r][j] q_x[j] over NTM tensor-memory
 // rows ([column / 8][row][8], read two rows at a time, the next pair in flight
-// during this pair's FMAs) and NSM shared-memory rows.  The loop over the
-// columns stays rolled: unrolled with rows in registers the step's code, run
-// once per step by a few warps, was bound by instruction fetch and spills.
-template <int R, int NTM, int NSM>
+// during this pair's FMAs), NSM shared-memory rows and NREG register rows.  A
+// chunk's shared-memory rows are loaded before and multiplied after its
+// tensor-memory rows, so the two warps of a scheduler do not alternate between
+// loading and multiplying.  Without register rows the loop over the columns
+// stays rolled.  SP chains per row (two where few rows leave the FMAs' latency
+// uncovered).
+template <int R, int NTM, int NSM, int NREG, int LMAX, int SP>
 __device__ __forceinline__ void row_products(const float4 *hs, int hs_stride, uint32_t taddr, int L,
-                                             const float *const (&q)[R], float (&u)[NTM + NSM][R]) {
-    constexpr int NA = NTM + NSM, NP = NTM / 2, UN = (NP & 1) ? 2 : 1;
-    // few rows: two chains per row, the FMAs' latency is what bounds them
-    constexpr int SP = NA <= 4 ? 2 : 1;
+                                             const u64 (&hr)[NREG > 0 ? NREG : 1][LMAX / 2],
+                                             const float *const (&q)[R], float (&u)[NTM + NSM + NREG][R]) {
+    constexpr int NA = NTM + NSM + NREG, NP = NTM / 2;
+    // all rows in tensor memory: the next right-hand sides are loaded during the
+    // FMAs (1.40 instead of 1.44 us a step at 100 x 30); not worth its registers
+    // where other rows' loads cover theirs (4.15 / 3.93 us at 96 plates)
+    constexpr bool PF = NA == NTM;
     static_assert(NTM > 0 && NTM % 2 == 0, "tensor-memory rows are read in pairs");
     u64 acc[NA][R][SP];
 #pragma unroll
@@ -217,54 +225,72 @@ __device__ __forceinline__ void row_products(const float4 *hs, int hs_stride, ui
     uint32_t tm[2][16];
     tmem_ld_rows2(taddr, tm[0]);
     const int row4 = (L / 4) * hs_stride;
+    ulonglong2 qv[2][R][2];
+    auto load_q = [&](int j, ulonglong2 (&d)[R][2]) {
+#pragma unroll
+        for (int x = 0; x < R; ++x) {
+            d[x][0] = *reinterpret_cast<const ulonglong2 *>(q[x] + j);
+            d[x][1] = *reinterpret_cast<const ulonglong2 *>(q[x] + j + 4);
+        }
+    };
+    auto mac = [&](u64 (&a)[SP], u64 h0, u64 h1, u64 h2, u64 h3, const ulonglong2 (&v)[2]) {
+        a[0] = ffma2(h0, v[0].x, a[0]);
+        a[SP - 1] = ffma2(h1, v[0].y, a[SP - 1]);
+        a[0] = ffma2(h2, v[1].x, a[0]);
+        a[SP - 1] = ffma2(h3, v[1].y, a[SP - 1]);
+    };
+    // columns j .. j + 7; h: parity of j / 8
+    auto chunk = [&](int j, int h) {
+        const float4 *hp = hs + (j / 4) * hs_stride;
+        ulonglong2 ha[NSM > 0 ? NSM : 1], hb[NSM > 0 ? NSM : 1];
+        if constexpr (!PF) load_q(j, qv[h]);
+#pragma unroll
+        for (int s = 0; s < NSM; ++s) {
+            ha[s] = *reinterpret_cast<const ulonglong2 *>(hp + s * row4);
+            hb[s] = *reinterpret_cast<const ulonglong2 *>(hp + s * row4 + hs_stride);
+        }
+        // (beyond the last chunk the padding of the block is read)
+        if constexpr (PF) load_q(j + 8, qv[h ^ 1]);
+#pragma unroll
+        for (int g = 0; g < NP; ++g) {
+            const int par = (h * NP + g) & 1;
+            uint32_t (&w)[16] = tm[par];
+            tmem_wait_ld(w);
+            // beyond the last chunk the first pair is read again and not used
+            const bool more = g + 1 < NP || j + 8 < L;
+            tmem_ld_rows2(taddr + (uint32_t)(more ? j * NTM + 16 * (g + 1) : 0), tm[par ^ 1]);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+#pragma unroll
+                for (int x = 0; x < R; ++x)
+                    mac(acc[2 * g + s][x], pack2(w[8 * s], w[8 * s + 1]), pack2(w[8 * s + 2], w[8 * s + 3]),
+                        pack2(w[8 * s + 4], w[8 * s + 5]), pack2(w[8 * s + 6], w[8 * s + 7]), qv[h][x]);
+        }
+#pragma unroll
+        for (int s = 0; s < NSM; ++s)
+#pragma unroll
+            for (int x = 0; x < R; ++x)
+                mac(acc[NTM + s][x], ha[s].x, ha[s].y, hb[s].x, hb[s].y, qv[h][x]);
+    };
+    if constexpr (PF) load_q(0, qv[0]);
+    if constexpr (NREG > 0) {
+#pragma unroll
+        for (int j = 0; j < LMAX; j += 8) {
+            if (j >= L) break;
+            chunk(j, (j / 8) & 1);
+#pragma unroll
+            for (int s = 0; s < NREG; ++s)
+#pragma unroll
+                for (int x = 0; x < R; ++x)
+                    mac(acc[NTM + NSM + s][x], hr[s][j / 2], hr[s][j / 2 + 1], hr[s][j / 2 + 2], hr[s][j / 2 + 3],
+                        qv[(j / 8) & 1][x]);
+        }
+    } else {
 #pragma unroll 1
-    for (int j0 = 0; j0 < L; j0 += 8 * UN) {
-#pragma unroll
-        for (int h = 0; h < UN; ++h) {
-            const int j = j0 + 8 * h;
-            if (UN > 1 && j >= L) break;
-            ulonglong2 qa[R], qb[R];
-#pragma unroll
-            for (int x = 0; x < R; ++x) {
-                qa[x] = *reinterpret_cast<const ulonglong2 *>(q[x] + j);
-                qb[x] = *reinterpret_cast<const ulonglong2 *>(q[x] + j + 4);
-            }
-            const float4 *hp = hs + (j / 4) * hs_stride;
-            ulonglong2 ha[NSM > 0 ? NSM : 1], hb[NSM > 0 ? NSM : 1];
-#pragma unroll
-            for (int s = 0; s < NSM; ++s) {
-                ha[s] = *reinterpret_cast<const ulonglong2 *>(hp + s * row4);
-                hb[s] = *reinterpret_cast<const ulonglong2 *>(hp + s * row4 + hs_stride);
-            }
-#pragma unroll
-            for (int g = 0; g < NP; ++g) {
-                const int par = (h * NP + g) & 1;
-                uint32_t (&w)[16] = tm[par];
-                tmem_wait_ld(w);
-                // beyond the last chunk the pair is read again and not used
-                const bool more = g + 1 < NP || j + 8 < L;
-                tmem_ld_rows2(taddr + (uint32_t)(more ? j * NTM + 16 * (g + 1) : 0), tm[par ^ 1]);
-#pragma unroll
-                for (int s = 0; s < 2; ++s)
-#pragma unroll
-                    for (int x = 0; x < R; ++x) {
-                        u64 (&a)[SP] = acc[2 * g + s][x];
-                        a[0] = ffma2(pack2(w[8 * s], w[8 * s + 1]), qa[x].x, a[0]);
-                        a[SP - 1] = ffma2(pack2(w[8 * s + 2], w[8 * s + 3]), qa[x].y, a[SP - 1]);
-                        a[0] = ffma2(pack2(w[8 * s + 4], w[8 * s + 5]), qb[x].x, a[0]);
-                        a[SP - 1] = ffma2(pack2(w[8 * s + 6], w[8 * s + 7]), qb[x].y, a[SP - 1]);
-                    }
-            }
-#pragma unroll
-            for (int s = 0; s < NSM; ++s)
-#pragma unroll
-                for (int x = 0; x < R; ++x) {
-                    u64 (&a)[SP] = acc[NTM + s][x];
-                    a[0] = ffma2(ha[s].x, qa[x].x, a[0]);
-                    a[SP - 1] = ffma2(ha[s].y, qa[x].y, a[SP - 1]);
-                    a[0] = ffma2(hb[s].x, qb[x].x, a[0]);
-                    a[SP - 1] = ffma2(hb[s].y, qb[x].y, a[SP - 1]);
-                }
+        for (int j = 0; j < L; j += 16) {
+            chunk(j, 0);
+            if (j + 8 >= L) break;
+            chunk(j + 8, 1);
         }
     }
     tmem_wait_ld(tm[0]);
@@ -276,9 +302,29 @@ __device__ __forceinline__ void row_products(const float4 *hs, int hs_stride, ui
             u[s][x] = SP == 2 ? sum2(acc[s][x][0]) + sum2(acc[s][x][SP - 1]) : sum2(acc[s][x][0]);
 }
 
+// The one row a lane holds of a plate without classes (N <= 32): rounded products
+// added in column order, as the streaming kernel's row groups combine them.
+template <int R, int NTM>
+__device__ __forceinline__ void dense_row(uint32_t taddr, int L, const float *const (&q)[R], float (&u)[R]) {
+#pragma unroll
+    for (int x = 0; x < R; ++x) u[x] = 0.f;
+#pragma unroll 1
+    for (int j = 0; j < L; j += 8) {
+        uint32_t w[16];
+        tmem_ld_rows2(taddr + (uint32_t)(j * NTM), w);
+        tmem_wait_ld(w);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+#pragma unroll
+            for (int x = 0; x < R; ++x)
+                u[x] = __fadd_rn(u[x], __fmul_rn(__uint_as_float(w[e]), q[x][j + e]));
+    }
+}
+
 }  // namespace
 
-template <int R, int NTM, int NSM, int LMAX>
+// SAME: with the streaming kernel's order of every sum, digit for digit.
+template <int R, int NTM, int NSM, int NREG, int LMAX, bool SAME>
 __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q) {
     extern __shared__ __align__(16) float sm[];
     __shared__ ResCta A;
@@ -286,11 +332,11 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     const PlateParams &P = Q.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr bool REV = R >= 2, FWD = R == 1, FUSED = R == 3;
-    constexpr int NR = NTM + NSM;                 // rows of a lane
+    constexpr int NR = NTM + NSM + NREG;          // rows of a lane
     constexpr int XF = R == 3 ? 4 : R;            // floats per exchanged entry
     constexpr int QB = ((LMAX + 31) & ~31) + 8;
     const int W = Q.warps, WT = 32 * W;
-    const ResLayout O = res_layout(R, W, LMAX, Q.L, Q.n_max, Q.no_max, Q.max_sub, NSM);
+    const ResLayout O = res_layout(R, W, LMAX, Q.L, Q.no_max, Q.max_sub, Q.segs, NSM);
     uint64_t *bar_f = reinterpret_cast<uint64_t *>(sm);        // forces of the owned modes
     uint64_t *bar_q = bar_f + 1;                               // new right-hand sides
     uint64_t *bar_y = bar_f + 2;                               // pickup terms (two buffers)
@@ -326,7 +372,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         bar_init(bar_y + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (sub > 1) {
-            bar_expect_tx(bar_f, (uint32_t)(sub * no * XF * 4));
+            bar_expect_tx(bar_f, (uint32_t)(A.segs_all * no * XF * 4));
             bar_expect_tx(bar_q, (uint32_t)(N * 4 * (FUSED ? 2 : 1)));
         }
     }
@@ -349,7 +395,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     int mp[2] = {0, 0};
     uint32_t mdst[2] = {0u, 0u}, mbar[2] = {0u, 0u};
     bool mon[2] = {false, false};
-    if (used && tid < WT) {
+    if (used) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = tid + h * WT;
@@ -360,7 +406,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             if (sub > 1) {
                 const int own = ((i + 1) * sub - 1) / N;
                 const int o0 = (int)((long long)N * own / sub);
-                mdst[h] = peer_addr(su32(sm + O.xch) + (uint32_t)((rank * Q.no_max + i - o0) * XF * 4),
+                mdst[h] = peer_addr(su32(sm + O.xch) + (uint32_t)((A.seg0 * Q.no_max + i - o0) * XF * 4),
                                     (uint32_t)(A.base + own));
                 mbar[h] = peer_addr(su32(bar_f), (uint32_t)(A.base + own));
             }
@@ -375,8 +421,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     __syncthreads();
     cluster_sync_all();      // every peer's barriers exist before the first store
 
-    const bool pick_here = FWD && used && rank == sub - 1;
-    if (used && tid < WT) {
+    if (used) {
         // ---- row role: rows of stress mode k0 + warp
         const bool kon = warp < nk;
         const int ra = cls ? lane >> 3 : 0;
@@ -386,9 +431,12 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const uint32_t taddr = tmem0 + ((uint32_t)(32 * (warp & 3)) << 16) +
                                (warp >= 4 ? (uint32_t)(Q.tcols / 2) : 0u);
         float4 *const hsm = reinterpret_cast<float4 *>(sm + O.hs) + tid;
+        u64 hreg[NREG > 0 ? NREG : 1][LMAX / 2];                // register rows
         float kap = 0.f, ks = 0.f, kcmp = 0.f;                  // kappa, d kappa (Kahan)
         {
             const int ncl = cls ? pick4r(d.ncls, ra) : N;       // rows of this lane's class
+            // element (row, j) at off + j stride + row: a row of H^k is read as the
+            // column the streaming kernel sums (H need not be symmetric to the last bit)
             long long off = 0;
             int n = 0, stride = 0;
             if (kon) {
@@ -400,10 +448,10 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 if (cls) {
                     const ClusterK K = Q.kinfo[d.k_off + kl];
                     kc = K.c;
+                    const int w = (ncl + 3) & ~3;
                     n = pick4r(d.ncls, ra ^ kc);
-                    const int w = (n + 3) & ~3;
                     long long sb = 0;
-                    for (int a2 = 0; a2 < ra; ++a2)
+                    for (int a2 = 0; a2 < (ra ^ kc); ++a2)
                         sb += (long long)pick4r(d.ncls, a2) * K.mc *
                               ((pick4r(d.ncls, a2 ^ kc) + 3) & ~3);
                     off = K.off + sb + (long long)K.kpos * w;
@@ -420,7 +468,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     float v[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e)
-                        v[e] = (row < ncl && j + e < n) ? P.H[off + (long long)row * stride + j + e]
+                        v[e] = (row < ncl && j + e < n) ? P.H[off + (long long)(j + e) * stride + row]
                                                         : 0.f;
                     __syncwarp();
                     tmem_st8(taddr + (uint32_t)(j * NTM + 8 * s), v);
@@ -432,12 +480,25 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 for (int j = 0; j < L; ++j)
                     if (row < ncl && j < n)
                         reinterpret_cast<float *>(hsm + (s * (L / 4) + j / 4) * WT)[j & 3] =
-                            P.H[off + (long long)row * stride + j];
+                            P.H[off + (long long)j * stride + row];
+            }
+#pragma unroll
+            for (int s = 0; s < NREG; ++s) {
+                const int row = l0 + gl * (NTM + NSM + s);
+#pragma unroll
+                for (int j = 0; j < LMAX; j += 2) {
+                    float v[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        v[e] = (row < ncl && j + e < n) ? P.H[off + (long long)(j + e) * stride + row] : 0.f;
+                    hreg[s][j / 2] = pack2(__float_as_uint(v[0]), __float_as_uint(v[1]));
+                }
             }
         }
         const float *const qcol = rhs + (cls ? (ra ^ kc) * QB : 0);
         const float *const qrow = rhs + ra * QB + l0;
-        float *const fp = sm + O.fp + warp * R * 4 * QB + ra * QB + l0;
+        float *const fpw = sm + O.fp + warp * R * 4 * QB, *const fp = fpw + ra * QB + l0;
+        float *const kew = sm + O.ke;
 
         // ---- update role: owned mode 32 chunk + lane.  The chunks go to the last
         // warps first (those without a stress mode, if any); the warps repeat them.
@@ -448,11 +509,11 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const bool on = upd && oi < no;
         const bool lead = on && rep == 0;                       // writes the mode's results
         // the warps that repeat a chunk share its sums and stores: bits 0..4 the
-        // gradient sums, then w, q', v' of the segments and the pickup
+        // gradient sums, then w, q', v' of the segments
         int duty = 0;
-        for (int g = 0; g < 9; ++g)
+        for (int g = 0; g < 8; ++g)
             if (on && g % reps == rep) duty |= 1 << g;
-        constexpr int kDutyW = 1 << 5, kDutyQ = 1 << 6, kDutyV = 1 << 7, kDutyY = 1 << 8;
+        constexpr int kDutyW = 1 << 5, kDutyQ = 1 << 6, kDutyV = 1 << 7;
         const long long m = d.mode_off + m0 + oi;
         float *const cf = sm + O.coef + tid;
         float *const ga = sm + O.gacc + tid;
@@ -481,7 +542,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             }
         }
         // running addresses of the step's stored states
-        const bool rec = FWD && P.mode == MODE_RECOMPUTE;
+        const bool rec = SAME && FWD && P.mode == MODE_RECOMPUTE;
         float *pq = (FUSED ? P.rseg_q : P.seg_q) + m, *pv = (FUSED ? P.rseg_v : P.seg_v) + m;
         float *pw = P.seg_w ? P.seg_w + (long long)(rsteps - 1) * TM + m : nullptr;
         const float *pvn = REV ? P.seg_v + (long long)(rsteps - 2) * TM + m : nullptr;
@@ -500,7 +561,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             ck[2 * TM + m] = y2;
             ck[3 * TM + m] = y3;
         };
-        const bool ckpt = FWD && P.mode == MODE_FORWARD && P.ckpt;
+        const bool ckpt = SAME && FWD && P.mode == MODE_FORWARD && P.ckpt;
         int ck_left = P.ckpt_K, ck_idx = 1;                     // steps to the next checkpoint
         if (on) {
             if (ckpt && lead) store_ckpt(0);
@@ -546,13 +607,38 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         float *px = (REV && P.xe && (d.has_dir || P.xe_all))
                         ? P.xe + (long long)(rsteps - 1) * 2 * P.total_k + d.k_off + kl : nullptr;
         const bool st_x = px && kon && lane == 0;
-        const uint32_t tx_f = (uint32_t)(sub * no * XF * 4), tx_q = (uint32_t)(N * 4 * (FUSED ? 2 : 1));
+        const uint32_t tx_f = (uint32_t)(A.segs_all * no * XF * 4), tx_q = (uint32_t)(N * 4 * (FUSED ? 2 : 1));
         const uint32_t q_dst = su32(rhs + cpos + (REV ? bw : 0)), q_bar = su32(bar_q);
         const uint32_t q_dst0 = sub > 1 ? peer_addr(q_dst, (uint32_t)(A.base + min(rep, sub - 1))) : 0u;
         const uint32_t q_bar0 = sub > 1 ? peer_addr(q_bar, (uint32_t)(A.base + min(rep, sub - 1))) : 0u;
-        const uint32_t y_dst0 = sub > 1 ? peer_addr(su32(sm + O.pick + 2 * (m0 + oi)), (uint32_t)(A.base + sub - 1)) : 0u;
+        // pickups: a warp per chunk sums its modes' terms every step; one warp of the
+        // last rank adds the chunks' terms, eight steps at a time
+        const bool picks = FWD && upd && rep == 0;
+        const bool collects = FWD && upd && rank == sub - 1 && wr == 0;
+        const int cmax = ((N + sub - 1) / sub + 31) / 32, yent = rank * cmax + chunk;
+        int chunks_all = 0;
+        for (int r = 0; r < sub; ++r)
+            chunks_all += max(((int)((long long)N * (r + 1) / sub) - (int)((long long)N * r / sub) + 31) / 32, 1);
+        float2 *const pst = reinterpret_cast<float2 *>(sm + O.pst) + chunk * kPickSteps * kPickPitch;
+        const uint32_t y_dst0 = sub > 1 ? peer_addr(su32(sm + O.pick + 2 * yent), (uint32_t)(A.base + sub - 1)) : 0u;
         const uint32_t y_bar0 = sub > 1 ? peer_addr(su32(bar_y), (uint32_t)(A.base + sub - 1)) : 0u;
-        const uint32_t xbuf = (uint32_t)(sub * Q.no_max * XF * 4);
+        auto arm_y = [&](int grp) {
+            const int cnt = min(kPickSteps, P.steps - grp * kPickSteps);
+            if (sub > 1 && cnt > 0 && lane == 0) bar_expect_tx(bar_y + (grp & 1), (uint32_t)(cnt * chunks_all * 8));
+        };
+        if (collects) {
+            arm_y(0);
+            arm_y(1);
+        }
+        bool bad = false;
+        const int seg_last = A.seg_last, segs_all = A.segs_all;
+        const unsigned long long new_item = A.new_item;
+        // every part a partial sum of its own, or one row of them: one chain (with the
+        // selects of the general case 24 parts took 1 230 cycles)
+        const unsigned long long later = segs_all < 64 ? (1ull << segs_all) - 2ull : ~1ull;
+        const bool flat = !SAME || new_item == later || new_item == 0ull;
+        const uint32_t xbuf = (uint32_t)(Q.segs * Q.no_max * XF * 4);
+        const uint32_t sbuf = (uint32_t)(Q.no_max * XF * 4);        // one part
         // the next phases are armed by a thread that has waited for the last ones
         const bool arms = sub > 1 && wr == 0 && lane == 0;
         bool dead = false;
@@ -564,6 +650,30 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             }
             dead = i >= kResWait;
         };
+        // lane = 4 step + part: a quarter of the chunks' terms of one of eight steps
+        auto collect = [&](int grp) {
+            if (sub > 1) wait(bar_y + (grp & 1), (uint32_t)((grp >> 1) & 1));
+            const int s8 = lane >> 2, part = lane & 3, n8 = grp * kPickSteps + s8;
+            const float *pk = sm + O.pick + ((grp & 1) * kPickSteps + s8) * 2 * O.PS;
+            float ys = 0.f, ye = 0.f;
+            for (int j = part; j < sub * cmax; j += 4) {
+                const float2 v = *reinterpret_cast<const float2 *>(pk + 2 * j);
+                pickup_merge(ys, ye, v.x, v.y);
+            }
+#pragma unroll
+            for (int o = 1; o <= 2; o <<= 1) {
+                const float s2 = __shfl_xor_sync(0xffffffffu, ys, o);
+                const float e2 = __shfl_xor_sync(0xffffffffu, ye, o);
+                pickup_merge(ys, ye, s2, e2);
+            }
+            const float y = ys + ye;
+            if (part == 0 && n8 < P.steps) {
+                if ((!SAME || P.mode == MODE_FORWARD) && P.audio)
+                    P.audio[(long long)A.plate * P.total_steps + P.n_begin + n8] = y;
+                if (!isfinite(y)) bad = true;
+            }
+            arm_y(grp + 2);
+        };
         bar_sync_id(1, WT);
 
         for (int it = 0; it < P.steps; ++it) {
@@ -571,7 +681,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             const bool rev_next = REV && it + 1 < rsteps;
             const int buf = it & 1;
             const int qb = REV ? buf * 4 * QB : 0;
-            if ((it & 31) == 0) load_block(it);
+            if (__builtin_expect((it & 31) == 0, 0)) load_block(it);
             // ---- row products, eta (xi, eta'), this warp's forces.  Rows and columns
             // beyond a class are zero, so nothing is guarded.
             float dot[R];
@@ -581,86 +691,167 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 if constexpr (REV) qs[1] = qcol + bw;
                 if constexpr (FUSED) qs[2] = qcol + br;
                 float u[NR][R];
-                row_products<R, NTM, NSM>(hsm, WT, taddr, L, qs, u);
+                if (SAME && !cls && N <= 32) {
+#pragma unroll
+                    for (int s = 0; s < NR; ++s)
+#pragma unroll
+                        for (int x = 0; x < R; ++x) u[s][x] = 0.f;
+                    dense_row<R, NTM>(taddr, L, qs, u[0]);
+                } else {
+                    row_products<R, NTM, NSM, NREG, LMAX, (SAME || NR > 4 ? 1 : 2)>(hsm, WT, taddr, L, hreg, qs, u);
+                }
+                if constexpr (SAME)
+#pragma unroll
+                    for (int s = 0; s < NR; ++s)
+#pragma unroll
+                        for (int x = 0; x < R; ++x) fp[x * 4 * QB + gl * s] = u[s][x];
 #pragma unroll
                 for (int x = 0; x < R; ++x) dot[x] = 0.f;
+                if (SAME && cls) {
+                    // lane = column quad, the four row classes in order, as the streaming
+                    // kernel's threads sum them
+                    __syncwarp();
+                    if (4 * lane < L)
 #pragma unroll
-                for (int s = 0; s < NR; ++s) {
-                    dot[0] = fmaf(qrow[qb + gl * s], u[s][0], dot[0]);
-                    if constexpr (REV) dot[1] = fmaf(qrow[bw + gl * s], u[s][0], dot[1]);
-                    if constexpr (FUSED) dot[2] = fmaf(qrow[br + gl * s], u[s][2], dot[2]);
+                        for (int a = 0; a < 4; ++a) {
+                            const int o = (a ^ kc) * QB + 4 * lane;
+                            const float4 uv = *reinterpret_cast<const float4 *>(fpw + o);
+                            const float4 qv = *reinterpret_cast<const float4 *>(rhs + qb + o);
+                            dot[0] = fmaf(qv.w, uv.w, fmaf(qv.z, uv.z, fmaf(qv.y, uv.y, fmaf(qv.x, uv.x, dot[0]))));
+                            if constexpr (REV) {
+                                const float4 wv4 = *reinterpret_cast<const float4 *>(rhs + bw + o);
+                                dot[1] = fmaf(wv4.w, uv.w, fmaf(wv4.z, uv.z, fmaf(wv4.y, uv.y, fmaf(wv4.x, uv.x, dot[1]))));
+                            }
+                            if constexpr (FUSED) {
+                                const float4 rv = *reinterpret_cast<const float4 *>(rhs + br + o);
+                                const float4 u2 = *reinterpret_cast<const float4 *>(fpw + 8 * QB + o);
+                                dot[2] = fmaf(rv.w, u2.w, fmaf(rv.z, u2.z, fmaf(rv.y, u2.y, fmaf(rv.x, u2.x, dot[2]))));
+                            }
+                        }
+                } else {
+#pragma unroll
+                    for (int s = 0; s < NR; ++s) {
+                        dot[0] = fmaf(qrow[qb + gl * s], u[s][0], dot[0]);
+                        if constexpr (REV) dot[1] = fmaf(qrow[bw + gl * s], u[s][0], dot[1]);
+                        if constexpr (FUSED) dot[2] = fmaf(qrow[br + gl * s], u[s][2], dot[2]);
+                    }
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
                     for (int x = 0; x < R; ++x) dot[x] += __shfl_xor_sync(0xffffffffu, dot[x], o);
-                const float ke = kap * dot[0];
+                if constexpr (!SAME) {
+                    const float ke = kap * dot[0];
 #pragma unroll
-                for (int s = 0; s < NR; ++s) {
-                    if constexpr (FWD) {
-                        fp[gl * s] = ke * u[s][0];
-                    } else {
-                        const float kx = kap * dot[1];
-                        fp[gl * s] = fmaf(ke, u[s][1], 2.f * kx * u[s][0]);   // J w
-                        fp[4 * QB + gl * s] = ke * u[s][0];                   // f(q^n)
-                    }
-                    if constexpr (FUSED) fp[8 * QB + gl * s] = (kap * dot[2]) * u[s][2];
+                    for (int s = 0; s < NR; ++s) fp[gl * s] = ke * u[s][0];
+                } else if (lane == 0) {
+                    float4 *const k4 = reinterpret_cast<float4 *>(kew + 8 * warp);
+                    k4[0] = make_float4(kap * dot[0], kap, REV ? 2.f * dot[REV ? 1 : 0] : 0.f, dot[0]);
+                    if constexpr (FUSED) k4[1] = make_float4(kap * dot[FUSED ? 2 : 0], 0.f, 0.f, 0.f);
                 }
             }
             const float qn = REV ? rhs[qb + cpos] : 0.f;
             if (REV) copies_done();   // the next step's q^n (and this step's v^n) have arrived
             bar_sync_id(1, WT);       // the CTA's forces are in place, its right-hand sides read
             const int pb = (it / kPickSteps) & 1, ps = it % kPickSteps;
-            if (pick_here && ps == 0 && it >= 2 * kPickSteps) bar_sync_id(4 + pb, WT + 32);
-            // ---- forces of the CTA's stress modes (warps without one left zeros),
-            // then of the plate
-            auto cta_force = [&](int pos, float (&f)[R]) {
+            // ---- forces.  A part is the sum over one run of stress modes, in order
+            // (emit is called with each); the plate's force adds its parts in order,
+            // item by item of the streaming kernel's work split where the plan asks
+            // for its rounding (new_item), else all in one row.
+            auto parts = [&](int pos, auto emit) {
                 const float *p = sm + O.fp + pos;
+                float f[R];
 #pragma unroll
                 for (int x = 0; x < R; ++x) f[x] = 0.f;
+                if constexpr (!SAME) {
 #pragma unroll
-                for (int w = 0; w < kResMaxWarps; ++w)
+                    for (int w = 0; w < kResMaxWarps; ++w) f[0] += w < nk ? p[w * 4 * QB] : 0.f;
+                    emit(0, f);
+                    return;
+                }
+                int seg = 0;
 #pragma unroll
-                    for (int x = 0; x < R; ++x) f[x] += w < W ? p[(w * R + x) * 4 * QB] : 0.f;
+                for (int w = 0; w < kResMaxWarps; ++w, p += R * 4 * QB) {
+                    if (w >= nk) break;
+                    const float4 k4 = *reinterpret_cast<const float4 *>(kew + 8 * w);
+                    const float uu = p[0];
+                    if constexpr (FWD) {
+                        f[0] = fmaf(k4.x, uu, f[0]);
+                    } else {
+                        f[1] = fmaf(k4.x, uu, f[1]);                                        // f(q^n)
+                        f[0] = fmaf(k4.y, fmaf(k4.z, uu, k4.w * p[4 * QB]), f[0]);          // J w
+                    }
+                    if constexpr (FUSED) f[2] = fmaf(kew[8 * w + 4], p[8 * QB], f[2]);
+                    if (seg_last >> w & 1) {
+                        emit(seg, f);
+#pragma unroll
+                        for (int x = 0; x < R; ++x) f[x] = 0.f;
+                        ++seg;
+                    }
+                }
             };
-            float F[R];
+            float F[R], item[R];
 #pragma unroll
-            for (int x = 0; x < R; ++x) F[x] = 0.f;
+            for (int x = 0; x < R; ++x) F[x] = item[x] = 0.f;
+            auto add_part = [&](int g, const float (&v)[R]) {
+                const bool fresh = SAME && (new_item >> g & 1);
+#pragma unroll
+                for (int x = 0; x < R; ++x) {
+                    F[x] += fresh ? item[x] : 0.f;
+                    item[x] = fresh ? v[x] : item[x] + v[x];
+                }
+            };
+            auto load_part = [&](const float *x, float (&v)[R]) {
+                if constexpr (R == 1) {
+                    v[0] = x[0];
+                } else if constexpr (R == 2) {
+                    const float2 t = *reinterpret_cast<const float2 *>(x);
+                    v[0] = t.x;
+                    v[R - 1] = t.y;
+                } else {
+                    const float4 t = *reinterpret_cast<const float4 *>(x);
+                    v[0] = t.x;
+                    v[R > 1 ? 1 : 0] = t.y;
+                    v[R - 1] = t.z;
+                }
+            };
             if (sub > 1) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (!mon[h]) continue;
-                    float f[R];
-                    cta_force(mp[h], f);
                     const uint32_t dst = mdst[h] + (buf ? xbuf : 0u);
-                    if constexpr (R == 1) push1(dst, mbar[h], f[0]);
-                    if constexpr (R == 2) push2(dst, mbar[h], f[0], f[1]);
-                    if constexpr (R == 3) push4(dst, mbar[h], f[0], f[1], f[2]);
+                    parts(mp[h], [&](int seg, const float (&f)[R]) {
+                        const uint32_t to = dst + seg * sbuf;
+                        if constexpr (R == 1) push1(to, mbar[h], f[0]);
+                        if constexpr (R == 2) push2(to, mbar[h], f[0], f[R - 1]);
+                        if constexpr (R == 3) push4(to, mbar[h], f[0], f[R > 1 ? 1 : 0], f[R - 1]);
+                    });
                 }
                 if (upd) {
                     wait(bar_f, (uint32_t)buf);
-                    const float *x = sm + O.xch + (buf * sub * Q.no_max + oi) * XF;
-                    if (on) {
+                    const float *x = sm + O.xch + (buf * Q.segs * Q.no_max + oi) * XF;
+                    if (on && flat) {
 #pragma unroll 8
-                        for (int pr = 0; pr < sub; ++pr, x += Q.no_max * XF) {
-                            if constexpr (R == 1) {
-                                F[0] += x[0];
-                            } else if constexpr (R == 2) {
-                                const float2 v = *reinterpret_cast<const float2 *>(x);
-                                F[0] += v.x;
-                                F[1] += v.y;
-                            } else {
-                                const float4 v = *reinterpret_cast<const float4 *>(x);
-                                F[0] += v.x;
-                                F[1] += v.y;
-                                F[2] += v.z;
-                            }
+                        for (int g = 0; g < segs_all; ++g, x += Q.no_max * XF) {
+                            float v[R];
+                            load_part(x, v);
+#pragma unroll
+                            for (int y = 0; y < R; ++y) F[y] += v[y];
+                        }
+                    } else if (on) {
+#pragma unroll 2
+                        for (int g = 0; g < segs_all; ++g, x += Q.no_max * XF) {
+                            float v[R];
+                            load_part(x, v);
+                            add_part(g, v);
                         }
                     }
                 }
             } else if (on) {
-                cta_force(cpos, F);
+                parts(cpos, [&](int seg, const float (&f)[R]) { add_part(seg, f); });
             }
+#pragma unroll
+            for (int x = 0; x < R; ++x) F[x] += item[x];
             // ---- update and the new right-hand sides
             const float a_old = x0;
             float rr = 0.f, bcf = 0.f, cw = 0.f, wv = 0.f;
@@ -708,18 +899,20 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             }
             if (REV) px -= 2 * P.total_k;
             if (REV && on && rev_on) {
-                auto acc = [&](int idx, float x) {
+                // Kahan sums of x y, the product and the first subtraction in one rounding
+                auto acc = [&](int idx, float x, float y) {
                     if (!(duty & (1 << idx))) return;
-                    float gs = ga[(2 * idx) * WT], gc = ga[(2 * idx + 1) * WT];
-                    kahan_add(gs, gc, x);
-                    ga[(2 * idx) * WT] = gs;
-                    ga[(2 * idx + 1) * WT] = gc;
+                    const float gs = ga[(2 * idx) * WT], gc = ga[(2 * idx + 1) * WT];
+                    const float v = fmaf(x, y, -gc);
+                    const float t = __fadd_rn(gs, v);
+                    ga[(2 * idx) * WT] = t;
+                    ga[(2 * idx + 1) * WT] = __fsub_rn(__fsub_rn(t, gs), v);
                 };
-                acc(GA_A, a_old * qn);
-                acc(GA_V, a_old * sm[O.vst + tid]);
-                acc(GA_F, a_old * fmaf(bcf, e, -F[R > 1 ? 1 : 0]));
-                acc(GA_E, a_old * e);
-                acc(GA_C, ybn * qn1);
+                acc(GA_A, a_old, qn);
+                acc(GA_V, a_old, sm[O.vst + tid]);
+                acc(GA_F, a_old, fmaf(bcf, e, -F[R > 1 ? 1 : 0]));
+                acc(GA_E, a_old, e);
+                acc(GA_C, ybn, qn1);
                 qn1 = qn;
                 if (rev_next) {
                     if (st_w) *pw = wv;
@@ -735,29 +928,59 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             if (FUSED || rec) store_state();
             if (on) {
                 if (ckpt && ck_left == 1 && it + 1 < P.steps && lead) store_ckpt(ck_idx);
-                if (FWD && (duty & kDutyY)) {
-                    // pickup terms of eight steps, summed by the last rank's spare warp
-                    float ys = 0.f, ye = 0.f;
-                    pickup_add(ys, ye, cw, cf[6 * WT], y0, y1);
-                    const int po = (pb * kPickSteps + ps) * O.PS;
-                    if (sub > 1)
-                        push2(y_dst0 + (uint32_t)(po * 4), y_bar0 + 8u * pb, ys, ye);
-                    else
-                        *reinterpret_cast<float2 *>(sm + O.pick + po + 2 * (m0 + oi)) =
-                            make_float2(ys, ye);
+            }
+            if (FWD && picks) {
+                float ys = 0.f, ye = 0.f;
+                if (on) pickup_add(ys, ye, cw, cf[6 * WT], y0, y1);
+                pst[ps * kPickPitch + lane] = make_float2(ys, ye);
+                if (__builtin_expect(ps == kPickSteps - 1 || it == P.steps - 1, 0)) {
+                    // the chunk's sums of up to eight steps, to the last rank
+                    // (lane = 4 step + part, a quarter of the modes each)
+                    __syncwarp();
+                    const int s8 = lane >> 2, part = lane & 3;
+                    ys = ye = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float2 v = pst[s8 * kPickPitch + part + 4 * j];
+                        pickup_merge(ys, ye, v.x, v.y);
+                    }
+#pragma unroll
+                    for (int o = 1; o <= 2; o <<= 1) {
+                        const float s2 = __shfl_xor_sync(0xffffffffu, ys, o);
+                        const float e2 = __shfl_xor_sync(0xffffffffu, ye, o);
+                        pickup_merge(ys, ye, s2, e2);
+                    }
+                    if (part == 0 && s8 <= ps) {
+                        const int po = (pb * kPickSteps + s8) * 2 * O.PS;
+                        if (sub > 1)
+                            push2(y_dst0 + (uint32_t)(po * 4), y_bar0 + 8u * pb, ys, ye);
+                        else
+                            *reinterpret_cast<float2 *>(sm + O.pick + po + 2 * yent) = make_float2(ys, ye);
+                    }
                 }
             }
+            // the last eight steps' samples, one step into the next eight
+            if (collects && __builtin_expect(ps == 1 && it > kPickSteps, 0)) collect(it / kPickSteps - 1);
             if (ckpt && --ck_left == 0) {
                 ck_left = P.ckpt_K;
                 ++ck_idx;
             }
-            if (FWD && sub == 1 && (ps == kPickSteps - 1 || it == P.steps - 1))
-                bar_arrive_id(2 + pb, WT + 32);
             wait(bar_q, (uint32_t)buf);
             if (arms && it + 1 < P.steps) bar_expect_tx(bar_q, tx_q);
         }
 
-        // ---- write back
+        // ---- the last samples, write back
+        if (FWD) {
+            bar_sync_id(1, WT);      // (one CTA: the terms of the last steps are in place)
+            if (collects)
+                for (int g = max(0, (P.steps - 2 - 1) / kPickSteps); g * kPickSteps < P.steps; ++g) {
+                    // groups whose second next step never came
+                    if (g * kPickSteps + kPickSteps + 1 < P.steps) continue;
+                    collect(g);
+                }
+            if (__any_sync(0xffffffffu, bad) && lane == 0)
+                set_status(P.status, A.plate, MDX_ERR_NONFINITE);
+        }
         if (lead) {
             if (FWD && P.mode == MODE_FORWARD) {
                 P.state_io[m] = y0;
@@ -782,49 +1005,6 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             P.kacc[2 * (d.k_off + kl) + 1] = kcmp;
         }
         if (dead && lane == 0) set_status(P.status, A.plate, MDX_ERR_TIMEOUT);
-    } else if (pick_here && warp == W) {
-        // ======================================================== spare warp: pickups
-        // lane = 4 ps + part: a quarter of the modes of one of eight steps
-        const int ps = lane >> 2, part = lane & 3;
-        bool bad = false, dead = false;
-        for (int i0 = 0; i0 < P.steps; i0 += kPickSteps) {
-            const int grp = i0 / kPickSteps, pb = grp & 1;
-            const int cnt = min(kPickSteps, P.steps - i0);
-            if (sub > 1) {
-                if (lane == 0) bar_expect_tx(bar_y + pb, (uint32_t)(cnt * N * 8));
-                long long i = 0;
-                while (!dead && !bar_try(bar_y + pb, (uint32_t)((grp >> 1) & 1)) &&
-                       ++i < 16 * kResWait) {
-                }
-                if (i >= 16 * kResWait) dead = true;
-                __syncwarp();
-            } else {
-                bar_sync_id(2 + pb, WT + 32);
-            }
-            const float *pk = sm + O.pick + (pb * kPickSteps + ps) * O.PS;
-            float ys = 0.f, ye = 0.f;
-            if (ps < cnt)
-                for (int j = part; j < N; j += 4) {
-                    const float2 v = *reinterpret_cast<const float2 *>(pk + 2 * j);
-                    pickup_merge(ys, ye, v.x, v.y);
-                }
-#pragma unroll
-            for (int o = 1; o <= 2; o <<= 1) {
-                const float s2 = __shfl_xor_sync(0xffffffffu, ys, o);
-                const float e2 = __shfl_xor_sync(0xffffffffu, ye, o);
-                pickup_merge(ys, ye, s2, e2);
-            }
-            // the buffer is free for the steps two groups on
-            if (i0 + 2 * kPickSteps < P.steps) bar_arrive_id(4 + pb, WT + 32);
-            const float y = ys + ye;
-            if (part == 0 && ps < cnt) {
-                if (P.mode == MODE_FORWARD && P.audio)
-                    P.audio[(long long)A.plate * P.total_steps + P.n_begin + i0 + ps] = y;
-                if (!isfinite(y)) bad = true;
-            }
-        }
-        if (__any_sync(0xffffffffu, bad) && lane == 0) set_status(P.status, A.plate, MDX_ERR_NONFINITE);
-        if (dead && lane == 0) set_status(P.status, A.plate, MDX_ERR_TIMEOUT);
     }
     __syncwarp();
     tc_fence_before();
@@ -840,28 +1020,39 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
 namespace {
 
 // Kernel variants by longest row: a lane's rows in tensor memory (256 words a
-// thread with more than four warps, else 512) and the rest in shared memory.
+// thread with more than four warps, else 512); of the others, those in registers
+// (kernels without a reverse pass or checkpoints, NREG) and in shared memory.
 constexpr int kVarLen[kResVariants] = {16, 24, 32, 40, 48, 56, 64};
 constexpr int kVarTm[kResVariants] = {2, 2, 4, 4, 4, 4, 6};
 constexpr int kVarSm[kResVariants] = {0, 1, 0, 1, 2, 3, 2};
-// the spare warp makes eight: 255 registers a thread
+constexpr int kVarReg[kResVariants] = {0, 1, 0, 1, 2, 2, 0};
 int var_warps(int v) { return kVarTm[v] * kVarLen[v] > 256 ? 4 : kResMaxWarps; }
+int var_sm(int v, bool same) { return kVarSm[v] - (same ? 0 : kVarReg[v]); }
 
-template <int R>
+template <int R, bool SAME, int V>
+const void *res_fn_v() {
+    constexpr int REG = SAME ? 0 : kVarReg[V];
+    return reinterpret_cast<const void *>(
+        resident_kernel<R, kVarTm[V], kVarSm[V] - REG, REG, kVarLen[V], SAME>);
+}
+template <int R, bool SAME>
 const void *res_fn_r(int v) {
     switch (v) {
-        case 0: return reinterpret_cast<const void *>(resident_kernel<R, 2, 0, 16>);
-        case 1: return reinterpret_cast<const void *>(resident_kernel<R, 2, 1, 24>);
-        case 2: return reinterpret_cast<const void *>(resident_kernel<R, 4, 0, 32>);
-        case 3: return reinterpret_cast<const void *>(resident_kernel<R, 4, 1, 40>);
-        case 4: return reinterpret_cast<const void *>(resident_kernel<R, 4, 2, 48>);
-        case 5: return reinterpret_cast<const void *>(resident_kernel<R, 4, 3, 56>);
-        default: return reinterpret_cast<const void *>(resident_kernel<R, 6, 2, 64>);
+        case 0: return res_fn_v<R, SAME, 0>();
+        case 1: return res_fn_v<R, SAME, 1>();
+        case 2: return res_fn_v<R, SAME, 2>();
+        case 3: return res_fn_v<R, SAME, 3>();
+        case 4: return res_fn_v<R, SAME, 4>();
+        case 5: return res_fn_v<R, SAME, 5>();
+        default: return res_fn_v<R, SAME, 6>();
     }
 }
 
-const void *res_fn(int r, int v) {
-    return r == 1 ? res_fn_r<1>(v) : (r == 2 ? res_fn_r<2>(v) : res_fn_r<3>(v));
+// Right-hand sides r; same: with the streaming kernel's order of the sums (the
+// passes with a reverse have no other).
+const void *res_fn(int r, int v, bool same) {
+    if (r == 1) return same ? res_fn_r<1, true>(v) : res_fn_r<1, false>(v);
+    return r == 2 ? res_fn_r<2, true>(v) : res_fn_r<3, true>(v);
 }
 
 void res_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, int grid, int cs, int threads,
@@ -903,8 +1094,8 @@ int resident_columns(int variant, int L, int warps) {
 // fit an SM together (of this or another launch) never wait for each other's
 // columns: a CTA whose cluster peers wait must not block on an allocation.
 size_t resident_smem(int R, const ResidentParams &Q) {
-    const ResLayout o = res_layout(R, Q.warps, kVarLen[Q.variant], Q.L, Q.n_max, Q.no_max,
-                                    Q.max_sub, kVarSm[Q.variant]);
+    const ResLayout o = res_layout(R, Q.warps, kVarLen[Q.variant], Q.L, Q.no_max, Q.max_sub,
+                                    Q.segs, var_sm(Q.variant, Q.same));
     return std::max(sizeof(float) * (size_t)o.end, (size_t)Q.tcols * kSmemPerColumn);
 }
 
@@ -912,8 +1103,8 @@ size_t resident_smem(int R, const ResidentParams &Q) {
 // once (0: the shape cannot be launched).
 cudaError_t resident_check(int cs, const ResidentParams &Q, size_t smem_optin, int *fit) {
     *fit = 1 << 30;
-    for (int r = 1; r <= 3; ++r) {
-        const void *fn = res_fn(r, Q.variant);
+    for (int r = 1; r <= (Q.same ? 3 : 1); ++r) {
+        const void *fn = res_fn(r, Q.variant, Q.same);
         const size_t smem = resident_smem(r, Q);
         if (smem + kResStatic > smem_optin) {
             *fit = 0;
@@ -927,7 +1118,7 @@ cudaError_t resident_check(int cs, const ResidentParams &Q, size_t smem_optin, i
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at[1];
-        res_config(cfg, at, cs, cs, 32 * Q.warps + (r == 1 ? 32 : 0), smem, nullptr);
+        res_config(cfg, at, cs, cs, 32 * Q.warps, smem, nullptr);
         int n = 0;
         e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
         if (e != cudaSuccess) return e;
@@ -941,10 +1132,10 @@ cudaError_t launch_resident(int R, const ResidentParams &Q, int grid, int cs, si
     if (grid <= 0 || Q.p.steps <= 0) return cudaSuccess;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
-    res_config(cfg, at, grid, cs, 32 * Q.warps + (R == 1 ? 32 : 0), smem, s);
+    res_config(cfg, at, grid, cs, 32 * Q.warps, smem, s);
     ResidentParams q = Q;
     void *args[] = {&q};
-    return cudaLaunchKernelExC(&cfg, res_fn(R, Q.variant), args);
+    return cudaLaunchKernelExC(&cfg, res_fn(R, Q.variant, Q.same), args);
 }
 
 }  // namespace mdx
