@@ -236,7 +236,9 @@ struct ClusterK {
 };
 
 constexpr int kResMaxModes = 256;     // transverse modes of a plate
-constexpr int kResVariants = 7;       // kernel variants, by row length
+constexpr int kResVariants = 8;       // kernel variants, by row length
+constexpr size_t kResStatic = 1024;   // room for the static shared memory
+constexpr int kResLays = 4;           // most layouts of the right-hand sides in a CTA
 
 // Work of one CTA: rank `rank` of the `sub` CTAs that share plate `plate`.
 struct ResCta {
@@ -248,6 +250,15 @@ struct ResCta {
     int seg_last;                     // bit w: warp w's mode ends a part of the force
     int seg0, segs_all;               // this CTA's first part, parts of the plate
     unsigned long long new_item;      // bit g: part g starts a new partial sum
+    // Layouts of the right-hand sides: 0 class by class; l > 0 with a zero after
+    // every gap[l - 1][class] modes of a class (0: none).  Warp w reads layout
+    // lay_of >> 4 w & 15.
+    int lays;
+    unsigned lay_of;
+    int gap[kResLays - 1][4];
+    int carry;                        // bit 0: the first part begins in the CTA before,
+                                      // bit 1: the last one ends in a later CTA
+    int tail;                         // first warp of the part that ends later (carry bit 1)
 };
 
 struct ResidentParams {
@@ -261,6 +272,8 @@ struct ResidentParams {
     int L;                            // longest padded row
     int no_max;                       // most modes owned by a CTA
     int max_sub, segs;                // most CTAs and parts of a plate
+    int n_max;                        // most modes of a plate
+    int lays, carry;                  // most layouts of a CTA; any part spans CTAs
     int tcols;                        // tensor-memory columns per CTA
 };
 

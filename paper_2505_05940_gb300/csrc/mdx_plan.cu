@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1183,14 +1184,35 @@ double res_load_cycles(int nk, int L) { return 0.1 * L * L * nk; }
 // A plate of the resident launch, and one way to share it: the stress modes of
 // its CTAs are [kb[r], kb[r + 1]).
 struct ResPlate {
-    int inst, N, M, L;
+    int inst, N, M, L;           // L: padded row length
+    // (same order) modes of a class after which the streaming kernel's rows change
+    // sides of its even / odd chains, by stress mode and class of the row (0: never)
+    std::vector<std::array<int, 4>> gaps;
     std::vector<int> runs;       // lengths of the runs of stress modes summed in one row
     unsigned long long new_item = 0;
+    bool starts(int k) const {   // a run starts at stress mode k
+        for (int len : runs) {
+            if (k <= 0) break;
+            k -= len;
+        }
+        return k == 0;
+    }
 };
 struct ResShare {
-    int sub, nk, warps;          // CTAs, most stress modes of one, its warps
+    int sub;                     // CTAs
+    int nk = 0, warps = 0;       // most stress modes of one, its warps
+    int lays = 1, hops = 0;      // most layouts of the right-hand sides; CTAs a run goes on in
     std::vector<int> kb;
 };
+
+// Layouts of the right-hand sides for stress modes k0 .. k1 - 1: the plain one
+// first, then every distinct set of gaps.
+std::vector<std::array<int, 4>> lays_of(const ResPlate &q, int k0, int k1) {
+    std::vector<std::array<int, 4>> v{{{0, 0, 0, 0}}};
+    for (int k = k0; k < k1; ++k)
+        if (std::find(v.begin(), v.end(), q.gaps[k]) == v.end()) v.push_back(q.gaps[k]);
+    return v;
+}
 
 // One resident launch: `same` keeps the runs of the streaming kernel's sums.
 int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, bool same,
@@ -1203,62 +1225,79 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
         const int own = ((q.N + s.sub - 1) / s.sub + 31) / 32;
         return std::max({s.nk, own, (q.N + 63) / 64, std::min(s.nk + own, wmax)});
     };
+    // (150: no warp without a stress mode is left for the pickups; 600: a hop of a
+    // part that spans CTAs)
+    auto cycles = [&](const ResPlate &q, const ResShare &s) {
+        return res_chain_cycles(s.nk, q.L, s.sub) + (s.nk < s.warps ? 0.0 : 150.0) + 600.0 * s.hops;
+    };
+    auto include = [&](ResidentParams &Q, const ResPlate &q, const ResShare &s) {
+        Q.variant = variant;
+        Q.same = same;
+        Q.L = std::max(Q.L, q.L);
+        Q.warps = std::max(Q.warps, s.warps);
+        Q.no_max = std::max(Q.no_max, (q.N + s.sub - 1) / s.sub);
+        Q.max_sub = std::max(Q.max_sub, s.sub);
+        Q.n_max = std::max(Q.n_max, q.N);
+        Q.lays = std::max(Q.lays, s.lays);
+        Q.carry |= s.hops > 0;
+        Q.segs = std::max(Q.segs, same ? (int)q.runs.size() : s.sub);
+        Q.tcols = resident_columns(variant, Q.L, Q.warps);
+    };
+    // the ways to share a plate, by their number of CTAs
     auto shares = [&](const ResPlate &q, int wmax, int csmax) {
         std::vector<ResShare> v;
         auto add = [&](ResShare s) {
-            s.nk = 0;
-            for (int r = 0; r < s.sub; ++r) s.nk = std::max(s.nk, s.kb[r + 1] - s.kb[r]);
+            if (s.sub > csmax || s.sub > q.M) return;
+            int hops = 0;
+            for (int r = 0; r < s.sub; ++r) {
+                s.nk = std::max(s.nk, s.kb[r + 1] - s.kb[r]);
+                if (!same) continue;
+                s.lays = std::max(s.lays, (int)lays_of(q, s.kb[r], s.kb[r + 1]).size());
+                hops = r > 0 && !q.starts(s.kb[r]) ? hops + 1 : 0;
+                s.hops = std::max(s.hops, hops);
+                // (the part that a CTA passes on waits for nothing if its run begins there)
+                for (int k = s.kb[r] + 1; k < s.kb[r + 1]; ++k)
+                    if (q.starts(k)) hops = 0;
+            }
             s.warps = warps_of(q, s, wmax);
-            if (s.sub <= csmax && s.warps <= wmax &&
-                (v.empty() || v.back().sub != s.sub))
-                v.push_back(s);
+            if (s.warps > wmax || s.lays > kResLays) return;
+            ResidentParams Q{};
+            include(Q, q, s);
+            if (resident_smem(same ? 3 : 1, Q) + kResStatic > (size_t)smem_optin) return;
+            auto at = std::find_if(v.begin(), v.end(), [&](const ResShare &o) { return o.sub >= s.sub; });
+            if (at == v.end() || at->sub != s.sub)
+                v.insert(at, s);
+            else if (cycles(q, s) < cycles(q, *at))
+                *at = s;
         };
-        if (same) {
-            // whole runs only, from many CTAs to few, then reversed
-            for (int cap = 1; cap <= wmax; ++cap) {
-                ResShare s{0, 0, 0, {0}};
-                int k = 0, n = 0;
-                bool fits = true;
-                for (int len : q.runs) {
-                    fits = fits && len <= cap;
-                    if (n + len > cap) {
-                        s.kb.push_back(k);
-                        n = 0;
-                    }
-                    n += len;
-                    k += len;
+        for (int sub : {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16}) {
+            ResShare s{sub};
+            for (int r = 0; r <= sub; ++r) s.kb.push_back((int)((long long)q.M * r / sub));
+            add(s);
+        }
+        for (int cap = 1; same && cap <= wmax; ++cap) {     // whole runs
+            ResShare s{0};
+            s.kb.push_back(0);
+            int k = 0, n = 0;
+            bool fits = true;
+            for (int len : q.runs) {
+                fits = fits && len <= cap;
+                if (n + len > cap) {
+                    s.kb.push_back(k);
+                    n = 0;
                 }
-                s.kb.push_back(k);
-                s.sub = (int)s.kb.size() - 1;
-                if (fits) add(s);
+                n += len;
+                k += len;
             }
-            std::reverse(v.begin(), v.end());
-        } else {
-            for (int sub : {1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 16}) {
-                if (sub > q.M) break;
-                ResShare s{sub, 0, 0, {}};
-                for (int r = 0; r <= sub; ++r) s.kb.push_back((int)((long long)q.M * r / sub));
-                add(s);
-            }
+            s.kb.push_back(k);
+            s.sub = (int)s.kb.size() - 1;
+            if (fits) add(s);
         }
         return v;
     };
-    // (150: no warp without a stress mode is left for the pickups)
-    auto cycles = [&](const ResPlate &q, const ResShare &s) {
-        return res_chain_cycles(s.nk, q.L, s.sub) + (s.nk < s.warps ? 0.0 : 150.0);
-    };
     auto shape = [&](const std::vector<ResShare> &sh) {
         ResidentParams Q{};
-        Q.variant = variant;
-        Q.same = same;
-        for (size_t i = 0; i < pls.size(); ++i) {
-            Q.L = std::max(Q.L, pls[i].L);
-            Q.warps = std::max(Q.warps, sh[i].warps);
-            Q.no_max = std::max(Q.no_max, (pls[i].N + sh[i].sub - 1) / sh[i].sub);
-            Q.max_sub = std::max(Q.max_sub, sh[i].sub);
-            Q.segs = std::max(Q.segs, same ? (int)pls[i].runs.size() : sh[i].sub);
-        }
-        Q.tcols = resident_columns(variant, Q.L, Q.warps);
+        for (size_t i = 0; i < pls.size(); ++i) include(Q, pls[i], sh[i]);
         return Q;
     };
     // clusters: plates sorted by (CTAs, time), as many per cluster as fit, longest
@@ -1305,7 +1344,8 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
     int best_cs = 0, best_fit = 1;
     std::vector<ResShare> best_sh;
     ResidentParams best_q{};
-    for (int wmax : {4, resident_max_warps(variant)})
+    for (int wmax : {4, 6, 8}) {
+        if (wmax > resident_max_warps(variant)) break;
         for (int csmax : {8, 16}) {
             std::vector<std::vector<ResShare>> cand;
             std::vector<double> taus;
@@ -1336,6 +1376,9 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
                 }
                 if (subs == prev) continue;
                 prev = subs;
+                double longest = 0.0;
+                for (size_t i = 0; i < pls.size(); ++i) longest = std::max(longest, cycles(pls[i], sh[i]));
+                if (longest >= 0.98 * best) continue;
                 const ResidentParams Q = shape(sh);
                 int fit = 0;
                 if (resident_check(cs, Q, (size_t)smem_optin, &fit) != cudaSuccess) {
@@ -1358,6 +1401,7 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
                 }
             }
         }
+    }
     if (best_cs == 0) return MDX_OK;
     // ---- tables
     std::vector<std::vector<int>> cl;
@@ -1390,8 +1434,21 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
                 for (int w = 0; w < A.nk; ++w)
                     if (last[A.k0 + w]) {
                         A.seg_last |= 1 << w;
+                        A.tail = w + 1;
                         ++seg;
                     }
+                A.lays = 1;
+                if (same) {
+                    if (r > 0 && !q.starts(A.k0)) A.carry |= 1;
+                    if (A.tail < A.nk) A.carry |= 2;
+                    const auto lays = lays_of(q, A.k0, A.k0 + A.nk);
+                    A.lays = (int)lays.size();
+                    for (int l = 1; l < A.lays; ++l)
+                        for (int c = 0; c < 4; ++c) A.gap[l - 1][c] = lays[l][c];
+                    for (int w = 0; w < A.nk; ++w)
+                        A.lay_of |= (unsigned)(std::find(lays.begin(), lays.end(), q.gaps[A.k0 + w]) - lays.begin())
+                                    << (4 * w);
+                }
                 ctas.push_back(A);
             }
             base += s.sub;
@@ -1418,8 +1475,8 @@ int build_resident(mdx_plan *p, const std::vector<ResPlate> &pls, int variant, b
 
 int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
                   const std::vector<PlateItem> &items, int smem_optin) {
-    std::vector<ResPlate> pls;
-    int variant = 0;
+    std::vector<ResPlate> pls, sames;
+    int variant = 0, variant_same = 0;
     bool same = true;
     std::vector<std::vector<const PlateItem *>> its(p->n_inst);
     for (const auto &it : items) its[it.inst].push_back(&it);
@@ -1435,15 +1492,17 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
         q.N = d.N;
         q.M = d.M;
         q.L = (w + 7) & ~7;
+        q.gaps.assign(d.M, {{0, 0, 0, 0}});
         // The streaming kernel's sums of this plate: per item (in contributor order)
         // a row of FMAs over each class chunk, or over the whole item without
         // classes.  Gradients depend on them in their last digits, so passes with
-        // checkpoints keep them: the resident kernel takes such a plan when its
-        // runs fit the CTAs and the rows' even / odd chains do not change sides
-        // within a chunk (a stage of an odd number of rows before the last).
+        // checkpoints keep them.  A row adds alternate modes to two chains and starts
+        // them anew with every stage of the ring, so behind a stage of an odd number
+        // of modes the chains change sides: the resident kernel's rows have a zero
+        // there (gaps).
         std::vector<const PlateItem *> &list = its[i];
         std::sort(list.begin(), list.end(), [](const PlateItem *a, const PlateItem *b) { return a->slot < b->slot; });
-        int k = 0;
+        int k = 0, ws = w;                       // ws: longest row with its gaps
         for (const PlateItem *it : list) {
             if (it->k0 != k) same = false;       // contributors out of order
             k = it->k1;
@@ -1462,12 +1521,20 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
                     const int na = d.ncls[a], nb = d.ncls[a ^ ch.c];
                     if (na == 0 || nb == 0) continue;
                     const int rps = std::max(1, p->stage_bytes / 4 / (ch.mc * ((nb + 3) & ~3)));
-                    if (rps < na && (rps & 1)) same = false;
+                    if (rps < na && (rps & 1)) {
+                        for (int kk = ch.kl0; kk < ch.kl0 + ch.mc; ++kk) q.gaps[kk][a] = rps;
+                        ws = std::max(ws, na + (na - 1) / rps);
+                    }
                 }
             }
         }
         if (k != d.M || q.runs.size() > 64) same = false;
         pls.push_back(q);
+        const int vs = resident_variant(ws, d.parity ? (w + 7) / 8 : (d.N + 31) / 32);
+        if (vs < 0) same = false;
+        variant_same = std::max(variant_same, vs);
+        q.L = (ws + 7) & ~7;
+        sames.push_back(q);
     }
     if (pls.empty()) return MDX_OK;
     std::vector<ClusterK> kinfo(std::max<long long>(p->total_k, 1));
@@ -1492,7 +1559,7 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
     int *di = nullptr, rc;
     if ((rc = upload(p, &dk, kinfo.data(), kinfo.size()))) return rc;
     if ((rc = upload(p, &di, iperm.data(), iperm.size()))) return rc;
-    if (same && (rc = build_resident(p, pls, variant, true, dk, di, smem_optin, &p->res_same))) return rc;
+    if (same && (rc = build_resident(p, sames, variant_same, true, dk, di, smem_optin, &p->res_same))) return rc;
     return build_resident(p, pls, variant, false, dk, di, smem_optin, &p->res_fast);
 }
 

@@ -14,19 +14,24 @@
 // forward, 40 us fused per step).  Plates are independent, so they need not
 // advance together: one plate at a time fits a few SMs.  A plate runs on `sub`
 // CTAs (1 to 16) of one thread-block cluster through the whole time loop;
-// clusters that do not fit at once run one after the other.
+// clusters that do not fit at once run one after the other.  Measured, streaming
+// and here: 100 x 30 plate, 11 025 steps, 34.3 and 13.1 ms; 96 plates of 50 to
+// 200 modes 196 and 37.5 ms; a fit's step (forward with checkpoints, recompute and
+// reverse) of 6 plates of 117 x 29, 3 001 steps, 79.6 and 14.2 ms, of 64 plates of
+// 200 x 50, 4 410 steps, 346 and 218 ms.
 //
 // Rows: one warp per stress mode k.  Lanes 8 a .. 8 a + 7 hold the rows of
 // class a (row l + 8 r of the class in lane l, register row r), whose only
 // nonzero columns are those of class a ^ class(k), so all rows of a lane share
 // their right-hand-side loads (four broadcast addresses a warp, one wavefront)
 // and eta_k is a sum within the warp: no barrier before the forces.  A plate
-// without classes (N <= 56) spreads its rows over the 32 lanes.  The rows live
-// in registers (NREG rows) and in tensor memory (NTM rows), used as a
-// thread-private extension of the register file.  Tensor memory rather than
-// shared memory: reading 224 words a thread with their FMAs took 512 cycles
-// per CTA of 256 threads (448 of them the FMAs), from shared memory (LDS.128)
-// 1 800.  Products are packed FMAs (two columns at a time).
+// without classes (N <= 64) spreads its rows over the 32 lanes.  The rows live
+// in tensor memory (NTM rows), used as a thread-private extension of the
+// register file, the others in registers (NREG, checkpoint-free passes) or shared
+// memory (NSM).  Tensor memory rather than shared memory: reading 224 words a
+// thread with their FMAs took 512 cycles per CTA of 256 threads (448 of them the
+// FMAs), from shared memory (LDS.128) 1 800.  Products are packed FMAs (two
+// columns at a time).
 //
 // Exchange: rank r owns the modes [N r / sub, N (r + 1) / sub).  After one CTA
 // barrier every CTA adds its warps' forces and stores each mode's part into
@@ -38,12 +43,24 @@
 // network takes at 13 cycles per warp store: 730 cycles a step for 8 CTAs of
 // 200 modes (1 525 with three right-hand sides).
 //
+// Order of the sums: a gradient's last digits follow the forward states', so
+// the passes with checkpoints keep the streaming kernel's order of every sum
+// (ORD 1, 2).  Products alternate between two chains per row (the halves of the
+// packed FMAs); the streaming kernel starts them anew with each stage of rows, so
+// behind a stage of an odd number of rows they change sides, here a zero column
+// (and a layout of the right-hand sides with that gap).  The force adds one chain
+// per run of stress modes; a CTA stores the runs that end in it as separate parts
+// and hands the one that goes on to the next CTA.
+//
 // Pickups: one warp per chunk of owned modes keeps its terms and sums them every
 // eight steps (with shuffles every step this was 320 cycles of the step's chain);
 // one warp of the last rank adds the chunks' terms.
 //
-// Bound: the packed FMAs (two warps a scheduler) plus the latency of the
-// dependent chain (one barrier, one warp reduction, two exchanges, the update).
+// Bound: the dependent chain of a step (one barrier, one warp reduction, two
+// exchanges of 400 cycles, the update; some 770 instructions a warp at 5 cycles)
+// plus the packed FMAs: 100 x 30 modes on 8 CTAs take 2 490 cycles a step, 620 of
+// them products; 196 x 49 on 7 CTAs 3 860 and 1 740; the fused sweep of 200 x 50
+// on 10 CTAs 11 300 and 4 950.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -67,7 +84,6 @@ constexpr int kPickPitch = 36;               // terms of a step: 4 lanes x 4 ste
 // shared memory over one allocation step more than its 512 columns, so any CTAs
 // that fit an SM by shared memory hold at most 512 columns together.
 constexpr size_t kSmemPerColumn = 430;
-constexpr size_t kResStatic = 1024;          // room for the static shared memory
 constexpr long long kResWait = 1LL << 22;    // bound of every wait (polls)
 
 __device__ __forceinline__ void cluster_sync_all() {
@@ -149,24 +165,33 @@ __host__ __device__ constexpr int rhs_blocks(int R) { return R == 1 ? 1 : R + 1;
 // host.  W warps, kernel row length LM, NO owned modes and segs parts at most.
 struct ResLayout {
     int QB, PS;                 // class block, pickup terms per step
-    int rhs, fp, ke, xch, hs, coef, pick, pst, gacc, vst, end;
+    int LF;                     // right-hand sides of one layout
+    int rhs, fp, ke, xch, car, lp, dp, hs, coef, pick, pst, gacc, vst, end;
 };
 
-__host__ __device__ inline ResLayout res_layout(int R, int W, int LM, int L, int NO, int sub, int segs,
-                                                int nsm) {
+__host__ __device__ inline ResLayout res_layout(int R, int LM, const ResidentParams &Q, int nsm) {
+    const int W = Q.warps, L = Q.L, NO = Q.no_max, sub = Q.max_sub, segs = Q.segs;
     ResLayout o;
     // class blocks 8 banks apart, so that the four classes' accesses do not collide
     o.QB = ((LM + 31) & ~31) + 8;
     o.PS = sub * ((NO + 31) / 32);
     int p = 16;                 // mbarriers, tensor-memory base
-    o.rhs = p;                  // [blocks][4][QB]
-    p += rhs_blocks(R) * 4 * o.QB + 8;   // (a chunk is read past the last block)
+    o.LF = rhs_blocks(R) * 4 * o.QB;
+    o.rhs = p;                  // [layouts][blocks][4][QB]
+    p += Q.lays * o.LF + 8;     // (a chunk is read past the last block)
     o.fp = p;                   // [W][R][4][QB] products of each warp's stress mode
     p += W * R * 4 * o.QB;
     o.ke = p;                   // [W][8] its factors of the forces
     p += W * 8;
     o.xch = p;                  // [2][segs][NO] x (1, 2 or 4 floats): parts of the owned modes
     if (sub > 1) p += 2 * segs * NO * (R == 3 ? 4 : R);
+    p = (p + 3) & ~3;
+    o.car = p;                  // [2][n_max] x (1, 2 or 4 floats): parts begun in the CTA before
+    if (Q.carry) p += 2 * Q.n_max * (R == 3 ? 4 : R);
+    o.lp = p;                   // [layouts - 1][64 W] places of the plate's modes (ints)
+    p += (Q.lays - 1) * 64 * W;
+    o.dp = p;                   // [sub][layouts][NO] places of the owned modes in a peer's layouts,
+    if (Q.lays > 1) p += sub * Q.lays * NO;   // row 0: their number
     p = (p + 3) & ~3;
     o.hs = p;                   // [nsm][L / 4][32 W] x 4: coupling rows (thread-private)
     p += nsm * L * 32 * W;
@@ -323,8 +348,10 @@ __device__ __forceinline__ void dense_row(uint32_t taddr, int L, const float *co
 
 }  // namespace
 
-// SAME: with the streaming kernel's order of every sum, digit for digit.
-template <int R, int NTM, int NSM, int NREG, int LMAX, bool SAME>
+// ORD: the order of the sums.  0: the fastest; 1, 2: the streaming kernel's, digit
+// for digit, 2 also where rows have gaps or a part spans CTAs (kept out of the
+// others: its code alone cost them 3 to 11 % of a step).
+template <int R, int NTM, int NSM, int NREG, int LMAX, int ORD>
 __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q) {
     extern __shared__ __align__(16) float sm[];
     __shared__ ResCta A;
@@ -332,15 +359,17 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     const PlateParams &P = Q.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr bool REV = R >= 2, FWD = R == 1, FUSED = R == 3;
+    constexpr bool SAME = ORD > 0, EXT = ORD == 2;
     constexpr int NR = NTM + NSM + NREG;          // rows of a lane
     constexpr int XF = R == 3 ? 4 : R;            // floats per exchanged entry
     constexpr int QB = ((LMAX + 31) & ~31) + 8;
     const int W = Q.warps, WT = 32 * W;
-    const ResLayout O = res_layout(R, W, LMAX, Q.L, Q.no_max, Q.max_sub, Q.segs, NSM);
+    const ResLayout O = res_layout(R, LMAX, Q, NSM);
     uint64_t *bar_f = reinterpret_cast<uint64_t *>(sm);        // forces of the owned modes
     uint64_t *bar_q = bar_f + 1;                               // new right-hand sides
     uint64_t *bar_y = bar_f + 2;                               // pickup terms (two buffers)
     uint32_t *tbase = reinterpret_cast<uint32_t *>(sm + 8);
+    uint64_t *bar_c = reinterpret_cast<uint64_t *>(sm + 10);   // parts begun in the CTA before
     const long long TM = P.total_modes;
     for (int e = tid; e < (int)(sizeof(ResCta) / 4); e += blockDim.x)
         reinterpret_cast<int *>(&A)[e] = reinterpret_cast<const int *>(Q.ctas + blockIdx.x)[e];
@@ -365,15 +394,19 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     const int m0 = (int)((long long)N * rank / sub);
     const int no = (int)((long long)N * (rank + 1) / sub) - m0;   // owned modes
     const int C = max((no + 31) / 32, 1);         // chunks of 32 owned modes
+    const int lays = EXT && used ? A.lays : 1;
+    const bool more_lays = EXT && Q.lays > 1;
     if (tid == 0) {
         bar_init(bar_f, 1);
         bar_init(bar_q, sub > 1 ? 1 : C);
         bar_init(bar_y, 1);
         bar_init(bar_y + 1, 1);
+        bar_init(bar_c, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (sub > 1) {
             bar_expect_tx(bar_f, (uint32_t)(A.segs_all * no * XF * 4));
-            bar_expect_tx(bar_q, (uint32_t)(N * 4 * (FUSED ? 2 : 1)));
+            bar_expect_tx(bar_q, (uint32_t)(N * 4 * (FUSED ? 2 : 1) * lays));
+            if (EXT && (A.carry & 1)) bar_expect_tx(bar_c, (uint32_t)(N * XF * 4));
         }
     }
     // class row of a user-order mode, and its place in a right-hand-side block
@@ -383,7 +416,13 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const int a = (row >= d.ocls[1]) + (row >= d.ocls[2]) + (row >= d.ocls[3]);
         return a * QB + row - pick4r(d.ocls, a);
     };
+    // the same in layout l of a CTA
+    auto lay_pos = [&](const ResCta &c, int l, int pos) {
+        const int a = pos / QB, i = pos - a * QB, g = c.gap[l - 1][a];
+        return l * O.LF + pos + (g > 0 ? i / g : 0);
+    };
     float *const rhs = sm + O.rhs;
+    int *const lp = reinterpret_cast<int *>(sm + O.lp) + tid, *const dp = reinterpret_cast<int *>(sm + O.dp);
     constexpr int bw = 2 * 4 * QB, br = 3 * 4 * QB;   // blocks: q (twice in reverse), w, q'
     const int rsteps = FUSED ? P.rev_steps : P.steps;
     const float *rec0 = P.state_io;                            // incoming forward state
@@ -410,14 +449,28 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                                     (uint32_t)(A.base + own));
                 mbar[h] = peer_addr(su32(bar_f), (uint32_t)(A.base + own));
             }
-            if (FWD) rhs[mp[h]] = rec0[m];
-            if (REV) {
-                rhs[mp[h]] = P.seg_q[(long long)(rsteps - 1) * TM + m];
-                rhs[bw + mp[h]] = P.coef.r[m] * P.adj[m];
+            for (int l = 0; l < lays; ++l) {
+                const int at = l == 0 ? mp[h] : lay_pos(A, l, mp[h]);
+                if (l > 0) lp[((l - 1) * 2 + h) * WT] = at;
+                if (FWD) rhs[at] = rec0[m];
+                if (REV) {
+                    rhs[at] = P.seg_q[(long long)(rsteps - 1) * TM + m];
+                    rhs[bw + at] = P.coef.r[m] * P.adj[m];
+                }
+                if (FUSED) rhs[br + at] = rec0[m];
             }
-            if (FUSED) rhs[br + mp[h]] = rec0[m];
         }
     }
+    // the owned modes' places in every CTA of the plate
+    if (more_lays && used)
+        for (int e = tid; e < sub * no; e += WT) {
+            const int pr = e / no, oi = e - pr * no;
+            const ResCta &c = Q.ctas[(int)blockIdx.x - rank + pr];
+            const int pos = class_pos(m0 + oi);
+            int *const row = dp + pr * Q.lays * Q.no_max + oi;
+            row[0] = c.lays;
+            for (int l = 1; l < c.lays; ++l) row[l * Q.no_max] = lay_pos(c, l, pos) - pos;
+        }
     __syncthreads();
     cluster_sync_all();      // every peer's barriers exist before the first store
 
@@ -439,6 +492,8 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             // column the streaming kernel sums (H need not be symmetric to the last bit)
             long long off = 0;
             int n = 0, stride = 0;
+            const int lay = EXT && kon ? A.lay_of >> (4 * warp) & 15 : 0;
+            int gap = 0;                                        // a zero column after every gap
             if (kon) {
                 kap = P.kappa[d.k_off + kl];
                 if (REV) {
@@ -450,6 +505,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     kc = K.c;
                     const int w = (ncl + 3) & ~3;
                     n = pick4r(d.ncls, ra ^ kc);
+                    if (lay > 0) gap = A.gap[lay - 1][ra ^ kc];
                     long long sb = 0;
                     for (int a2 = 0; a2 < (ra ^ kc); ++a2)
                         sb += (long long)pick4r(d.ncls, a2) * K.mc *
@@ -462,14 +518,17 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     stride = d.Npad;
                 }
             }
+            auto element = [&](int row, int p) {
+                const int s = gap > 0 ? p / (gap + 1) : 0, j = p - s;
+                const bool in = row < ncl && j < n && (gap == 0 || p - s * (gap + 1) < gap);
+                return in ? P.H[off + (long long)j * stride + row] : 0.f;
+            };
             for (int s = 0; s < NTM; ++s) {
                 const int row = l0 + gl * s;
                 for (int j = 0; j < L; j += 8) {
                     float v[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        v[e] = (row < ncl && j + e < n) ? P.H[off + (long long)(j + e) * stride + row]
-                                                        : 0.f;
+                    for (int e = 0; e < 8; ++e) v[e] = element(row, j + e);
                     __syncwarp();
                     tmem_st8(taddr + (uint32_t)(j * NTM + 8 * s), v);
                 }
@@ -478,9 +537,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             for (int s = 0; s < NSM; ++s) {
                 const int row = l0 + gl * (NTM + s);
                 for (int j = 0; j < L; ++j)
-                    if (row < ncl && j < n)
-                        reinterpret_cast<float *>(hsm + (s * (L / 4) + j / 4) * WT)[j & 3] =
-                            P.H[off + (long long)j * stride + row];
+                    reinterpret_cast<float *>(hsm + (s * (L / 4) + j / 4) * WT)[j & 3] = element(row, j);
             }
 #pragma unroll
             for (int s = 0; s < NREG; ++s) {
@@ -489,13 +546,13 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 for (int j = 0; j < LMAX; j += 2) {
                     float v[2];
 #pragma unroll
-                    for (int e = 0; e < 2; ++e)
-                        v[e] = (row < ncl && j + e < n) ? P.H[off + (long long)(j + e) * stride + row] : 0.f;
+                    for (int e = 0; e < 2; ++e) v[e] = element(row, j + e);
                     hreg[s][j / 2] = pack2(__float_as_uint(v[0]), __float_as_uint(v[1]));
                 }
             }
         }
-        const float *const qcol = rhs + (cls ? (ra ^ kc) * QB : 0);
+        const float *const qcol = rhs + (cls ? (ra ^ kc) * QB : 0) +
+                                  (EXT && kon ? (int)(A.lay_of >> (4 * warp) & 15) * O.LF : 0);
         const float *const qrow = rhs + ra * QB + l0;
         float *const fpw = sm + O.fp + warp * R * 4 * QB, *const fp = fpw + ra * QB + l0;
         float *const kew = sm + O.ke;
@@ -600,6 +657,15 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                         copy4(nb + mp[h], nq_src + h * WT);
                     else
                         nb[mp[h]] = 0.f;
+                    if (more_lays)
+#pragma unroll 1
+                      for (int l = 0; l < lays - 1; ++l) {
+                        const int at = lp[(l * 2 + h) * WT];
+                        if (it < rsteps)
+                            copy4(nb + at, nq_src + h * WT);
+                        else
+                            nb[at] = 0.f;
+                    }
                 }
             nq_src -= TM;
         };
@@ -607,7 +673,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         float *px = (REV && P.xe && (d.has_dir || P.xe_all))
                         ? P.xe + (long long)(rsteps - 1) * 2 * P.total_k + d.k_off + kl : nullptr;
         const bool st_x = px && kon && lane == 0;
-        const uint32_t tx_f = (uint32_t)(A.segs_all * no * XF * 4), tx_q = (uint32_t)(N * 4 * (FUSED ? 2 : 1));
+        const uint32_t tx_f = (uint32_t)(A.segs_all * no * XF * 4), tx_q = (uint32_t)(N * 4 * (FUSED ? 2 : 1) * lays);
         const uint32_t q_dst = su32(rhs + cpos + (REV ? bw : 0)), q_bar = su32(bar_q);
         const uint32_t q_dst0 = sub > 1 ? peer_addr(q_dst, (uint32_t)(A.base + min(rep, sub - 1))) : 0u;
         const uint32_t q_bar0 = sub > 1 ? peer_addr(q_bar, (uint32_t)(A.base + min(rep, sub - 1))) : 0u;
@@ -632,6 +698,9 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         }
         bool bad = false;
         const int seg_last = A.seg_last, segs_all = A.segs_all;
+        const int carry = EXT ? A.carry : 0, nw = carry & 2 ? A.tail : nk;
+        const uint32_t c_dst = carry & 2 ? peer_addr(su32(sm + O.car) + (uint32_t)(tid * XF * 4), (uint32_t)(A.base + rank + 1)) : 0u;
+        const uint32_t c_bar = carry & 2 ? peer_addr(su32(bar_c), (uint32_t)(A.base + rank + 1)) : 0u;
         const unsigned long long new_item = A.new_item;
         // every part a partial sum of its own, or one row of them: one chain (with the
         // selects of the general case 24 parts took 1 230 cycles)
@@ -758,11 +827,19 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             // (emit is called with each); the plate's force adds its parts in order,
             // item by item of the streaming kernel's work split where the plan asks
             // for its rounding (new_item), else all in one row.
-            auto parts = [&](int pos, auto emit) {
+            auto add_term = [&](int w, const float *p, float (&f)[R]) {
+                const float4 k4 = *reinterpret_cast<const float4 *>(kew + 8 * w);
+                const float uu = p[0];
+                if constexpr (FWD) {
+                    f[0] = fmaf(k4.x, uu, f[0]);
+                } else {
+                    f[1] = fmaf(k4.x, uu, f[1]);                                        // f(q^n)
+                    f[0] = fmaf(k4.y, fmaf(k4.z, uu, k4.w * p[4 * QB]), f[0]);          // J w
+                }
+                if constexpr (FUSED) f[2] = fmaf(kew[8 * w + 4], p[8 * QB], f[2]);
+            };
+            auto parts = [&](int pos, float (&f)[R], auto emit) {      // f: where the first part stands
                 const float *p = sm + O.fp + pos;
-                float f[R];
-#pragma unroll
-                for (int x = 0; x < R; ++x) f[x] = 0.f;
                 if constexpr (!SAME) {
 #pragma unroll
                     for (int w = 0; w < kResMaxWarps; ++w) f[0] += w < nk ? p[w * 4 * QB] : 0.f;
@@ -772,16 +849,8 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 int seg = 0;
 #pragma unroll
                 for (int w = 0; w < kResMaxWarps; ++w, p += R * 4 * QB) {
-                    if (w >= nk) break;
-                    const float4 k4 = *reinterpret_cast<const float4 *>(kew + 8 * w);
-                    const float uu = p[0];
-                    if constexpr (FWD) {
-                        f[0] = fmaf(k4.x, uu, f[0]);
-                    } else {
-                        f[1] = fmaf(k4.x, uu, f[1]);                                        // f(q^n)
-                        f[0] = fmaf(k4.y, fmaf(k4.z, uu, k4.w * p[4 * QB]), f[0]);          // J w
-                    }
-                    if constexpr (FUSED) f[2] = fmaf(kew[8 * w + 4], p[8 * QB], f[2]);
+                    if (w >= nw) break;
+                    add_term(w, p, f);
                     if (seg_last >> w & 1) {
                         emit(seg, f);
 #pragma unroll
@@ -789,6 +858,21 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                         ++seg;
                     }
                 }
+            };
+            auto push_part = [&](uint32_t to, uint32_t bar, const float (&f)[R]) {
+                if constexpr (R == 1) push1(to, bar, f[0]);
+                if constexpr (R == 2) push2(to, bar, f[0], f[R - 1]);
+                if constexpr (R == 3) push4(to, bar, f[0], f[R > 1 ? 1 : 0], f[R - 1]);
+            };
+            // a part that began in the CTA before goes on from there
+            auto carried = [&](int h, float (&f)[R]) {
+                const float *x = sm + O.car + (buf * Q.n_max + tid + h * WT) * XF;
+#pragma unroll
+                for (int y = 0; y < R; ++y) f[y] = x[y];
+            };
+            auto take_carry = [&]() {
+                if (32 * warp < N) wait(bar_c, (uint32_t)buf);
+                if (tid == 0 && it + 1 < P.steps) bar_expect_tx(bar_c, (uint32_t)(N * XF * 4));
             };
             float F[R], item[R];
 #pragma unroll
@@ -816,16 +900,35 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 }
             };
             if (sub > 1) {
+                if (EXT && carry != 0) {
+                    // the part that ends in a later CTA first: the next one waits for it
+                    const bool through = carry == 3 && nw == 0;
+                    if (through) take_carry();
+                    if (carry & 2) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (!mon[h]) continue;
+                            float f[R];
+#pragma unroll
+                            for (int x = 0; x < R; ++x) f[x] = 0.f;
+                            if (through) carried(h, f);
+                            const float *p = sm + O.fp + mp[h] + nw * R * 4 * QB;
+#pragma unroll 2
+                            for (int w = nw; w < nk; ++w, p += R * 4 * QB) add_term(w, p, f);
+                            push_part(c_dst + (uint32_t)((buf * Q.n_max + h * WT) * XF * 4), c_bar, f);
+                        }
+                    }
+                    if ((carry & 1) && !through) take_carry();
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (!mon[h]) continue;
                     const uint32_t dst = mdst[h] + (buf ? xbuf : 0u);
-                    parts(mp[h], [&](int seg, const float (&f)[R]) {
-                        const uint32_t to = dst + seg * sbuf;
-                        if constexpr (R == 1) push1(to, mbar[h], f[0]);
-                        if constexpr (R == 2) push2(to, mbar[h], f[0], f[R - 1]);
-                        if constexpr (R == 3) push4(to, mbar[h], f[0], f[R > 1 ? 1 : 0], f[R - 1]);
-                    });
+                    float f[R];
+#pragma unroll
+                    for (int x = 0; x < R; ++x) f[x] = 0.f;
+                    if (EXT && (carry & 1)) carried(h, f);
+                    parts(mp[h], f, [&](int seg, const float (&v)[R]) { push_part(dst + seg * sbuf, mbar[h], v); });
                 }
                 if (upd) {
                     wait(bar_f, (uint32_t)buf);
@@ -848,7 +951,10 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     }
                 }
             } else if (on) {
-                parts(cpos, [&](int seg, const float (&f)[R]) { add_part(seg, f); });
+                float f[R];
+#pragma unroll
+                for (int x = 0; x < R; ++x) f[x] = 0.f;
+                parts(cpos, f, [&](int seg, const float (&v)[R]) { add_part(seg, v); });
             }
 #pragma unroll
             for (int x = 0; x < R; ++x) F[x] += item[x];
@@ -869,20 +975,38 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                             fmaf(bcf, FWD ? e : er, -F[FUSED ? 2 : 0]));
                 if (sub > 1) {
                     if (on && rep < sub) {
-                        push1(q_dst0, q_bar0, REV ? wv : y0);
-                        if (FUSED) push1(q_dst0 + (uint32_t)((br - bw) * 4), q_bar0, y0);
-                        for (int pr = rep + reps; pr < sub; pr += reps) {
-                            const uint32_t qa = peer_addr(q_dst, (uint32_t)(A.base + pr));
-                            const uint32_t ba = peer_addr(q_bar, (uint32_t)(A.base + pr));
-                            push1(qa, ba, REV ? wv : y0);
+                        const float x = REV ? wv : y0;
+                        auto push_q = [&](uint32_t qa, uint32_t ba) {
+                            push1(qa, ba, x);
                             if (FUSED) push1(qa + (uint32_t)((br - bw) * 4), ba, y0);
-                        }
+                        };
+                        auto push_lays = [&](int pr, uint32_t qa, uint32_t ba) {
+                            push_q(qa, ba);
+                            if (more_lays) {
+                                const int *row = dp + pr * Q.lays * Q.no_max + oi;
+                                const int nl = row[0];
+#pragma unroll 1
+                                for (int l = 1; l < nl; ++l) push_q(qa + 4u * row[l * Q.no_max], ba);
+                            }
+                        };
+                        push_lays(rep, q_dst0, q_bar0);
+                        for (int pr = rep + reps; pr < sub; pr += reps)
+                            push_lays(pr, peer_addr(q_dst, (uint32_t)(A.base + pr)),
+                                      peer_addr(q_bar, (uint32_t)(A.base + pr)));
                     }
                 } else {
                     if (on) {
                         if (FWD) rhs[cpos] = y0;
                         if (REV) rhs[bw + cpos] = wv;
                         if (FUSED) rhs[br + cpos] = y0;
+                        if (more_lays)
+#pragma unroll 1
+                            for (int l = 1; l < lays; ++l) {
+                                const int at = cpos + dp[l * Q.no_max + oi];
+                                if (FWD) rhs[at] = y0;
+                                if (REV) rhs[bw + at] = wv;
+                                if (FUSED) rhs[br + at] = y0;
+                            }
                     }
                     __syncwarp();
                     if (lane == 0) bar_arrive(bar_q);
@@ -1022,37 +1146,41 @@ namespace {
 // Kernel variants by longest row: a lane's rows in tensor memory (256 words a
 // thread with more than four warps, else 512); of the others, those in registers
 // (kernels without a reverse pass or checkpoints, NREG) and in shared memory.
-constexpr int kVarLen[kResVariants] = {16, 24, 32, 40, 48, 56, 64};
-constexpr int kVarTm[kResVariants] = {2, 2, 4, 4, 4, 4, 6};
-constexpr int kVarSm[kResVariants] = {0, 1, 0, 1, 2, 3, 2};
-constexpr int kVarReg[kResVariants] = {0, 1, 0, 1, 2, 2, 0};
+constexpr int kVarLen[kResVariants] = {16, 24, 32, 40, 48, 56, 64, 64};
+constexpr int kVarTm[kResVariants] = {2, 2, 4, 4, 4, 4, 4, 6};
+constexpr int kVarSm[kResVariants] = {0, 1, 0, 1, 2, 3, 3, 2};
+constexpr int kVarReg[kResVariants] = {0, 1, 0, 1, 2, 2, 0, 0};
 int var_warps(int v) { return kVarTm[v] * kVarLen[v] > 256 ? 4 : kResMaxWarps; }
 int var_sm(int v, bool same) { return kVarSm[v] - (same ? 0 : kVarReg[v]); }
 
-template <int R, bool SAME, int V>
+template <int R, int ORD, int V>
 const void *res_fn_v() {
-    constexpr int REG = SAME ? 0 : kVarReg[V];
+    constexpr int REG = ORD > 0 ? 0 : kVarReg[V];
     return reinterpret_cast<const void *>(
-        resident_kernel<R, kVarTm[V], kVarSm[V] - REG, REG, kVarLen[V], SAME>);
+        resident_kernel<R, kVarTm[V], kVarSm[V] - REG, REG, kVarLen[V], ORD>);
 }
-template <int R, bool SAME>
+
+template <int R, int ORD>
 const void *res_fn_r(int v) {
     switch (v) {
-        case 0: return res_fn_v<R, SAME, 0>();
-        case 1: return res_fn_v<R, SAME, 1>();
-        case 2: return res_fn_v<R, SAME, 2>();
-        case 3: return res_fn_v<R, SAME, 3>();
-        case 4: return res_fn_v<R, SAME, 4>();
-        case 5: return res_fn_v<R, SAME, 5>();
-        default: return res_fn_v<R, SAME, 6>();
+        case 0: return res_fn_v<R, ORD, 0>();
+        case 1: return res_fn_v<R, ORD, 1>();
+        case 2: return res_fn_v<R, ORD, 2>();
+        case 3: return res_fn_v<R, ORD, 3>();
+        case 4: return res_fn_v<R, ORD, 4>();
+        case 5: return res_fn_v<R, ORD, 5>();
+        case 6: return res_fn_v<R, ORD, 6>();
+        default: return res_fn_v<R, ORD, 7>();
     }
 }
 
-// Right-hand sides r; same: with the streaming kernel's order of the sums (the
-// passes with a reverse have no other).
-const void *res_fn(int r, int v, bool same) {
-    if (r == 1) return same ? res_fn_r<1, true>(v) : res_fn_r<1, false>(v);
-    return r == 2 ? res_fn_r<2, true>(v) : res_fn_r<3, true>(v);
+// The kernel of r right-hand sides (passes with a reverse keep the streaming
+// kernel's order, they have no other).
+const void *res_fn(int r, const ResidentParams &Q) {
+    const bool ext = Q.lays > 1 || Q.carry;
+    if (r == 1) return !Q.same ? res_fn_r<1, 0>(Q.variant) : (ext ? res_fn_r<1, 2>(Q.variant) : res_fn_r<1, 1>(Q.variant));
+    if (r == 2) return ext ? res_fn_r<2, 2>(Q.variant) : res_fn_r<2, 1>(Q.variant);
+    return ext ? res_fn_r<3, 2>(Q.variant) : res_fn_r<3, 1>(Q.variant);
 }
 
 void res_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *at, int grid, int cs, int threads,
@@ -1094,8 +1222,7 @@ int resident_columns(int variant, int L, int warps) {
 // fit an SM together (of this or another launch) never wait for each other's
 // columns: a CTA whose cluster peers wait must not block on an allocation.
 size_t resident_smem(int R, const ResidentParams &Q) {
-    const ResLayout o = res_layout(R, Q.warps, kVarLen[Q.variant], Q.L, Q.no_max, Q.max_sub,
-                                    Q.segs, var_sm(Q.variant, Q.same));
+    const ResLayout o = res_layout(R, kVarLen[Q.variant], Q, var_sm(Q.variant, Q.same));
     return std::max(sizeof(float) * (size_t)o.end, (size_t)Q.tcols * kSmemPerColumn);
 }
 
@@ -1104,7 +1231,7 @@ size_t resident_smem(int R, const ResidentParams &Q) {
 cudaError_t resident_check(int cs, const ResidentParams &Q, size_t smem_optin, int *fit) {
     *fit = 1 << 30;
     for (int r = 1; r <= (Q.same ? 3 : 1); ++r) {
-        const void *fn = res_fn(r, Q.variant, Q.same);
+        const void *fn = res_fn(r, Q);
         const size_t smem = resident_smem(r, Q);
         if (smem + kResStatic > smem_optin) {
             *fit = 0;
@@ -1135,7 +1262,7 @@ cudaError_t launch_resident(int R, const ResidentParams &Q, int grid, int cs, si
     res_config(cfg, at, grid, cs, 32 * Q.warps, smem, s);
     ResidentParams q = Q;
     void *args[] = {&q};
-    return cudaLaunchKernelExC(&cfg, res_fn(R, Q.variant, Q.same), args);
+    return cudaLaunchKernelExC(&cfg, res_fn(R, Q), args);
 }
 
 }  // namespace mdx

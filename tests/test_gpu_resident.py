@@ -100,3 +100,29 @@ def test_more_plates_than_clusters():
     for i in (0, 1, 2, 3, 90, 91, 178, 179):
         one = modal.Simulator([plans[i]]).simulate(steps)["audio"]
         assert rel(r["audio"][i].cpu().numpy(), one[0].cpu().numpy()) <= 1e-5, i
+
+
+@pytest.mark.parametrize("count,n,m", [(20, 150, 37), (32, 150, 37), (24, 200, 50), (48, 130, 32)])
+def test_sums_that_span_ctas(count, n, m):
+    """Many large plates: the streaming kernel sums more stress modes in a row
+    than a CTA holds (parts of the force pass from CTA to CTA) and its rows change
+    sides of their two chains (rows with gaps).  Gradients digit for digit."""
+    steps, K = 40, 16
+    oi, fs = _plate(n, m, steps)
+    plans = []
+    for i in range(count):
+        d = to_plan(oi, fs)
+        d["kappa"] = oi.kappa * (0.5 + i / count)
+        plans.append(d)
+    ybar = np.random.default_rng(n).normal(size=(count, steps))
+    yb = torch.tensor(ybar, dtype=torch.float32, device="cuda")
+    grads = []
+    for flags in (0, 16):          # 16: the streaming kernel
+        sim = modal.Simulator(plans, debug_flags=flags)
+        r = sim.simulate(steps, K=K)
+        g = sim.grad(steps, yb, K, r["ckpt"], want_status=True)
+        torch.cuda.synchronize()
+        assert (g["status"].cpu().numpy() == 0).all()
+        grads.append(g)
+    for k in grads[0]:
+        assert torch.equal(grads[0][k], grads[1][k]), k
