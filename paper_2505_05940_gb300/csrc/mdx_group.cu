@@ -24,15 +24,15 @@
 // whose error is about 2^-21 of |H||Q| (the dropped H_lo Q_lo and the TF32
 // rounding of the remainders), the accuracy of the FP32 path.
 //
-// Execution (one 256-thread CTA per SM, cooperative launch, all steps in one
+// Execution (one 320-thread CTA per SM, cooperative launch, all steps in one
 // launch).  Each CTA holds a contiguous range of one group's stress modes:
 //   warp 0  producer: streams the CTA's coupling tiles from global memory in
 //           16-column chunks (cp.async.bulk into a ring of 8 KB stages,
 //           mbarrier transaction counts); the tiles were laid out at plan time
 //           as the MMA's shared-memory image (8-row x 16-byte core matrices,
 //           K-major, no swizzle), so one bulk copy moves one chunk;
-//   warps 2-3 convert each chunk in place into its TF32 high part plus a
-//           remainder stage;
+//   warps 2-3 and 8-9 convert each chunk in place into its TF32 high part plus
+//           a remainder stage;
 //   warp 1  issues the MMAs (one thread) into tensor memory: per tile a
 //           [128 rows x Bp plates] FP32 accumulator;
 //   warps 4-7 (epilogue, one tensor-memory lane quarter each): eta from the
@@ -44,6 +44,16 @@
 // its audio sample and its new q, and arrives at the second, on which all wait
 // before they fetch the next step's Q image.  (One counter for both would let
 // CTAs without a plate run ahead into the owners' count.)
+//
+// Bound: 160 plates on 4 geometries (20 to 400 modes, 24 plates and two stress
+// modes of 400 x 400 on a CTA), cycles of the longest chain of a step: Q image 2 000, MMAs
+// 25 400 (per chunk 460, of them some 440 shared-memory wavefronts: the bulk
+// copy, the conversion and the operands), eta and forces of the last unit 5 500,
+// partial forces 3 400, owners 12 900.  Before, of 102 000: eta 23 000 (the
+// Q image's rows lie eight lanes to a bank; the rows' states now sit in
+// tensor memory), owners 18 000 to 31 000 (one mode at a time, the plates' table
+// searched in global memory), partial forces 12 000 (64-bit addresses).  Together
+// 95 us a step at first, 53 with the gathers in batches, 38 now.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -74,9 +84,10 @@ __device__ __forceinline__ unsigned ld_acq(const unsigned *p) {
     return v;
 }
 
-__device__ __forceinline__ float ldcg(const float *p) {
-    float v;
-    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+__device__ __forceinline__ float4 ldcg4(const float *p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 
@@ -126,7 +137,13 @@ struct Ctrl {
     int pad[2];
     float eta_red[4][kGrpMaxB];
     float ke[kGrpMaxB];
-    float pick[2][8];
+    // the plates this CTA steps: place in the group, instance, modes
+    int n_own;
+    struct {
+        int b, inst, N, pad;
+        long long mode_off;
+        float ys[4], ye[4];   // pickup terms of the epilogue warps
+    } own[kGrpMaxB];
 };
 
 }  // namespace
@@ -153,7 +170,7 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         for (int s = 0; s < R; ++s) {
             bar_init(&C.full[s], 1);
             bar_init(&C.empty[s], 1);
-            bar_init(&C.conv[s], 2);
+            bar_init(&C.conv[s], kGrpConvWarps);
         }
         bar_init(&C.qready, 1);
         for (int b = 0; b < 2; ++b) {
@@ -162,10 +179,24 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         }
         bar_init(&C.drain, 1);
         C.fail = 0;
+        C.n_own = 0;
+        for (int b = 0; b < G.B; ++b) {
+            const GrpPlate pl = P.plates[G.plate0 + b];
+            if (pl.owner != cta) continue;
+            auto &o = C.own[C.n_own++];
+            o.b = b;
+            o.inst = pl.inst;
+            o.N = P.inst[pl.inst].N;
+            o.mode_off = P.inst[pl.inst].mode_off;
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int x = tid; x < (u1 - u0) * (int)(sizeof(GrpUnit) / 4); x += kGrpThreads)
         reinterpret_cast<int *>(units)[x] = reinterpret_cast<const int *>(P.units + u0)[x];
+    // user mode of each class-order position of the group
+    unsigned short *inv = reinterpret_cast<unsigned short *>(smem + P.inv_off);
+    for (int j = tid; j < P.groups[gi].N; j += kGrpThreads)
+        inv[P.gpos[P.groups[gi].gpos_off + j]] = (unsigned short)j;
     if (warp == 1) {
         // the whole tensor memory of the SM (one CTA per SM)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
@@ -226,6 +257,9 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         // ============================================================ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = idesc_tf32(128, Bp);
+            // the ring's first stage; 8-row groups are kGrpChunk / 4 core matrices apart
+            const uint64_t ad0 = smem_desc(su32(ring), 128u, (kGrpChunk / 4) * 128u);
+            const uint64_t ald0 = smem_desc(su32(lo), 128u, (kGrpChunk / 4) * 128u);
             int slot = 0;
             uint32_t ph = 0;
             long long ucount = 0;
@@ -249,31 +283,29 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                         if (U.off[t] < 0) continue;
                         const int a = U.c ^ G.tile_sb[t];
                         const int kp = G.kpad[a];
+                        // (built once per tile, then advanced: descriptors built for
+                        // every MMA by the one issuing thread took 500 cycles a chunk)
                         const uint32_t sbo_q = (uint32_t)(kp / 4) * 128u;
-                        const uint32_t qa = su32(qimg + G.qoff[a]);
-                        const uint32_t qla = su32(qimg + G.qoff[a] + Bp * kp);
+                        uint64_t qd = smem_desc(su32(qimg + G.qoff[a]), 128u, sbo_q);
+                        uint64_t qld = smem_desc(su32(qimg + G.qoff[a] + Bp * kp), 128u, sbo_q);
                         const uint32_t d = tmem + (uint32_t)((buf * nt + t) * Bp);
                         for (int j = 0; j < kp / kGrpChunk; ++j) {
-                            if (!bar_spin(&C.conv[slot], ph, P.wait_limit, gabort)) {
+                            if (!bar_try(&C.conv[slot], ph) &&
+                                !bar_wait(&C.conv[slot], ph, P.wait_limit, gabort)) {
                                 ok = false;
                                 break;
                             }
                             tc_fence_after();
-                            const uint32_t as = su32(ring + (size_t)slot * (kGrpStageBytes / 4));
-                            const uint32_t als = su32(lo + (size_t)slot * (kGrpStageBytes / 4));
-                            // K-steps of 8 columns (two core matrices) within the chunk;
-                            // 8-row groups are kGrpChunk / 4 core matrices apart
-                            constexpr uint32_t sbo_a = (kGrpChunk / 4) * 128u;
+                            // K-steps of 8 columns (two core matrices, 256 bytes) within the chunk
+                            const uint64_t so = (uint64_t)(slot * (kGrpStageBytes >> 4));
 #pragma unroll
                             for (int kk = 0; kk < kGrpChunk / 8; ++kk) {
-                                const uint64_t ad = smem_desc(as + kk * 256u, 128u, sbo_a);
-                                const uint64_t ald = smem_desc(als + kk * 256u, 128u, sbo_a);
-                                const uint32_t qo = (uint32_t)(j * (kGrpChunk / 4) + kk * 2) * 128u;
-                                const uint64_t qd = smem_desc(qa + qo, 128u, sbo_q);
-                                const uint64_t qld = smem_desc(qla + qo, 128u, sbo_q);
+                                const uint64_t ad = ad0 + so + kk * 16u, ald = ald0 + so + kk * 16u;
                                 mma_tf32(d, ad, qd, idesc, (j | kk) ? 1u : 0u);
                                 mma_tf32(d, ad, qld, idesc, 1u);
                                 mma_tf32(d, ald, qd, idesc, 1u);
+                                qd += 16u;
+                                qld += 16u;
                             }
                             mma_issued = true;
                             mma_commit(&C.empty[slot]);
@@ -298,9 +330,9 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                 }
             }
         }
-    } else if (warp < 4) {
+    } else if (warp < 4 || warp >= 8) {
         // ============================================================ converters
-        const int ct = tid - 64;   // 0..63
+        const int ct = 32 * (warp < 4 ? warp - 2 : warp - 6) + lane;
         int slot = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -313,23 +345,21 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     const int r8 = (G.tile_rows[t] + 7) & ~7;
                     const int n4 = r8 * kGrpChunk / 4;
                     for (int j = 0; j < G.kpad[a] / kGrpChunk; ++j) {
-                        if (!bar_spin(&C.full[slot], ph, P.wait_limit, gabort)) {
+                        if (!bar_try(&C.full[slot], ph) &&
+                            !bar_wait(&C.full[slot], ph, P.wait_limit, gabort)) {
                             ok = false;
                             break;
                         }
                         float4 *x = reinterpret_cast<float4 *>(ring + (size_t)slot * (kGrpStageBytes / 4));
                         float4 *y = reinterpret_cast<float4 *>(lo + (size_t)slot * (kGrpStageBytes / 4));
-                        // the thread's share of the stage (eight float4 at most) is
-                        // loaded before the first store: one load, store pair after
-                        // the other made this conversion the pipeline's slowest stage
-                        constexpr int kV = kGrpStageBytes / 16 / 64;
+                        constexpr int kCT = 32 * kGrpConvWarps, kV = kGrpStageBytes / 16 / kCT;
                         float4 v[kV];
 #pragma unroll
                         for (int q = 0; q < kV; ++q)
-                            if (ct + 64 * q < n4) v[q] = x[ct + 64 * q];
+                            if (ct + kCT * q < n4) v[q] = x[ct + kCT * q];
 #pragma unroll
                         for (int q = 0; q < kV; ++q) {
-                            if (ct + 64 * q >= n4) continue;
+                            if (ct + kCT * q >= n4) continue;
                             float4 h, l;
                             h.x = tf32_hi(v[q].x);
                             h.y = tf32_hi(v[q].y);
@@ -339,8 +369,8 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                             l.y = v[q].y - h.y;
                             l.z = v[q].z - h.z;
                             l.w = v[q].w - h.w;
-                            x[ct + 64 * q] = h;
-                            y[ct + 64 * q] = l;
+                            x[ct + kCT * q] = h;
+                            y[ct + kCT * q] = l;
                         }
                         fence_async_smem();
                         __syncwarp();
@@ -364,23 +394,22 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
         const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
         const unsigned nct = (unsigned)G.n_ctas;
         const int fcol = 2 * nt * Bp;          // first column of the force accumulators
+        // q of this thread's rows in tensor memory, if there is room for it
+        const int qcol = 3 * nt * Bp;
+        const bool qrows = 4 * nt * Bp <= 512;
         const int slot_in_group = cta - G.cta0;
         // arrivals of every CTA with its partial forces, and of the owners with new q
         unsigned *cnt_f = P.counters + 2 * gi, *cnt_q = cnt_f + 1;
         const long long TM = P.total_modes;
         long long ucount = 0;
         bool ok = true;
-        bool owner = false;
-        for (int b = 0; b < G.B; ++b) owner = owner || (P.plates[G.plate0 + b].owner == cta);
+        const int n_own = C.n_own;
+        const bool owner = n_own > 0;
         // owners: initial q (class order) of the plates this CTA steps
-        for (int b = 0; b < G.B; ++b) {
-            const GrpPlate pl = P.plates[G.plate0 + b];
-            if (pl.owner != cta) continue;
-            const InstDesc d = P.inst[pl.inst];
-            for (int j = et; j < d.N; j += 128)
-                q_image_put(P.qbuf + G.qbuf_off, G, b, P.gpos[G.gpos_off + j],
-                            P.state_io[d.mode_off + j]);
-        }
+        for (int x = 0; x < n_own; ++x)
+            for (int j = et; j < C.own[x].N; j += 128)
+                q_image_put(P.qbuf + G.qbuf_off, G, C.own[x].b, P.gpos[G.gpos_off + j],
+                            P.state_io[C.own[x].mode_off + j]);
         epi_bar();
         if (et == 0 && owner) {
             __threadfence();
@@ -432,6 +461,42 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                         tmem_st16(tmem + lane_base + (uint32_t)(fcol + t * Bp + cb), z);
                 tmem_wait_st();
             }
+            // ---- q of the thread's rows: the image's rows lie 8 lanes to a bank, so
+            // each of the eight lanes groups starts at another plate and rotates the
+            // values into place
+            if (qrows)
+                for (int t = 0; t < nt; ++t) {
+                    const int sb = G.tile_sb[t], kp = G.kpad[sb];
+                    const bool in = r < G.tile_rows[t];
+                    const int p = G.tile_r0[t] + r, m = (lane >> 2) & 7;
+                    const float *qh = qimg + G.qoff[sb] + ((p >> 2) << 5) + (p & 3);
+                    const float *ql = qh + Bp * kp;
+                    for (int cb = 0; cb < Bp; cb += 16) {
+                        float y[16];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int o = ((cb >> 3) + h) * (kp >> 2) * 32;
+                            float x[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                const int e = o + (((i + m) & 7) << 2);
+                                x[i] = in ? qh[e] + ql[e] : 0.f;
+                            }
+#pragma unroll
+                            for (int sh = 1; sh < 8; sh <<= 1) {
+                                float z[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) z[i] = (m & sh) ? x[(i - sh) & 7] : x[i];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) x[i] = z[i];
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) y[8 * h + i] = x[i];
+                        }
+                        tmem_st16(tmem + lane_base + (uint32_t)(qcol + t * Bp + cb), y);
+                    }
+                }
+            tmem_wait_st();
             // ---- stress modes of this CTA
             for (int u = u0; u < u1; ++u, ++ucount) {
                 const GrpUnit &U = units[u - u0];
@@ -454,9 +519,16 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     for (int t = 0; t < nt; ++t) {
                         if (U.off[t] < 0) continue;
                         float v[16];
-                        tmem_ld16(tmem + lane_base + dcol + (uint32_t)(t * Bp + cb), v);
+                        const uint32_t va = tmem + lane_base + dcol + (uint32_t)(t * Bp + cb);
                         const int sb = G.tile_sb[t];
-                        if (r < G.tile_rows[t]) {
+                        if (!qrows) tmem_ld16(va, v);
+                        if (qrows) {
+                            float q[16];
+                            tmem_ld16x2(va, v, tmem + lane_base + (uint32_t)(qcol + t * Bp + cb), q);
+                            if (r < G.tile_rows[t])
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) acc[i] = fmaf(q[i], v[i], acc[i]);
+                        } else if (r < G.tile_rows[t]) {
                             const int kp = G.kpad[sb];
                             const float *qh = qimg + G.qoff[sb];
                             const float *ql = qh + Bp * kp;
@@ -483,8 +555,8 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     if (U.off[t] < 0) continue;
                     for (int cb = 0; cb < Bp; cb += 16) {
                         float v[16], f[16];
-                        tmem_ld16(tmem + lane_base + dcol + (uint32_t)(t * Bp + cb), v);
-                        tmem_ld16(tmem + lane_base + (uint32_t)(fcol + t * Bp + cb), f);
+                        tmem_ld16x2(tmem + lane_base + dcol + (uint32_t)(t * Bp + cb), v,
+                                    tmem + lane_base + (uint32_t)(fcol + t * Bp + cb), f);
 #pragma unroll
                         for (int i = 0; i < 16; ++i) f[i] = fmaf(C.ke[cb + i], v[i], f[i]);
                         tmem_st16(tmem + lane_base + (uint32_t)(fcol + t * Bp + cb), f);
@@ -498,18 +570,16 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
             if (!ok) break;
             // ---- partial forces of this CTA -> global slot (class order)
             for (int t = 0; t < nt; ++t) {
-                const int sb = G.tile_sb[t];
+                float *dst = P.part + G.part_off + (long long)slot_in_group * Bp * G.Np +
+                             (G.ocls[G.tile_sb[t]] + G.tile_r0[t] + r);
+                const int plates = r < G.tile_rows[t] ? G.B : 0;
                 for (int cb = 0; cb < Bp; cb += 16) {
                     float f[16];
                     tmem_ld16(tmem + lane_base + (uint32_t)(fcol + t * Bp + cb), f);
-                    if (r < G.tile_rows[t]) {
-                        const long long pos = G.ocls[sb] + G.tile_r0[t] + r;
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const int b = cb + i;
-                            if (b < G.B)
-                                P.part[G.part_off + ((long long)slot_in_group * Bp + b) * G.Np + pos] = f[i];
-                        }
+                    for (int i = 0; i < 16; ++i) {
+                        if (cb + i < plates) *dst = f[i];
+                        dst += G.Np;
                     }
                 }
             }
@@ -524,41 +594,67 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                     ok = false;
                     break;
                 }
-                for (int b = 0; b < G.B; ++b) {
-                    const GrpPlate pl = P.plates[G.plate0 + b];
-                    if (pl.owner != cta) continue;
-                    const InstDesc d = P.inst[pl.inst];
-                    const float e = P.exc ? P.exc[(long long)pl.inst * P.total_steps + n] : 0.f;
+                for (int own = 0; own < n_own; ++own) {
+                    const int b = C.own[own].b, Nb = C.own[own].N;
+                    const long long mode_off = C.own[own].mode_off;
+                    const float e = P.exc ? P.exc[(long long)C.own[own].inst * P.total_steps + n] : 0.f;
                     float ys = 0.f, ye = 0.f;
-                    for (int j = et; j < d.N; j += 128) {
-                        const int pos = P.gpos[G.gpos_off + j];
-                        const long long m = d.mode_off + j;
+                    for (int p0 = 4 * et; p0 < G.N; p0 += 512) {
+                        // four modes in class order: their states and coefficients, then
                         // the CTAs' parts in batches, all loads of a batch in flight at
-                        // once (one load per add took 45 us of the step for 38 CTAs and
-                        // plates of 400 modes), added in CTA order
-                        float f = 0.f;
-                        const float *part = P.part + G.part_off + (long long)b * G.Np + pos;
-                        const long long pst = (long long)Bp * G.Np;
-                        constexpr int kPB = 20;
-                        for (int s0 = 0; s0 < G.n_ctas; s0 += kPB) {
-                            float x[kPB];
+                        // once, added in CTA order (one mode at a time took 12 000 to
+                        // 30 000 cycles a step)
+                        long long m[4];
+                        bool on[4];
+                        float x0[4], x1[4], x2[4], x3[4], eps[4], rw2[4], rw2lo[4], rr[4], be[4], cc[4], cl[4];
 #pragma unroll
-                            for (int q = 0; q < kPB; ++q)
-                                x[q] = s0 + q < G.n_ctas ? ldcg(part + (s0 + q) * pst) : 0.f;
-#pragma unroll
-                            for (int q = 0; q < kPB; ++q)
-                                if (s0 + q < G.n_ctas) f += x[q];
+                        for (int i = 0; i < 4; ++i) {
+                            const int j = p0 + i < G.N ? inv[p0 + i] : Nb;
+                            on[i] = j < Nb;
+                            m[i] = mode_off + (on[i] ? j : 0);
+                            x0[i] = P.state_io[m[i]];
+                            x1[i] = P.state_io[TM + m[i]];
+                            x2[i] = P.state_io[2 * TM + m[i]];
+                            x3[i] = P.state_io[3 * TM + m[i]];
+                            eps[i] = P.coef.eps[m[i]];
+                            rw2[i] = P.coef.rw2[m[i]];
+                            rw2lo[i] = P.coef.rw2lo[m[i]];
+                            rr[i] = P.coef.r[m[i]];
+                            be[i] = P.coef.b[m[i]];
+                            cc[i] = P.coef.c[m[i]];
+                            cl[i] = P.coef.clo[m[i]];
                         }
-                        float x0 = P.state_io[m], x1 = P.state_io[TM + m];
-                        float x2 = P.state_io[2 * TM + m], x3 = P.state_io[3 * TM + m];
-                        sv_step(x0, x1, x2, x3, P.coef.eps[m], P.coef.rw2[m], P.coef.rw2lo[m],
-                                P.coef.r[m], fmaf(P.coef.b[m], e, -f));
-                        pickup_add(ys, ye, P.coef.c[m], P.coef.clo[m], x0, x1);
-                        P.state_io[m] = x0;
-                        P.state_io[TM + m] = x1;
-                        P.state_io[2 * TM + m] = x2;
-                        P.state_io[3 * TM + m] = x3;
-                        q_image_put(P.qbuf + G.qbuf_off, G, b, pos, x0);
+                        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float *part = P.part + G.part_off + (long long)b * G.Np + p0;
+                        const long long pst = (long long)Bp * G.Np;
+                        constexpr int kPB = 14;
+                        for (int s0 = 0; s0 < G.n_ctas; s0 += kPB, part += kPB * pst) {
+                            float4 x[kPB];
+#pragma unroll
+                            for (int q = 0; q < kPB; ++q)
+                                if (s0 + q < G.n_ctas) x[q] = ldcg4(part + q * pst);
+#pragma unroll
+                            for (int q = 0; q < kPB; ++q)
+                                if (s0 + q < G.n_ctas) {
+                                    f.x += x[q].x;
+                                    f.y += x[q].y;
+                                    f.z += x[q].z;
+                                    f.w += x[q].w;
+                                }
+                        }
+                        const float fv[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            sv_step(x0[i], x1[i], x2[i], x3[i], eps[i], rw2[i], rw2lo[i], rr[i],
+                                    fmaf(be[i], e, -fv[i]));
+                            if (!on[i]) continue;
+                            pickup_add(ys, ye, cc[i], cl[i], x0[i], x1[i]);
+                            P.state_io[m[i]] = x0[i];
+                            P.state_io[TM + m[i]] = x1[i];
+                            P.state_io[2 * TM + m[i]] = x2[i];
+                            P.state_io[3 * TM + m[i]] = x3[i];
+                            q_image_put(P.qbuf + G.qbuf_off, G, b, p0 + i, x0[i]);
+                        }
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) {
@@ -567,22 +663,23 @@ __global__ void __launch_bounds__(kGrpThreads, 1) group_kernel(const GroupParams
                         pickup_merge(ys, ye, s2, e2);
                     }
                     if (lane == 0) {
-                        C.pick[0][quarter] = ys;
-                        C.pick[1][quarter] = ye;
+                        C.own[own].ys[quarter] = ys;
+                        C.own[own].ye[quarter] = ye;
                     }
-                    epi_bar();
-                    if (et == 0) {
-                        float y = 0.f, yc = 0.f;
-                        for (int w = 0; w < 4; ++w) pickup_merge(y, yc, C.pick[0][w], C.pick[1][w]);
-                        y += yc;
-                        if (P.audio) P.audio[(long long)pl.inst * P.total_steps + n] = y;
-                        if (!isfinite(y)) set_status(P.status, pl.inst, MDX_ERR_NONFINITE);
-                    }
-                    epi_bar();
                 }
+                epi_bar();
                 if (et == 0) {
                     __threadfence();
                     atomicAdd(cnt_q, 1u);
+                }
+                // the samples, after the arrival that the group waits for
+                if (et < n_own) {
+                    float y = 0.f, yc = 0.f;
+                    for (int w = 0; w < 4; ++w) pickup_merge(y, yc, C.own[et].ys[w], C.own[et].ye[w]);
+                    y += yc;
+                    const int inst = C.own[et].inst;
+                    if (P.audio) P.audio[(long long)inst * P.total_steps + n] = y;
+                    if (!isfinite(y)) set_status(P.status, inst, MDX_ERR_NONFINITE);
                 }
             }
             epi_bar();
@@ -622,7 +719,7 @@ struct GroupPlan {
     int n_ctas = 0;
     int ring_stages = 3;
     size_t smem = 0;
-    int ring_off = 0, lo_off = 0, q_off = 0, scratch_off = 0;
+    int ring_off = 0, lo_off = 0, q_off = 0, scratch_off = 0, inv_off = 0;
     std::vector<GrpDesc> groups;
     std::vector<GrpUnit> units;
     std::vector<int> cta_group, cta_units;
@@ -999,15 +1096,19 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
     int max_units = 1;
     for (size_t c = 0; c + 1 < gp->cta_units.size(); c += 2)
         max_units = std::max(max_units, gp->cta_units[c + 1] - gp->cta_units[c]);
+    int n_max = 1;
+    for (const GrpDesc &d : gp->groups) n_max = std::max(n_max, d.N);
+    const int inv_bytes = (2 * n_max + 127) & ~127;
     const int unit_bytes = (int)((max_units * sizeof(GrpUnit) + 127) & ~size_t(127));
-    const int ring = std::max(min_ring, std::min(8, (smem_optin - ctrl_bytes - q_floats_max * 4 -
-                                                     unit_bytes) / (2 * kGrpStageBytes)));
+    const int ring = std::max(min_ring - 1, std::min(8, (smem_optin - ctrl_bytes - q_floats_max * 4 -
+                                                     unit_bytes - inv_bytes) / (2 * kGrpStageBytes)));
     gp->ring_stages = ring;
     gp->ring_off = ctrl_bytes;
     gp->lo_off = gp->ring_off + ring * kGrpStageBytes;
     gp->q_off = gp->lo_off + ring * kGrpStageBytes;
     gp->scratch_off = gp->q_off + q_floats_max * 4;
-    gp->smem = (size_t)gp->scratch_off + unit_bytes;
+    gp->inv_off = gp->scratch_off + unit_bytes;
+    gp->smem = (size_t)gp->inv_off + inv_bytes;
     if ((int)gp->smem > smem_optin)
         return bail(gfail(MDX_ERR_UNSUPPORTED, "grouped plates exceed the shared-memory budget"));
     // kappa tables stay zero until group_plan_set_kappa
@@ -1094,6 +1195,7 @@ cudaError_t group_plan_launch(GroupPlan *g, const InstDesc *d_inst, const ModeCo
     P.lo_off = g->lo_off;
     P.q_off = g->q_off;
     P.scratch_off = g->scratch_off;
+    P.inv_off = g->inv_off;
     P.l2_keep = l2_keep;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g->n_ctas);

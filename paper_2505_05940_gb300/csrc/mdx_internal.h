@@ -311,7 +311,8 @@ struct TensionParams {
 // together: per step and stress mode k, U^k = H^k [q_1 ... q_B] is one
 // tensor-core GEMM over the plates of the group (split TF32 on tcgen05, FP32
 // accumulation in tensor memory), see mdx_group.cu.
-constexpr int kGrpThreads = 256;      // 8 warps: producer, MMA, 2 converters, 4 epilogue
+constexpr int kGrpConvWarps = 4;      // converter warps
+constexpr int kGrpThreads = 32 * (6 + kGrpConvWarps);   // with producer, MMA, 4 epilogue
 constexpr int kGrpChunk = 16;         // K elements (columns of H^k) per ring stage
 constexpr int kGrpStageBytes = 128 * kGrpChunk * 4;   // one 128-row stage (8 KB)
 constexpr int kGrpMaxTiles = 16;      // (row class, 128-row tile) blocks per stress mode
@@ -377,7 +378,7 @@ struct GroupParams {
     int *abort_flag;
     long long wait_limit;
     int ring_stages;
-    int ring_off, lo_off, q_off, scratch_off;   // shared-memory byte offsets
+    int ring_off, lo_off, q_off, scratch_off, inv_off;   // shared-memory byte offsets
     float l2_keep;
 };
 

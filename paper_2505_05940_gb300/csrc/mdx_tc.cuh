@@ -171,6 +171,35 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Two loads with one wait (the words are operands of the wait, so no use of them
+// moves above it).
+__device__ __forceinline__ void tmem_ld16x2(uint32_t ta, float (&a)[16], uint32_t tb, float (&b)[16]) {
+    uint32_t r[2][16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+            "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+            : "=r"(r[h][0]), "=r"(r[h][1]), "=r"(r[h][2]), "=r"(r[h][3]), "=r"(r[h][4]), "=r"(r[h][5]),
+              "=r"(r[h][6]), "=r"(r[h][7]), "=r"(r[h][8]), "=r"(r[h][9]), "=r"(r[h][10]),
+              "=r"(r[h][11]), "=r"(r[h][12]), "=r"(r[h][13]), "=r"(r[h][14]), "=r"(r[h][15])
+            : "r"(h == 0 ? ta : tb)
+            : "memory");
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                     : "+r"(r[h][0]), "+r"(r[h][1]), "+r"(r[h][2]), "+r"(r[h][3]), "+r"(r[h][4]),
+                       "+r"(r[h][5]), "+r"(r[h][6]), "+r"(r[h][7]), "+r"(r[h][8]), "+r"(r[h][9]),
+                       "+r"(r[h][10]), "+r"(r[h][11]), "+r"(r[h][12]), "+r"(r[h][13]), "+r"(r[h][14]),
+                       "+r"(r[h][15])
+                     :: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        a[i] = __uint_as_float(r[0][i]);
+        b[i] = __uint_as_float(r[1][i]);
+    }
+}
+
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
