@@ -143,8 +143,8 @@ typedef struct mdx_options {
                           equivalence tests);
                           bit 3: run the direction contraction on the CUDA-core kernel instead
                           of the tensor cores (equivalence tests);
-                          bit 4: run forward passes on the streaming plate kernel even where
-                          the plates fit cluster-resident (equivalence tests); 0 in normal use */
+                          bit 4: run every pass on the streaming plate kernel even where the
+                          plates fit the resident one (equivalence tests); 0 in normal use */
     int scheme;        /* MDX_SCHEME_SV (default) or MDX_SCHEME_TF */
     int group_engine;  /* plates with geom_group > 0: MDX_GROUP_TF32X3 (default) steps each
                           group with one shared coupling tensor on the tensor cores;

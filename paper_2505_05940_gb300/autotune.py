@@ -1,10 +1,10 @@
 """Tile autotuner for the plate kernel.
 
 For a given set of instances the tuner times a short checkpointed forward
-run (the streaming plate kernel, which also serves every gradient pass) for
-each candidate TMA stage size (the ring depth follows from the shared memory
-left over) and keeps the fastest.  Checkpoint-free forward passes of a few
-small plates run cluster-resident instead and have no stages to tune.  Results are cached in a JSON file keyed by the
+run for each candidate TMA stage size of the streaming plate kernel (the ring
+depth follows from the shared memory left over) and keeps the fastest.  Plans
+that the resident kernel takes have no stages to tune: every candidate then
+times alike.  Results are cached in a JSON file keyed by the
 GPU name and a signature of the plate shapes, so a workload is tuned once per
 device type.  Timing uses the library's own per-launch CUDA events
 (mdx_plan_kernel_stats).
