@@ -915,8 +915,10 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
     }
     // ---- kernel groups: members of an image in batches of at most Bsub plates
     const int ctrl_bytes = (int)((sizeof(Ctrl) + 1023) & ~size_t(1023));
-    const int min_ring = 4;   // at least this many stages beside the Q images
-    const int fixed = ctrl_bytes + 2 * min_ring * kGrpStageBytes;
+    // room for four stages beside the Q images decides the plates of a group; the
+    // owners' list and the mode table may take the fourth's
+    const int min_ring = 3;
+    const int fixed = 2048 + 2 * (min_ring + 1) * kGrpStageBytes;
     struct KG {
         int image;
         std::vector<int> plates;
@@ -927,8 +929,8 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
         int sumk = 0;
         for (int a = 0; a < 4; ++a) sumk += im.kpad[a];
         const int nt = (int)im.tile_sb.size();
-        // two accumulator sets and the forces in tensor memory; the Q images and
-        // at least min_ring stages in shared memory
+        // two accumulator sets and the forces in tensor memory; the Q images and the
+        // stages in shared memory
         int bsub = 32;
         while (bsub > 16 && (3 * nt * bsub > 512 || fixed + 8LL * bsub * sumk > smem_optin)) bsub -= 16;
         if (3 * nt * bsub > 512 || fixed + 8LL * bsub * sumk > smem_optin)
@@ -1100,7 +1102,7 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
     for (const GrpDesc &d : gp->groups) n_max = std::max(n_max, d.N);
     const int inv_bytes = (2 * n_max + 127) & ~127;
     const int unit_bytes = (int)((max_units * sizeof(GrpUnit) + 127) & ~size_t(127));
-    const int ring = std::max(min_ring - 1, std::min(8, (smem_optin - ctrl_bytes - q_floats_max * 4 -
+    const int ring = std::max(min_ring, std::min(8, (smem_optin - ctrl_bytes - q_floats_max * 4 -
                                                      unit_bytes - inv_bytes) / (2 * kGrpStageBytes)));
     gp->ring_stages = ring;
     gp->ring_off = ctrl_bytes;
