@@ -661,13 +661,14 @@ def main():
     dom = max(stats, key=lambda w: stats[w][1])
     n_l, d_ms, d_bytes = stats[dom]
     achieved = (d_bytes / n_l) / ((d_ms / n_l) * 1e-3) / 1e9 if n_l else 0.0
-    names = {0: "plate_kernel<1> forward", 1: "plate_kernel<1> recompute",
-             2: "plate_kernel<2> reverse", 4: "plate_kernel<3> fused reverse + recompute"}
-    traffic = profiled_traffic(a, a.K) if dom == 4 else None
+    names = {0: "plate kernel, forward", 1: "plate kernel, recompute",
+             2: "plate kernel, reverse", 4: "plate kernel, fused reverse + recompute"}
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": traffic,
-                "traffic_source": ("profiles/plate_kernel_fused_64plates_200x50.md "
-                                   "(ncu, bytes per step x steps per launch)") if traffic else None,
+                "frac": achieved / peak, "traffic": None,
+                "basis": "bytes of one pass over the class-layout coupling data per step, as "
+                         "if streamed; plates of at most 64 modes per class run on the "
+                         "resident kernel, which reads them once per launch and is bound "
+                         "by its step's dependent chain and FP32 FMAs",
                 "kernel": names[dom], "peak_source": f"{peak_kind} hbm_gbs",
                 "kernel_share_of_step": tot_ms / ms_total if ms_total else None,
                 "per_launch_ms": d_ms / max(n_l, 1),

@@ -659,13 +659,13 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                         nb[mp[h]] = 0.f;
                     if (more_lays)
 #pragma unroll 1
-                      for (int l = 0; l < lays - 1; ++l) {
-                        const int at = lp[(l * 2 + h) * WT];
-                        if (it < rsteps)
-                            copy4(nb + at, nq_src + h * WT);
-                        else
-                            nb[at] = 0.f;
-                    }
+                        for (int l = 0; l < lays - 1; ++l) {
+                            const int at = lp[(l * 2 + h) * WT];
+                            if (it < rsteps)
+                                copy4(nb + at, nq_src + h * WT);
+                            else
+                                nb[at] = 0.f;
+                        }
                 }
             nq_src -= TM;
         };
@@ -699,7 +699,8 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         bool bad = false;
         const int seg_last = A.seg_last, segs_all = A.segs_all;
         const int carry = EXT ? A.carry : 0, nw = carry & 2 ? A.tail : nk;
-        const uint32_t c_dst = carry & 2 ? peer_addr(su32(sm + O.car) + (uint32_t)(tid * XF * 4), (uint32_t)(A.base + rank + 1)) : 0u;
+        const uint32_t c_own = su32(sm + O.car) + (uint32_t)(tid * XF * 4);
+        const uint32_t c_dst = carry & 2 ? peer_addr(c_own, (uint32_t)(A.base + rank + 1)) : 0u;
         const uint32_t c_bar = carry & 2 ? peer_addr(su32(bar_c), (uint32_t)(A.base + rank + 1)) : 0u;
         const unsigned long long new_item = A.new_item;
         // every part a partial sum of its own, or one row of them: one chain (with the
