@@ -517,7 +517,9 @@ __global__ void __launch_bounds__(kPlateBlock, 1) plate_kernel(const PlateParams
                     for (int a = 0; a < 4; ++a) {
                         const int bcl = a ^ ch.c;
                         const int na = pick4(d.ncls, a), nbc = pick4(d.ncls, bcl);
-                        if (na == 0 || nbc == 0) continue;
+                        // (no rows, na = 0: u^k is zero on these columns and is stored as such,
+                        // the force reads every column)
+                        if (nbc == 0) continue;
                         const int oa = pick4(d.ocls, a), ob = pick4(d.ocls, bcl);
                         const int nb4 = (nbc + 3) & ~3, nq = nb4 >> 2;
                         const int L = mc * nb4;
