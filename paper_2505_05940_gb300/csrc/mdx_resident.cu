@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         bar_init(bar_c, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (sub > 1) {
-            bar_expect_tx(bar_f, (uint32_t)(A.segs_all * no * XF * 4));
+            if (no > 0) bar_expect_tx(bar_f, (uint32_t)(A.segs_all * no * XF * 4));
             bar_expect_tx(bar_q, (uint32_t)(N * 4 * (FUSED ? 2 : 1) * lays));
             if (EXT && (A.carry & 1)) bar_expect_tx(bar_c, (uint32_t)(N * XF * 4));
         }
@@ -709,8 +709,12 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const bool flat = !SAME || new_item == later || new_item == 0ull;
         const uint32_t xbuf = (uint32_t)(Q.segs * Q.no_max * XF * 4);
         const uint32_t sbuf = (uint32_t)(Q.no_max * XF * 4);        // one part
-        // the next phases are armed by a thread that has waited for the last ones
+        // the next phases are armed by a thread that has waited for the last ones.  A
+        // CTA without modes (more CTAs than modes) receives no parts: it neither arms
+        // nor awaits bar_f, whose phases of no bytes would end by being armed and run
+        // ahead of the warps that wait for them
         const bool arms = sub > 1 && wr == 0 && lane == 0;
+        const bool owns = no > 0;
         bool dead = false;
         // a wait that runs out keeps the common control flow without further waits
         auto wait = [&](uint64_t *b, uint32_t parity) {
@@ -931,7 +935,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     if (EXT && (carry & 1)) carried(h, f);
                     parts(mp[h], f, [&](int seg, const float (&v)[R]) { push_part(dst + seg * sbuf, mbar[h], v); });
                 }
-                if (upd) {
+                if (upd && owns) {
                     wait(bar_f, (uint32_t)buf);
                     const float *x = sm + O.xch + (buf * Q.segs * Q.no_max + oi) * XF;
                     if (on && flat) {
@@ -1014,7 +1018,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 }
             }
             // ---- off the chain: gradient sums, stores, pickups, the next step's inputs
-            if (arms && it + 1 < P.steps) bar_expect_tx(bar_f, tx_f);
+            if (arms && owns && it + 1 < P.steps) bar_expect_tx(bar_f, tx_f);
             if (REV && rev_on && kon) {
                 kahan_add(ks, kcmp, -dot[0] * dot[1]);
                 if (st_x) {
