@@ -132,7 +132,8 @@ typedef struct mdx_options {
     int ring_stages;   /* TMA ring depth of the plate kernel (0 = default) */
     int stage_bytes;   /* bytes per ring stage (0 = default; multiple of 16) */
     int force_split;   /* >0: split every plate over at least this many CTAs (tests) */
-    int wait_limit;    /* >0: spin-iteration cap of device waits (tests); 0 = default */
+    int wait_limit;    /* >0: spin-iteration cap of the device waits of the plate kernels
+                          (streaming, resident, grouped; tests); 0 = default */
     int debug_flags;   /* bit 0: the second contributor of every shared plate withholds its
                           arrival, so the other contributors' bounded waits run out and the
                           call reports MDX_ERR_TIMEOUT (fault-path tests);
@@ -144,7 +145,10 @@ typedef struct mdx_options {
                           bit 3: run the direction contraction on the CUDA-core kernel instead
                           of the tensor cores (equivalence tests);
                           bit 4: run every pass on the streaming plate kernel even where the
-                          plates fit the resident one (equivalence tests); 0 in normal use */
+                          plates fit the resident one (equivalence tests);
+                          bit 5: on the resident kernel the second CTA of every shared plate
+                          withholds its parts of the force, so the owners' bounded waits run
+                          out (fault-path tests); 0 in normal use */
     int scheme;        /* MDX_SCHEME_SV (default) or MDX_SCHEME_TF */
     int group_engine;  /* plates with geom_group > 0: MDX_GROUP_TF32X3 (default) steps each
                           group with one shared coupling tensor on the tensor cores;

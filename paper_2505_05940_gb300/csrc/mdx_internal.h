@@ -275,6 +275,7 @@ struct ResidentParams {
     int n_max;                        // most modes of a plate
     int lays, carry;                  // most layouts of a CTA; any part spans CTAs
     int tcols;                        // tensor-memory columns per CTA
+    int wait_limit;                   // polls of a wait
 };
 
 int resident_variant(int w, int rows);

@@ -1566,6 +1566,7 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
 int run_resident(mdx_plan *p, const mdx_plan::Resident &res, const PlateParams &P, cudaStream_t s) {
     ResidentParams Q = res.q;
     Q.p = P;
+    Q.wait_limit = (int)std::min<long long>(P.wait_limit, 0x7fffffff);
     const int R = P.mode == MODE_FUSED ? 3 : (P.mode == MODE_REVERSE ? 2 : 1);
     mdx_plan::Rec rec{};
     if (p->profiling) {

@@ -84,7 +84,6 @@ constexpr int kPickPitch = 36;               // terms of a step: 4 lanes x 4 ste
 // shared memory over one allocation step more than its 512 columns, so any CTAs
 // that fit an SM by shared memory hold at most 512 columns together.
 constexpr size_t kSmemPerColumn = 430;
-constexpr long long kResWait = 1LL << 22;    // bound of every wait (polls)
 
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
@@ -356,6 +355,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     extern __shared__ __align__(16) float sm[];
     __shared__ ResCta A;
     __shared__ InstDesc d;
+    __shared__ int gave_up;                       // a wait of this CTA ran out
     const PlateParams &P = Q.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr bool REV = R >= 2, FWD = R == 1, FUSED = R == 3;
@@ -374,6 +374,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     for (int e = tid; e < (int)(sizeof(ResCta) / 4); e += blockDim.x)
         reinterpret_cast<int *>(&A)[e] = reinterpret_cast<const int *>(Q.ctas + blockIdx.x)[e];
     for (int e = 16 + tid; e < O.end; e += blockDim.x) sm[e] = 0.f;
+    if (tid == 0) gave_up = 0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          su32(tbase)), "r"(Q.tcols)
@@ -439,7 +440,8 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         for (int h = 0; h < 2; ++h) {
             const int i = tid + h * WT;
             if (i >= N) continue;
-            mon[h] = true;
+            // (bit 5 of the debug flags: the second CTA of a plate withholds its parts)
+            mon[h] = !((P.debug_flags & 32) && rank == 1);
             const long long m = d.mode_off + i;
             mp[h] = class_pos(i);
             if (sub > 1) {
@@ -562,8 +564,11 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const int wr = W - 1 - warp, reps = sub > 1 ? max(W / C, 1) : 1;
         const int chunk = wr % C, rep = wr / C;
         const int oi = 32 * chunk + lane;                       // owned index
-        const bool upd = rep < reps;                            // this warp updates
-        const bool on = upd && oi < no;
+        // This warp updates.  None does in a CTA without modes (more CTAs than modes): it
+        // receives no parts, and a phase of bar_f without bytes ends by being armed, so
+        // it would run ahead of a warp that waited for it.
+        const bool upd = rep < reps && no > 0;
+        bool on = upd && oi < no;
         const bool lead = on && rep == 0;                       // writes the mode's results
         // the warps that repeat a chunk share its sums and stores: bits 0..4 the
         // gradient sums, then w, q', v' of the segments
@@ -684,7 +689,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const int cmax = ((N + sub - 1) / sub + 31) / 32, yent = rank * cmax + chunk;
         int chunks_all = 0;
         for (int r = 0; r < sub; ++r)
-            chunks_all += max(((int)((long long)N * (r + 1) / sub) - (int)((long long)N * r / sub) + 31) / 32, 1);
+            chunks_all += ((int)((long long)N * (r + 1) / sub) - (int)((long long)N * r / sub) + 31) / 32;
         float2 *const pst = reinterpret_cast<float2 *>(sm + O.pst) + chunk * kPickSteps * kPickPitch;
         const uint32_t y_dst0 = sub > 1 ? peer_addr(su32(sm + O.pick + 2 * yent), (uint32_t)(A.base + sub - 1)) : 0u;
         const uint32_t y_bar0 = sub > 1 ? peer_addr(su32(bar_y), (uint32_t)(A.base + sub - 1)) : 0u;
@@ -709,20 +714,22 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
         const bool flat = !SAME || new_item == later || new_item == 0ull;
         const uint32_t xbuf = (uint32_t)(Q.segs * Q.no_max * XF * 4);
         const uint32_t sbuf = (uint32_t)(Q.no_max * XF * 4);        // one part
-        // the next phases are armed by a thread that has waited for the last ones.  A
-        // CTA without modes (more CTAs than modes) receives no parts: it neither arms
-        // nor awaits bar_f, whose phases of no bytes would end by being armed and run
-        // ahead of the warps that wait for them
-        const bool arms = sub > 1 && wr == 0 && lane == 0;
-        const bool owns = no > 0;
+        // the next phases are armed by a thread that has waited for the last ones
+        bool arms = sub > 1 && wr == 0 && lane == 0;
+        // A thread whose wait runs out keeps the common control flow, but waits for
+        // nothing more, stores nothing into peers and arms nothing (a phase that it has
+        // not seen complete must not be armed again).  So the peers' waits run out in
+        // turn, after a step or two whose stores complete no phase.
         bool dead = false;
-        // a wait that runs out keeps the common control flow without further waits
         auto wait = [&](uint64_t *b, uint32_t parity) {
             if (dead) return;
-            long long i = 0;
-            while (!bar_try(b, parity) && ++i < kResWait) {
-            }
-            dead = i >= kResWait;
+            for (int i = 0; !bar_try(b, parity);)
+                if (__builtin_expect(++i >= Q.wait_limit, 0)) {
+                    dead = true;
+                    mon[0] = mon[1] = on = arms = false;
+                    gave_up = 1;
+                    break;
+                }
         };
         // lane = 4 step + part: a quarter of the chunks' terms of one of eight steps
         auto collect = [&](int grp) {
@@ -746,7 +753,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     P.audio[(long long)A.plate * P.total_steps + P.n_begin + n8] = y;
                 if (!isfinite(y)) bad = true;
             }
-            arm_y(grp + 2);
+            if (!dead) arm_y(grp + 2);
         };
         bar_sync_id(1, WT);
 
@@ -877,7 +884,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             };
             auto take_carry = [&]() {
                 if (32 * warp < N) wait(bar_c, (uint32_t)buf);
-                if (tid == 0 && it + 1 < P.steps) bar_expect_tx(bar_c, (uint32_t)(N * XF * 4));
+                if (tid == 0 && !dead && it + 1 < P.steps) bar_expect_tx(bar_c, (uint32_t)(N * XF * 4));
             };
             float F[R], item[R];
 #pragma unroll
@@ -935,7 +942,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                     if (EXT && (carry & 1)) carried(h, f);
                     parts(mp[h], f, [&](int seg, const float (&v)[R]) { push_part(dst + seg * sbuf, mbar[h], v); });
                 }
-                if (upd && owns) {
+                if (upd) {
                     wait(bar_f, (uint32_t)buf);
                     const float *x = sm + O.xch + (buf * Q.segs * Q.no_max + oi) * XF;
                     if (on && flat) {
@@ -1018,7 +1025,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                 }
             }
             // ---- off the chain: gradient sums, stores, pickups, the next step's inputs
-            if (arms && owns && it + 1 < P.steps) bar_expect_tx(bar_f, tx_f);
+            if (arms && it + 1 < P.steps) bar_expect_tx(bar_f, tx_f);
             if (REV && rev_on && kon) {
                 kahan_add(ks, kcmp, -dot[0] * dot[1]);
                 if (st_x) {
@@ -1079,7 +1086,7 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
                         const float e2 = __shfl_xor_sync(0xffffffffu, ye, o);
                         pickup_merge(ys, ye, s2, e2);
                     }
-                    if (part == 0 && s8 <= ps) {
+                    if (part == 0 && s8 <= ps && !dead) {
                         const int po = (pb * kPickSteps + s8) * 2 * O.PS;
                         if (sub > 1)
                             push2(y_dst0 + (uint32_t)(po * 4), y_bar0 + 8u * pb, ys, ye);
@@ -1133,8 +1140,9 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
             P.kacc[2 * (d.k_off + kl)] = ks;
             P.kacc[2 * (d.k_off + kl) + 1] = kcmp;
         }
-        if (dead && lane == 0) set_status(P.status, A.plate, MDX_ERR_TIMEOUT);
+        if (__any_sync(0xffffffffu, dead) && lane == 0) set_status(P.status, A.plate, MDX_ERR_TIMEOUT);
     }
+    copies_done();
     __syncwarp();
     tc_fence_before();
     __syncthreads();
@@ -1142,8 +1150,13 @@ __global__ void __launch_bounds__(256, 1) resident_kernel(const ResidentParams Q
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem0), "r"(Q.tcols)
                      : "memory");
-    // no CTA leaves while a peer may still store into its shared memory
+    // No peer stores into this CTA's shared memory from here on, and a CTA that waited for
+    // everything sent to it has it.  Into one that gave up stores may still be on their
+    // way, which no barrier counts to their end: it stays for far longer than their
+    // hop of some 400 cycles.
     cluster_sync_all();
+    if (gave_up)
+        for (int i = 0; i < 64; ++i) __nanosleep(1000);
 }
 
 namespace {
