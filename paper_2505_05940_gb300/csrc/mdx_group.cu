@@ -1110,7 +1110,8 @@ int group_plan_build(GroupPlan **out, const mdx_instance *I, const std::vector<I
     gp->q_off = gp->lo_off + ring * kGrpStageBytes;
     gp->scratch_off = gp->q_off + q_floats_max * 4;
     gp->inv_off = gp->scratch_off + unit_bytes;
-    gp->smem = (size_t)gp->inv_off + inv_bytes;
+    // (its CTAs take all columns: the share of the shared memory that goes with them)
+    gp->smem = std::max((size_t)gp->inv_off + inv_bytes, kTmemColumns * kSmemPerColumn);
     if ((int)gp->smem > smem_optin)
         return bail(gfail(MDX_ERR_UNSUPPORTED, "grouped plates exceed the shared-memory budget"));
     // kappa tables stay zero until group_plan_set_kappa

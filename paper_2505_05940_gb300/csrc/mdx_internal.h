@@ -227,6 +227,17 @@ struct DirParams {
     int *status;
 };
 
+// Shared memory asked for per tensor-memory column by kernels whose CTAs wait for
+// one another (resident and grouped plates): above 233 472 / 544, the SM's shared
+// memory over one allocation step more than its 512 columns, so any of their CTAs
+// that fit an SM by shared memory hold at most 512 columns together.  A CTA whose
+// peers wait for it must not block on another's columns: with a resident CTA
+// beside a grouped one, each behind the other's columns on two SMs, neither plan
+// would go on until the waits ran out.
+constexpr size_t kSmemPerColumn = 430;
+constexpr int kTmemColumns = 512;
+static_assert(kSmemPerColumn * (kTmemColumns + 32) > 233472, "two such CTAs must not share an SM");
+
 // Resident plates (mdx_resident.cu): a plate's coupling tensor held by `sub`
 // CTAs of one thread-block cluster for the whole launch.
 struct ClusterK {

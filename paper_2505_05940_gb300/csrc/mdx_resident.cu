@@ -80,10 +80,6 @@ typedef unsigned long long u64;
 constexpr int kResMaxWarps = 8;              // warps of a CTA
 constexpr int kPickSteps = 8;                // pickups reduced together
 constexpr int kPickPitch = 36;               // terms of a step: 4 lanes x 4 steps on distinct banks
-// Shared memory asked for per tensor-memory column: above 233 472 / 544, the SM's
-// shared memory over one allocation step more than its 512 columns, so any CTAs
-// that fit an SM by shared memory hold at most 512 columns together.
-constexpr size_t kSmemPerColumn = 430;
 
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
