@@ -175,7 +175,7 @@ struct LayerArgs {
 struct GemmCtrl {
     uint64_t bar[kGemmStages];
     uint32_t tmem;
-    int fail;
+    int fail;                // first chunk after which a wait ran out
 };
 
 }  // namespace
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const __grid_con
     const int chunks = (g.K + TBK - 1) / TBK;
     if (tid == 0) {
         for (int b = 0; b < kGemmStages; ++b) bar_init(&C.bar[b], 1);
-        C.fail = 0;
+        C.fail = chunks;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -264,7 +264,8 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const __grid_con
         fence_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (C.fail) {
+        // (a failure counts behind the next barrier, where every thread reads it)
+        if (C.fail < c) {
             ok = false;
             break;
         }
@@ -282,8 +283,10 @@ __global__ void __launch_bounds__(kGemmThreads) mlp_gemm_kernel(const __grid_con
             ++committed;
         }
         // the buffer of chunk c + 3 was read by chunk c - 1
-        if (c + kGemmStages - 1 < chunks && c >= 1 && !mma_wait(c - 1)) C.fail = 1;
-        stage_group(c + kGemmStages - 1);
+        if (c + kGemmStages - 1 < chunks && c >= 1 && !mma_wait(c - 1))
+            atomicMin(&C.fail, c);
+        else
+            stage_group(c + kGemmStages - 1);
     }
     // the last commit covers every MMA issued before it
     if (ok && chunks > 0) ok = mma_wait(chunks - 1);
