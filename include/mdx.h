@@ -206,7 +206,11 @@ int mdx_plan_set_coefficients(mdx_plan *plan, const double *omega2, const double
  * A of the mode's poles.  Time is cut into chunks of 256 steps: each chunk's
  * response to its own input from rest, then the chunk boundary states
  * S_j = A^256 S_{j-1} + E_j, then every chunk again from its true state with
- * the pickup.  FP64 arithmetic, FP32 audio.  Arguments as in mdx_simulate;
+ * the pickup.  The chunks' responses, the boundary states and q_end, qm1_end
+ * are FP64.  The pass with the pickup steps each chunk from its FP64 state in pairs
+ * of FP32 numbers (about 48 bits), scaled per mode and chunk by a power of two; the
+ * audio is FP32, and a sample beyond the range of FP32 counts as non-finite in
+ * `status`.  Arguments as in mdx_simulate;
  * work is caller-owned device scratch of mdx_linear_workspace_bytes(plan,
  * steps).  Asynchronous on `stream`.  Errors: MDX_ERR_ARG (workspace, steps),
  * MDX_ERR_CUDA.

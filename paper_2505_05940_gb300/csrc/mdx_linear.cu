@@ -16,15 +16,19 @@
 //   3. every chunk reruns from its true incoming state S_{j-1} and writes the
 //      pickup y^n = sum_mu c_mu q_mu^{n+1}.
 //
-// Arithmetic of the passes over the steps: unevaluated FP32 pairs (about 48
-// bits) for state, coefficients and products, in the difference form
-// (q, v = q - q^{n-1}).  The FP64 units do 2 operations a cycle and SM, the FP32
-// units 128; a step costs 48 of the latter against 3 to 4 of the former, and 64
-// objects of 20 to 400 modes over 22 050 steps took 5.1 ms in FP64, 0.86 ms so.
-// The chain over the chunks stays in the FP64 companion form: its rounding sets
-// the digits of the final states beyond the eighth.  The pickup's terms go
-// through shared memory and each lane sums one step (shuffle sums of every step
-// were the larger half of the time).
+// Arithmetic.  The chunks' own responses, the chain over the chunks and the end
+// states are FP64: a strongly damped mode's state leaves the range of FP32 within a
+// chunk (eps reaches 1.2 for the upper modes of an ordinary plate).  Step 3 needs
+// its states for FP32 samples only: it starts from the FP64 state and steps
+// unevaluated FP32 pairs (about 48 bits) in the difference form (q, v = q - q^{n-1}),
+// scaled per mode and chunk by a power of two to about 1 (its underflow is then
+// below 2^-140 of the mode's largest value in the chunk).  The FP64 units do 2
+// operations a cycle and SM, the FP32 units 128; a step costs 48 of the latter
+// against 4 of the former.  The pickup's terms go through shared memory and each
+// lane sums one step (shuffle sums of every step were the larger half of the
+// time).  64 objects of 20 to 400 modes over 22 050 steps: 5.07 ms in FP64 throughout,
+// 1.23 ms so (0.86 ms with step 1 in FP32 pairs too, which lost the end states of
+// one mode in ten).
 #include <cuda_runtime.h>
 
 #include "../../include/mdx.h"
@@ -48,7 +52,6 @@ __device__ __forceinline__ Pair pair_of(double x) {
     p.l = (float)(x - (double)p.h);
     return p;
 }
-__device__ __forceinline__ double value(Pair p) { return (double)p.h + (double)p.l; }
 
 // (h, l) of a + b with |l| at most half an ulp of h, b any pair.
 __device__ __forceinline__ Pair add(Pair a, Pair b) {
@@ -73,23 +76,17 @@ struct LinCoef {
     Pair neps, nrho, rb;
 };
 
-// eps and rho of the companion form as FP64 holds it: g = 2 - eps - rho and
-// p = eps - 1 are rounded there (rho of a slow mode loses digits against 2), and
-// the difference form of the same recursion keeps those digits, not more.
-__device__ __forceinline__ SchemeCoef scheme_of(const LinearParams &P, long long gm) {
-    SchemeCoef k = scheme_coef(P.scheme, P.omega2[gm], P.gamma[gm], P.dt[gm]);
-    const double p = k.eps - 1.0, g = 2.0 - k.eps - k.rho;
-    k.eps = 1.0 + p;
-    k.rho = (1.0 - g) - p;
-    return k;
-}
+// The recursion's coefficients in FP64: q^{n+1} = g q^n + p q^{n-1} + rb e^n.
+struct LinCoef64 {
+    double g, p, rb;
+};
 
-__device__ __forceinline__ LinCoef lin_coef(const LinearParams &P, long long gm) {
-    const SchemeCoef k = scheme_of(P, gm);
-    LinCoef o;
-    o.neps = pair_of(-k.eps);
-    o.nrho = pair_of(-k.rho);
-    o.rb = pair_of(k.r * P.b[gm]);
+__device__ __forceinline__ LinCoef64 lin_coef64(const LinearParams &P, long long gm) {
+    const SchemeCoef k = scheme_coef(P.scheme, P.omega2[gm], P.gamma[gm], P.dt[gm]);
+    LinCoef64 o;
+    o.p = k.eps - 1.0;             // eps = 1 + p
+    o.g = 2.0 - k.eps - k.rho;     // rho = 1 - g - p
+    o.rb = k.r * P.b[gm];
     return o;
 }
 
@@ -103,36 +100,50 @@ __device__ __forceinline__ void lin_step(const LinCoef &k, float e, Pair &q, Pai
 }
 
 // Excitation of a chunk in shared memory (zeros without one).
-__device__ __forceinline__ void load_exc(const LinearParams &P, int inst, int n0, int n1, float *es) {
+template <typename T>
+__device__ __forceinline__ void load_exc(const LinearParams &P, int inst, int n0, int n1, T *es) {
     const float *e = P.exc ? P.exc + (long long)inst * P.total_steps : nullptr;
-    for (int n = n0 + threadIdx.x; n < n1; n += blockDim.x) es[n - n0] = e ? e[n] : 0.f;
+    for (int n = n0 + threadIdx.x; n < n1; n += blockDim.x) es[n - n0] = e ? (T)e[n] : (T)0;
     __syncthreads();
 }
 
+// Largest magnitude of the chunk's excitation (NaN if there is one: its bits are the
+// largest).
+__device__ __forceinline__ float largest(const float *es, int cnt) {
+    unsigned u = 0;
+    for (int t = threadIdx.x & 31; t < cnt; t += 32) u = max(u, __float_as_uint(fabsf(es[t])));
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, u));
+}
+
+// A step is two FP64 operations: the response to e alone, r b applied at the end.
 __global__ void __launch_bounds__(kLinThreads) lin_local_kernel(const LinearParams P) {
-    __shared__ float es[kLinChunk];
+    __shared__ double es[kLinChunk];
     const int j = blockIdx.x, inst = blockIdx.y;
     if (j >= P.n_chunks - 1) return;        // the last chunk's end state is not needed
     const InstDesc d = P.inst[inst];
     const int n0 = j * P.L, n1 = min(P.steps, n0 + P.L);
     load_exc(P, inst, n0, n1, es);
     for (int m = threadIdx.x; m < d.N; m += kLinThreads) {
-        const LinCoef k = lin_coef(P, d.mode_off + m);
-        Pair q = {0.f, 0.f}, v = {0.f, 0.f};
+        const LinCoef64 k = lin_coef64(P, d.mode_off + m);
+        double x0 = 0.0, x1 = 0.0;
 #pragma unroll 4
-        for (int n = 0; n < n1 - n0; ++n) lin_step(k, es[n], q, v);
+        for (int n = 0; n < n1 - n0; ++n) {
+            const double x = fma(k.g, x0, fma(k.p, x1, es[n]));
+            x1 = x0;
+            x0 = x;
+        }
         double *E = P.E + ((long long)j * P.total_modes + d.mode_off + m) * 2;
-        E[0] = value(q);
-        E[1] = value(q) - value(v);
+        E[0] = k.rb * x0;
+        E[1] = k.rb * x1;
     }
 }
 
 __global__ void lin_carry_kernel(const LinearParams P) {
     const long long gmode = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (gmode >= P.total_modes) return;
-    const SchemeCoef k = scheme_coef(P.scheme, P.omega2[gmode], P.gamma[gmode], P.dt[gmode]);
+    const LinCoef64 k = lin_coef64(P, gmode);
     // A^L by repeated squaring
-    double a00 = 2.0 - k.eps - k.rho, a01 = k.eps - 1.0, a10 = 1.0, a11 = 0.0;
+    double a00 = k.g, a01 = k.p, a10 = 1.0, a11 = 0.0;
     double r00 = 1.0, r01 = 0.0, r10 = 0.0, r11 = 1.0;
     for (int L = P.L; L > 0; L >>= 1) {
         if (L & 1) {
@@ -177,12 +188,14 @@ __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams
     __shared__ float es[kLinChunk];
     __shared__ float2 terms[kLinWarps][32][33];       // [step][mode], rows without conflicts
     __shared__ float2 ypart[kLinWarps][kLinChunk];
-    const int j = blockIdx.x, inst = blockIdx.y;
+    // the last chunks, which also step the end states in FP64, come first
+    const int inst = blockIdx.x % P.n_inst, j = P.n_chunks - 1 - blockIdx.x / P.n_inst;
     const InstDesc d = P.inst[inst];
     const int n0 = j * P.L, cnt = min(P.steps, n0 + P.L) - n0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = lane; t < kLinChunk; t += 32) ypart[warp][t] = make_float2(0.f, 0.f);
     load_exc(P, inst, n0, n0 + cnt, es);
+    const float emax = largest(es, cnt);
     // every warp walks whole rounds of 32 modes
     for (int m0 = warp * 32; m0 < d.N; m0 += kLinThreads) {
         const int m = m0 + lane;
@@ -191,11 +204,23 @@ __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams
         LinCoef k = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
         Pair q = {0.f, 0.f}, v = {0.f, 0.f}, c = {0.f, 0.f};
         if (on) {
-            k = lin_coef(P, gm);
+            const SchemeCoef sc = scheme_coef(P.scheme, P.omega2[gm], P.gamma[gm], P.dt[gm]);
             const double *S = P.S + ((long long)j * P.total_modes + gm) * 2;
-            q = pair_of(S[0]);
-            v = pair_of(S[0] - S[1]);
-            c = pair_of(P.c[gm]);
+            const double q0 = S[0], v0 = S[0] - S[1], rb = sc.r * P.b[gm];
+            // the scale 2^x: state and input to about 1 (r b stays an FP32 number where
+            // the whole input is tiny), its inverse in the pickup weight
+            const double big = fmax(fmax(fabs(q0), fabs(v0)), fabs(rb) * (double)emax);
+            int x = 0;
+            if (big > 0.0 && isfinite(big)) {
+                x = -ilogb(big);
+                if (rb != 0.0) x = min(x, 120 - ilogb(rb));
+            }
+            k.neps = pair_of(-sc.eps);
+            k.nrho = pair_of(-sc.rho);
+            k.rb = pair_of(scalbn(rb, x));
+            q = pair_of(scalbn(q0, x));
+            v = pair_of(scalbn(v0, x));
+            c = pair_of(scalbn(P.c[gm], -x));
         }
         const int modes = min(32, d.N - m0);
         for (int i0 = 0; i0 < cnt; i0 += 32) {
@@ -220,11 +245,22 @@ __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams
             }
             __syncwarp();
         }
-        if (on && j == P.n_chunks - 1) {
-            if (P.q_end) P.q_end[gm] = value(q);
-            if (P.qm1_end) P.qm1_end[gm] = value(q) - value(v);
-        }
     }
+    if (j == P.n_chunks - 1 && (P.q_end || P.qm1_end))
+        for (int m = threadIdx.x; m < d.N; m += kLinThreads) {
+            const long long gm = d.mode_off + m;
+            const LinCoef64 k = lin_coef64(P, gm);
+            const double *S = P.S + ((long long)j * P.total_modes + gm) * 2;
+            double x0 = S[0], x1 = S[1];
+#pragma unroll 4
+            for (int n = 0; n < cnt; ++n) {
+                const double x = fma(k.g, x0, fma(k.p, x1, k.rb * (double)es[n]));
+                x1 = x0;
+                x0 = x;
+            }
+            if (P.q_end) P.q_end[gm] = x0;
+            if (P.qm1_end) P.qm1_end[gm] = x1;
+        }
     __syncthreads();
     for (int t = threadIdx.x; t < cnt; t += kLinThreads) {
         float ys = 0.f, ye = 0.f;
@@ -248,7 +284,7 @@ cudaError_t launch_linear(const LinearParams &P, cudaStream_t s) {
     lin_carry_kernel<<<(int)((P.total_modes + cb - 1) / cb), cb, 0, s>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    lin_out_kernel<<<grid, kLinThreads, 0, s>>>(P);
+    lin_out_kernel<<<(unsigned)((long long)P.n_chunks * P.n_inst), kLinThreads, 0, s>>>(P);
     return cudaGetLastError();
 }
 
