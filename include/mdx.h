@@ -344,14 +344,20 @@ int mdx_grad(mdx_plan *plan, const float *exc, const double *q0, const double *q
  * Tile configuration of the plate kernel (used by the autotuner; a
  * performance control with no counterpart in the paper): TMA stage
  * size in bytes (multiple of 16, 0 = default 64 KB) and ring depth (0 = as
- * many stages as shared memory allows).  Takes effect for later launches;
- * fails with MDX_ERR_UNSUPPORTED if the stages do not fit in shared memory.
+ * many stages as shared memory allows).  Takes effect for later launches of the
+ * streaming kernel (a resident plan keeps the order of sums of the stage size it
+ * was created with); fails with MDX_ERR_UNSUPPORTED if the stages do not fit in shared memory.
  * mdx_plan_tiles reports the current stage size, ring depths of the forward
  * and reverse launches, and the number of persistent CTAs.
  */
 int mdx_plan_configure(mdx_plan *plan, int stage_bytes, int ring_stages);
 int mdx_plan_tiles(const mdx_plan *plan, int *stage_bytes, int *ring_fwd, int *ring_rev,
                    int *ctas);
+/* Which passes of the plan's plates run on the resident kernel, whose launch the
+ * tile configuration does not touch: 1 or 0 for forward passes without
+ * checkpoints, and for passes with checkpoints and gradients (bookkeeping of this
+ * library).  Pointers may be NULL.  Errors: MDX_ERR_ARG for a NULL plan. */
+int mdx_plan_resident(const mdx_plan *plan, int *forward, int *checkpointed);
 
 /*
  * L2 residency of the coupling stream.  Every step re-reads the whole

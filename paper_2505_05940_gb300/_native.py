@@ -26,7 +26,7 @@ EXPORTED = ("mdx_last_error", "mdx_version", "mdx_plan_create", "mdx_plan_destro
             "mdx_plan_info", "mdx_checkpoint_bytes", "mdx_simulate", "mdx_grad_workspace_bytes",
             "mdx_grad", "mdx_coeffs_from_physics", "mdx_coeffs_vjp", "mdx_plan_set_profiling",
             "mdx_plan_kernel_stats", "mdx_plan_reset_stats", "mdx_plan_configure",
-            "mdx_plan_tiles", "mdx_simulate_strings_noalloc", "mdx_plan_set_coefficients",
+            "mdx_plan_tiles", "mdx_plan_resident", "mdx_simulate_strings_noalloc", "mdx_plan_set_coefficients",
             "mdx_mlp_act_elems", "mdx_mlp_work_elems", "mdx_mlp_forward", "mdx_mlp_backward",
             "mdx_adam_step", "mdx_f32_to_bf16", "mdx_plan_set_l2_keep", "mdx_plan_l2_keep",
             "mdx_difference_coefficients", "mdx_coefficient_grads", "mdx_modal_from_physics",
@@ -166,6 +166,7 @@ def load(build_if_missing: bool = True):
         L.mdx_plan_l2_keep.argtypes = [vp]
         L.mdx_plan_l2_keep.restype = ctypes.c_double
         L.mdx_plan_tiles.argtypes = [vp] + [ctypes.POINTER(i32)] * 4
+        L.mdx_plan_resident.argtypes = [vp] + [ctypes.POINTER(i32)] * 2
         L.mdx_plan_set_profiling.argtypes = [vp, i32]
         L.mdx_plan_group_work.argtypes = [vp, ctypes.POINTER(ctypes.c_double),
                                           ctypes.POINTER(ctypes.c_double)]
@@ -327,6 +328,12 @@ class Plan:
         check(load().mdx_plan_tiles(self._h, *[ctypes.byref(x) for x in v]))
         return dict(stage_bytes=v[0].value, ring_fwd=v[1].value, ring_rev=v[2].value,
                     ctas=v[3].value)
+
+    def resident(self):
+        """Which passes of the plates run on the resident kernel."""
+        v = [ctypes.c_int() for _ in range(2)]
+        check(load().mdx_plan_resident(self._h, *[ctypes.byref(x) for x in v]))
+        return dict(forward=bool(v[0].value), checkpointed=bool(v[1].value))
 
     # ------------------------------------------------------------------ tracing
     def group_work(self):

@@ -2,9 +2,9 @@
 
 For a given set of instances the tuner times a short checkpointed forward
 run for each candidate TMA stage size of the streaming plate kernel (the ring
-depth follows from the shared memory left over) and keeps the fastest.  Plans
-that the resident kernel takes have no stages to tune: every candidate then
-times alike.  Results are cached in a JSON file keyed by the
+depth follows from the shared memory left over) and keeps the fastest.  A plan
+whose checkpointed passes run on the resident kernel has no stages to tune: it
+keeps its stage size, and nothing is timed.  Results are cached in a JSON file keyed by the
 GPU name and a signature of the plate shapes, so a workload is tuned once per
 device type.  Timing uses the library's own per-launch CUDA events
 (mdx_plan_kernel_stats).
@@ -42,19 +42,39 @@ def _load(path):
         return {}
 
 
+def _store(path, key, entry):
+    with _lock:
+        cache = _load(path)
+        cache[key] = entry
+        os.makedirs(os.path.dirname(path), exist_ok=True)
+        tmp = path + f".{os.getpid()}.tmp"
+        with open(tmp, "w") as f:
+            json.dump(cache, f, indent=1)
+        os.replace(tmp, path)
+
+
 def tune(sim, steps=128, repeats=2, cache_path=None, candidates=STAGE_CANDIDATES, force=False):
     """Pick the stage size for sim.plan (a modal.Simulator); applies it and
-    returns {'stage_bytes', 'us_per_step', 'cached', 'trials'}."""
+    returns {'stage_bytes', 'us_per_step', 'cached', 'trials'} (a resident plan:
+    its own stage size, no time, no trials)."""
     import torch
     if not any(p["kind"] == "plate" and p.get("H") is not None for p in sim.prepared):
         return {"stage_bytes": 0, "us_per_step": None, "cached": False, "trials": []}
     path = cache_path or default_cache_path()
     key = f"{torch.cuda.get_device_name(sim.device)}|{signature(sim.prepared)}"
+    resident = sim.plan.resident()["checkpointed"]
     with _lock:
         cache = _load(path)
-    if not force and key in cache:
-        sim.plan.configure(stage_bytes=cache[key]["stage_bytes"])
+    # an entry of the other kind (the same shapes under other options) does not count
+    if not force and key in cache and cache[key].get("resident", False) == resident:
+        if not resident:
+            sim.plan.configure(stage_bytes=cache[key]["stage_bytes"])
         return dict(cache[key], cached=True)
+    if resident:
+        entry = {"stage_bytes": sim.plan.tiles()["stage_bytes"], "us_per_step": None,
+                 "trials": [], "resident": True}
+        _store(path, key, entry)
+        return dict(entry, cached=False)
     trials = []
     for stage in candidates:
         try:
@@ -77,12 +97,5 @@ def tune(sim, steps=128, repeats=2, cache_path=None, candidates=STAGE_CANDIDATES
     sim.plan.configure(stage_bytes=best["stage_bytes"])
     entry = {"stage_bytes": best["stage_bytes"], "us_per_step": best["us_per_step"],
              "trials": trials}
-    with _lock:
-        cache = _load(path)
-        cache[key] = entry
-        os.makedirs(os.path.dirname(path), exist_ok=True)
-        tmp = path + f".{os.getpid()}.tmp"
-        with open(tmp, "w") as f:
-            json.dump(cache, f, indent=1)
-        os.replace(tmp, path)
+    _store(path, key, entry)
     return dict(entry, cached=False)

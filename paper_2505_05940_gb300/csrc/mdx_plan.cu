@@ -2161,6 +2161,13 @@ extern "C" int mdx_plan_tiles(const mdx_plan *p, int *stage_bytes, int *ring_fwd
     return MDX_OK;
 }
 
+extern "C" int mdx_plan_resident(const mdx_plan *p, int *forward, int *checkpointed) {
+    if (!p) return fail(MDX_ERR_ARG, "plan is NULL");
+    if (forward) *forward = p->res_fast.ok || p->res_same.ok;
+    if (checkpointed) *checkpointed = p->res_same.ok;
+    return MDX_OK;
+}
+
 extern "C" int mdx_plan_set_coefficients(mdx_plan *p, const double *omega2, const double *gamma,
                                          const double *b, const double *c, const double *tau,
                                          const double *kappa) {
