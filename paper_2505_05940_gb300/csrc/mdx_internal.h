@@ -297,6 +297,30 @@ cudaError_t resident_check(int cs, const ResidentParams &Q, size_t smem_optin, i
 cudaError_t launch_resident(int R, const ResidentParams &Q, int grid, int cs, size_t smem,
                             cudaStream_t s);
 
+// Small plates with many stress modes (mdx_cluster.cu): one cluster a plate.
+constexpr int kClusterCtas = 16;        // CTAs of a cluster
+constexpr int kClusterMaxNkc = 16;      // stress modes of a CTA, one warp each
+constexpr int kClusterMaxModes = 32;    // transverse modes, one lane each
+struct ClusterParams {
+    const InstDesc *inst;
+    const int *plates;            // plate instance indices (one cluster each)
+    const ClusterK *kinfo;        // [total_k]
+    const float *H;
+    const float *kappa;
+    const int *perm;
+    ModeCoef coef;
+    int cs;                       // CTAs per cluster
+    int nkc;                      // stress modes per CTA
+    int steps, n_begin, total_steps;
+    const float *exc;
+    float *audio;
+    float *state_io;              // [4][total_modes]: q_hi, q_lo, v_hi, v_lo
+    long long total_modes;
+    int *status;
+};
+cudaError_t launch_cluster(const ClusterParams &P, int n_plates, cudaStream_t s);
+cudaError_t cluster_check(int cs, int nkc, int *max_clusters);
+
 struct TensionParams {
     const InstDesc *inst;
     const int *list;              // tension instance indices

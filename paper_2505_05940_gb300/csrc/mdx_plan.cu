@@ -156,6 +156,11 @@ struct mdx_plan {
         ResidentParams q{};                  // launch shape and tables (p unset)
         size_t smem[4] = {0, 0, 0, 0};       // by right-hand sides
     } res_same, res_fast;
+    // forward pass of small plates with more stress modes than the resident kernel
+    // takes (mdx_cluster.cu): stress modes per CTA (0: not taken), plates
+    int cl_nkc = 0, n_cplates = 0;
+    const ClusterK *cl_kinfo = nullptr;
+    int *d_cplates = nullptr;
     bool fused_sweep = false;        // mdx_grad fuses reverse and recompute
 };
 
@@ -1560,7 +1565,64 @@ int plan_resident(mdx_plan *p, const std::vector<ParityChunk> &chunks,
     if ((rc = upload(p, &dk, kinfo.data(), kinfo.size()))) return rc;
     if ((rc = upload(p, &di, iperm.data(), iperm.size()))) return rc;
     if (same && (rc = build_resident(p, sames, variant_same, true, dk, di, smem_optin, &p->res_same))) return rc;
-    return build_resident(p, pls, variant, false, dk, di, smem_optin, &p->res_fast);
+    if ((rc = build_resident(p, pls, variant, false, dk, di, smem_optin, &p->res_fast))) return rc;
+    if (p->res_same.ok || p->res_fast.ok || !p->parity) return MDX_OK;
+    // more stress modes than 16 CTAs of eight warps hold: the cluster kernel, if it
+    // takes every plate and all clusters run at once
+    int max_m = 0, fit = 0;
+    std::vector<int> list;
+    for (const ResPlate &q : pls) {
+        if (q.N > kClusterMaxModes) return MDX_OK;
+        max_m = std::max(max_m, q.M);
+        list.push_back(q.inst);
+    }
+    const int nkc = (max_m + kClusterCtas - 1) / kClusterCtas;
+    if (max_m < kClusterCtas || nkc > kClusterMaxNkc) return MDX_OK;
+    if (cluster_check(kClusterCtas, nkc, &fit) != cudaSuccess) {
+        cudaGetLastError();
+        return MDX_OK;
+    }
+    if (fit < (int)list.size()) return MDX_OK;
+    if ((rc = upload(p, &p->d_cplates, list.data(), list.size()))) return rc;
+    p->cl_nkc = nkc;
+    p->n_cplates = (int)list.size();
+    p->cl_kinfo = dk;
+    return MDX_OK;
+}
+
+int run_cluster(mdx_plan *p, const PlateParams &P, cudaStream_t s) {
+    ClusterParams C{};
+    C.inst = p->d_inst;
+    C.plates = p->d_cplates;
+    C.kinfo = p->cl_kinfo;
+    C.H = p->d_H;
+    C.kappa = p->d_kappa;
+    C.perm = p->d_perm;
+    C.coef = p->coef;
+    C.cs = kClusterCtas;
+    C.nkc = p->cl_nkc;
+    C.steps = P.steps;
+    C.n_begin = P.n_begin;
+    C.total_steps = P.total_steps;
+    C.exc = P.exc;
+    C.audio = P.audio;
+    C.state_io = P.state_io;
+    C.total_modes = p->total_modes;
+    C.status = P.status;
+    mdx_plan::Rec rec{};
+    if (p->profiling) {
+        rec.which = 6;
+        rec.bytes = (double)P.steps * p->H_bytes_per_step;
+        MDX_CUDA(cudaEventCreate(&rec.a), "event");
+        MDX_CUDA(cudaEventCreate(&rec.b), "event");
+        MDX_CUDA(cudaEventRecord(rec.a, s), "event");
+    }
+    MDX_CUDA(launch_cluster(C, p->n_cplates, s), "cluster plate kernel");
+    if (p->profiling) {
+        MDX_CUDA(cudaEventRecord(rec.b, s), "event");
+        p->recs.push_back(rec);
+    }
+    return MDX_OK;
 }
 
 int run_resident(mdx_plan *p, const mdx_plan::Resident &res, const PlateParams &P, cudaStream_t s) {
@@ -1588,6 +1650,7 @@ int run_plate(mdx_plan *p, PlateParams &P, cudaStream_t s) {
     if (!p->any_plate) return MDX_OK;
     if (P.mode == MODE_FORWARD && !P.ckpt && p->res_fast.ok) return run_resident(p, p->res_fast, P, s);
     if (p->res_same.ok) return run_resident(p, p->res_same, P, s);
+    if (P.mode == MODE_FORWARD && !P.ckpt && p->cl_nkc > 0) return run_cluster(p, P, s);
     MDX_CUDA(cudaMemsetAsync(p->d_counters, 0, p->n_inst * sizeof(unsigned), s), "memset");
     MDX_CUDA(cudaMemsetAsync(p->d_abort, 0, sizeof(int), s), "memset");
     const size_t smem = (P.mode == MODE_FUSED) ? p->smem_fused
@@ -2163,7 +2226,7 @@ extern "C" int mdx_plan_tiles(const mdx_plan *p, int *stage_bytes, int *ring_fwd
 
 extern "C" int mdx_plan_resident(const mdx_plan *p, int *forward, int *checkpointed) {
     if (!p) return fail(MDX_ERR_ARG, "plan is NULL");
-    if (forward) *forward = p->res_fast.ok || p->res_same.ok;
+    if (forward) *forward = p->res_fast.ok || p->res_same.ok || p->cl_nkc > 0;
     if (checkpointed) *checkpointed = p->res_same.ok;
     return MDX_OK;
 }
