@@ -184,12 +184,41 @@ __global__ void lin_carry_kernel(const LinearParams P) {
     }
 }
 
+// End states of an instance: its last chunk from its true incoming state, FP64.
+__device__ void end_states(const LinearParams &P, int inst, float *es) {
+    const InstDesc d = P.inst[inst];
+    const int j = P.n_chunks - 1, n0 = j * P.L, cnt = P.steps - n0;
+    load_exc(P, inst, n0, P.steps, es);
+    for (int m = threadIdx.x; m < d.N; m += kLinThreads) {
+        const long long gm = d.mode_off + m;
+        const LinCoef64 k = lin_coef64(P, gm);
+        const double *S = P.S + ((long long)j * P.total_modes + gm) * 2;
+        double x0 = S[0], x1 = S[1];
+#pragma unroll 4
+        for (int n = 0; n < cnt; ++n) {
+            const double x = fma(k.g, x0, fma(k.p, x1, k.rb * (double)es[n]));
+            x1 = x0;
+            x0 = x;
+        }
+        if (P.q_end) P.q_end[gm] = x0;
+        if (P.qm1_end) P.qm1_end[gm] = x1;
+    }
+}
+
+// Blocks: the instances' end states if asked for, then every (chunk, instance).
 __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams P) {
     __shared__ float es[kLinChunk];
     __shared__ float2 terms[kLinWarps][32][33];       // [step][mode], rows without conflicts
     __shared__ float2 ypart[kLinWarps][kLinChunk];
-    // the last chunks, which also step the end states in FP64, come first
-    const int inst = blockIdx.x % P.n_inst, j = P.n_chunks - 1 - blockIdx.x / P.n_inst;
+    unsigned blk = blockIdx.x;
+    if (P.q_end || P.qm1_end) {
+        if (blk < (unsigned)P.n_inst) {
+            end_states(P, (int)blk, es);
+            return;
+        }
+        blk -= P.n_inst;
+    }
+    const int inst = (int)(blk % P.n_inst), j = (int)(blk / P.n_inst);
     const InstDesc d = P.inst[inst];
     const int n0 = j * P.L, cnt = min(P.steps, n0 + P.L) - n0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -246,21 +275,6 @@ __global__ void __launch_bounds__(kLinThreads) lin_out_kernel(const LinearParams
             __syncwarp();
         }
     }
-    if (j == P.n_chunks - 1 && (P.q_end || P.qm1_end))
-        for (int m = threadIdx.x; m < d.N; m += kLinThreads) {
-            const long long gm = d.mode_off + m;
-            const LinCoef64 k = lin_coef64(P, gm);
-            const double *S = P.S + ((long long)j * P.total_modes + gm) * 2;
-            double x0 = S[0], x1 = S[1];
-#pragma unroll 4
-            for (int n = 0; n < cnt; ++n) {
-                const double x = fma(k.g, x0, fma(k.p, x1, k.rb * (double)es[n]));
-                x1 = x0;
-                x0 = x;
-            }
-            if (P.q_end) P.q_end[gm] = x0;
-            if (P.qm1_end) P.qm1_end[gm] = x1;
-        }
     __syncthreads();
     for (int t = threadIdx.x; t < cnt; t += kLinThreads) {
         float ys = 0.f, ye = 0.f;
@@ -284,7 +298,8 @@ cudaError_t launch_linear(const LinearParams &P, cudaStream_t s) {
     lin_carry_kernel<<<(int)((P.total_modes + cb - 1) / cb), cb, 0, s>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    lin_out_kernel<<<(unsigned)((long long)P.n_chunks * P.n_inst), kLinThreads, 0, s>>>(P);
+    const long long blocks = (P.n_chunks + (P.q_end || P.qm1_end ? 1LL : 0LL)) * P.n_inst;
+    lin_out_kernel<<<(unsigned)blocks, kLinThreads, 0, s>>>(P);
     return cudaGetLastError();
 }
 
