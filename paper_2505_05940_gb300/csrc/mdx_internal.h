@@ -423,7 +423,6 @@ constexpr int kLinChunk = 256;
 struct LinearParams {
     const InstDesc *inst;
     int n_inst;
-    const int *mode_inst;           // [total_modes] instance of each mode
     const double *omega2, *gamma, *dt, *b, *c;   // per mode FP64
     int scheme;
     int steps, total_steps, L, n_chunks;

@@ -67,7 +67,6 @@ struct mdx_plan {
     ModeCoef coef{};
     double *d_omega2 = nullptr, *d_gamma = nullptr, *d_dt = nullptr;
     double *d_b64 = nullptr, *d_c64 = nullptr;   // FP64 b, c (linear solver)
-    int *d_mode_inst = nullptr;                  // instance of each mode
     float *d_H = nullptr, *d_dH = nullptr, *d_kappa = nullptr;
     // plate work assignment
     int n_cta = 0;
@@ -467,9 +466,6 @@ int mdx_plan_create(mdx_plan **out, const mdx_instance *I, int n_inst, const mdx
         if ((rc = upload(p, &p->d_dt, dtd.data(), TM))) return bail(rc);
         if ((rc = upload(p, &p->d_b64, p->h_b.data(), TM))) return bail(rc);
         if ((rc = upload(p, &p->d_c64, p->h_c.data(), TM))) return bail(rc);
-        std::vector<int> mi;
-        for (int i = 0; i < n_inst; ++i) mi.insert(mi.end(), (size_t)p->inst[i].N, i);
-        if ((rc = upload(p, &p->d_mode_inst, mi.data(), mi.size()))) return bail(rc);
     }
     // ---- tension list (strings, membranes and plates without coupling)
     for (int i = 0; i < n_inst; ++i) {
@@ -2123,7 +2119,6 @@ extern "C" int mdx_simulate_linear(mdx_plan *p, const float *exc, const double *
     LinearParams L{};
     L.inst = p->d_inst;
     L.n_inst = p->n_inst;
-    L.mode_inst = p->d_mode_inst;
     L.omega2 = p->d_omega2;
     L.gamma = p->d_gamma;
     L.dt = p->d_dt;
