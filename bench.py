@@ -120,6 +120,41 @@ def profiled_traffic(a, steps_per_launch):
     return float(m_tr.group(1)) * steps_per_launch
 
 
+def plate_roofline(stats, names, resident, peak, peak_kind, sms):
+    """The dominant plate launch class against what bounds it.  stats: class ->
+    (launches, ms, bytes of one pass over the coupling data per step).  The
+    streaming kernel moves those bytes; the resident kernel reads them once per
+    launch, so its figure is the FP32 multiply-adds of the products (one per
+    coupling entry and right-hand side) against the CUDA cores' nominal rate."""
+    dom = max(stats, key=lambda w: stats[w][1])
+    rhs = {0: 1, 1: 1, 2: 2, 4: 3}
+    fp32_peak = sms * 128 * 2 * 2.07e9 / 1e12
+
+    def rate(w):
+        n, ms, b = stats[w]
+        if not ms:
+            return None
+        return (2.0 * rhs[w] * b / 4.0 / (ms * 1e-3) / 1e12 if resident else b / (ms * 1e-3) / 1e9)
+
+    unit = "TFLOP/s" if resident else "GB/s"
+    n, ms, b = stats[dom]
+    out = {"bound": "fp32" if resident else "hbm", "achieved": rate(dom),
+           "peak": fp32_peak if resident else peak, "unit": unit, "traffic": None,
+           "kernel": ("resident plate kernel, " if resident else "streaming plate kernel, ") + names[dom],
+           "peak_source": ("nominal: SMs x 128 FP32 lanes x 2 x 2.07 GHz" if resident
+                           else f"{peak_kind} hbm_gbs"),
+           "per_launch_ms": ms / max(n, 1)}
+    out["frac"] = out["achieved"] / out["peak"] if out["achieved"] else None
+    if resident:
+        out["basis"] = ("multiply-adds of the coupling products; a step's dependent chain "
+                        "(barrier, reductions, two exchanges between CTAs) takes most of its time")
+    else:
+        out["per_launch_algorithmic_bytes"] = b / max(n, 1)
+    out["all_plate_kernels"] = {names[w]: {"launches": stats[w][0], "ms": stats[w][1], unit: rate(w)}
+                                for w in stats}
+    return out
+
+
 # ----------------------------------------------------------------- ranks
 
 def shard_seed(rank):
@@ -380,10 +415,10 @@ def forward_workload(a):
                                 "peak_source": f"{peak_kind} hbm_gbs",
                                 "share_of_time": pms / (ms * a.steps)}
     if cn:
-        # a few small plates, coupling rows resident in the registers of one
-        # thread-block cluster per plate: bound by the latency of a step's
-        # dependent chain (matvec, reductions, one cluster barrier), not by bytes
-        line["cluster_kernel"] = {"us_per_step": cms * 1e3 / (cn * steps),
+        # plates whose coupling rows stay on the SMs (tensor memory, shared memory,
+        # registers) of a thread-block cluster: bound by the latency of a step's
+        # dependent chain (products, reductions, two exchanges), not by bytes
+        line["resident_kernel"] = {"us_per_step": cms * 1e3 / (cn * steps),
                                   "share_of_time": cms / (ms * a.steps),
                                   "bound": "latency (H read once per launch)"}
     if gn:
@@ -658,26 +693,11 @@ def main():
     sim.plan.set_profiling(False)
     peak, peak_kind = load_peaks()
     tot_ms = sum(s[1] for s in stats.values())
-    dom = max(stats, key=lambda w: stats[w][1])
-    n_l, d_ms, d_bytes = stats[dom]
-    achieved = (d_bytes / n_l) / ((d_ms / n_l) * 1e-3) / 1e9 if n_l else 0.0
-    names = {0: "plate kernel, forward", 1: "plate kernel, recompute",
-             2: "plate kernel, reverse", 4: "plate kernel, fused reverse + recompute"}
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": None,
-                "basis": "bytes of one pass over the class-layout coupling data per step, as "
-                         "if streamed; plates of at most 64 modes per class run on the "
-                         "resident kernel, which reads them once per launch and is bound "
-                         "by its step's dependent chain and FP32 FMAs",
-                "kernel": names[dom], "peak_source": f"{peak_kind} hbm_gbs",
-                "kernel_share_of_step": tot_ms / ms_total if ms_total else None,
-                "per_launch_ms": d_ms / max(n_l, 1),
-                "per_launch_algorithmic_bytes": d_bytes / max(n_l, 1)}
+    names = {0: "forward", 1: "recompute", 2: "reverse", 4: "fused reverse + recompute"}
+    roofline = plate_roofline(stats, names, sim.plan.resident()["checkpointed"], peak, peak_kind,
+                              torch.cuda.get_device_properties(dev).multi_processor_count)
+    roofline["kernel_share_of_step"] = tot_ms / ms_total if ms_total else None
     roofline["direction_contraction"] = {"launches": dir_stats[0], "ms": dir_stats[1]}
-    roofline["all_plate_kernels"] = {
-        names[w]: {"launches": s[0], "ms": s[1],
-                   "GB/s": (s[2] / (s[1] * 1e-3) / 1e9) if s[1] else None}
-        for w, s in stats.items()}
     # end-to-end through the public API with host buffers
     e2e = None
     if not a.no_e2e:
@@ -722,7 +742,7 @@ def main():
                 "config": {"workload": workload_name(a), "instances_per_gpu": a.n_inst,
                            "n_phi": a.n_phi, "n_psi": a.n_psi, "sim_steps": a.sim_steps,
                            "K": a.K, "loss": "multi-resolution log-STFT L1 (256/1024/4096)",
-                           "l2": ("working set larger than L2, no flush: every step re-reads "
+                           "l2": ("working set larger than L2, no flush: every launch reads "
                                   "the class-layout coupling data (128 MB) and each segment its "
                                   "aspect derivative (128 MB), beside checkpoints and segment "
                                   "buffers"),

@@ -360,8 +360,8 @@ int mdx_plan_tiles(const mdx_plan *plan, int *stage_bytes, int *ring_fwd, int *r
 int mdx_plan_resident(const mdx_plan *plan, int *forward, int *checkpointed);
 
 /*
- * L2 residency of the coupling stream.  Every step re-reads the whole
- * coupling tensor; the plate kernel's bulk copies carry an L2 policy that
+ * L2 residency of the coupling stream.  Every step of the streaming plate kernel
+ * re-reads the whole coupling tensor; its bulk copies carry an L2 policy that
  * gives a fraction of those addresses evict_last priority (the rest
  * evict_first), so that when the tensors of the plan are about as large as
  * the L2 (129 MB on GB300) that fraction stays resident across steps.
@@ -383,12 +383,12 @@ double mdx_plan_l2_keep(const mdx_plan *plan);
  * segment and the recompute of the previous one in the same launch,
  * 5 = grouped plates on the tensor cores: bytes are the nonzero class blocks
  * of each group's shared coupling tensor, one pass per step, 6 = forward pass
- * of a few plates with their coupling rows resident in the registers of one
- * thread-block cluster per plate: bytes count one pass over H per step as for
- * class 0, although H is read from memory once per launch), the
- * number of launches, their summed device time in ms and their summed
- * algorithmic bytes (coupling-tensor bytes each launch must stream: one pass
- * over H per step; the direction tensor is counted by class 3).
+ * without checkpoints of plates whose coupling rows stay on the SMs of a
+ * thread-block cluster), the number of launches, their summed device time in ms
+ * and their summed algorithmic bytes (one pass over H per step: what the
+ * streaming kernel must move.  Class 6, and classes 0, 1, 2 and 4 where
+ * mdx_plan_resident says so, read H once per launch; the direction tensor is
+ * counted by class 3).
  * mdx_plan_reset_stats clears the counters.  Off by default.
  */
 int mdx_plan_set_profiling(mdx_plan *plan, int enable);
