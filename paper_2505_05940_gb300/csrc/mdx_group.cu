@@ -53,7 +53,9 @@
 // Q image's rows lie eight lanes to a bank; the rows' states now sit in
 // tensor memory), owners 18 000 to 31 000 (one mode at a time, the plates' table
 // searched in global memory), partial forces 12 000 (64-bit addresses).  Together
-// 95 us a step at first, 53 with the gathers in batches, 38 now.
+// 95 us a step at first, 53 with the gathers in batches, 37.5 now (some 75 000
+// cycles: CTAs with three stress modes take about 12 700 more than the sum above,
+// and what the counters' waits add was not measured apart).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -17,8 +17,8 @@
 // clusters that do not fit at once run one after the other.  Measured, streaming
 // and here: 100 x 30 plate, 11 025 steps, 34.3 and 13.1 ms; 96 plates of 50 to
 // 200 modes 196 and 37.5 ms; a fit's step (forward with checkpoints, recompute and
-// reverse) of 6 plates of 117 x 29, 3 001 steps, 79.6 and 14.2 ms, of 64 plates of
-// 200 x 50, 4 410 steps, 346 and 218 ms.
+// reverse) of 6 plates of 117 x 29, 3 001 steps, 79.6 and 14.0 ms, of 64 plates of
+// 200 x 50, 4 410 steps, 346 and 219 ms.
 //
 // Rows: one warp per stress mode k.  Lanes 8 a .. 8 a + 7 hold the rows of
 // class a (row l + 8 r of the class in lane l, register row r), whose only
